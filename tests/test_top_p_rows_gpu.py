@@ -1,0 +1,96 @@
+"""massv_sample_top_p where its row-per-cluster kernel can go wrong: one entry, slices with a ragged last group, rows that
+start off a 16-byte boundary, a last CTA with few entries or none, every cluster size, ties cut between two CTAs, the
+longest row that fits, and the first one that does not (the one-CTA kernel)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(z, u, T, top_p, allow=0):
+    import paper_2505_10526_b200 as mv
+    rows, vocab = z.shape
+    tok = torch.full((rows,), -5, dtype=torch.int32, device="cuda")
+    pad = torch.full((rows * vocab + 8,), -1.0, device="cuda")
+    q = pad[4:4 + rows * vocab].view(rows, vocab)
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    mv.massv_sample_top_p(z, u, tok, T, top_p, q, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert float(pad[:4].max()) == -1.0 and float(pad[4 + rows * vocab:].max()) == -1.0
+    ref = oracle.sample_top_p(z.cpu().numpy(), u.cpu().numpy(), T, top_p)
+    qg, tg = q.cpu().double().numpy(), tok.cpu().numpy()
+    moved = 0
+    for r in range(rows):
+        same = np.array_equal(qg[r] > 0, ref["q"][r] > 0)
+        # fp32 weights against fp64 ones: the mass at which the prefix stops is known to about 1e-6 of the total
+        if not same and ref["margin_set"][r] < 1e-5:
+            moved += 1
+            continue
+        assert same, (r, int((qg[r] > 0).sum()), int(ref["nucleus_size"][r]))
+        assert np.abs(qg[r] - ref["q"][r]).max() < 1e-4
+        assert tg[r] == ref["token"][r] or ref["margin_sample"][r] < 1e-5, (r, tg[r], ref["token"][r])
+    assert moved <= allow
+    tok2 = torch.empty_like(tok)
+    mv.massv_sample_top_p(z, u, tok2, T, top_p, None, status)        # without the distribution, and again: the same tokens
+    assert torch.equal(tok, tok2)
+
+
+@pytest.mark.parametrize("rows,vocab", [(1, 1), (2, 3), (1, 4095), (3, 4097), (1, 8192), (150, 1021), (40, 21 * 1024), (37, 21 * 1024 + 1),
+                                        (18, 43009), (1, 131071), (9, 152064), (2, 48 * 1024 * 8), (2, 48 * 1024 * 8 + 1)])
+def test_sizes(rows, vocab):
+    g = torch.Generator(device="cuda").manual_seed(vocab)
+    z = torch.randn((rows, vocab), generator=g, device="cuda") * 4.0
+    z[:, vocab // 2:vocab // 2 + vocab // 8] = -float("inf")
+    _check(z, torch.rand((rows,), generator=g, device="cuda"), 0.8, 0.9, allow=1 + rows // 16)
+
+
+@pytest.mark.parametrize("vocab,shift", [(8192, 1), (50264, 2), (152064, 3)])
+def test_rows_off_the_alignment(vocab, shift):
+    g = torch.Generator(device="cuda").manual_seed(vocab)
+    z = torch.randn((3 * vocab + 4,), generator=g, device="cuda")[shift:shift + 3 * vocab].view(3, vocab)
+    _check(z, torch.rand((3,), generator=g, device="cuda"), 1.0, 0.7, allow=1)
+
+
+@pytest.mark.parametrize("top_p", [0.25, 0.5, 0.75, 1.0])
+def test_ties_over_several_ctas(top_p):
+    """Two levels of logit only: the prefix stops among equal weights, at an index that every CTA has to agree on.  The
+    weights are powers of two, so all masses are exact and the last member is known."""
+    vocab, rows = 65536, 4
+    z = torch.full((rows, vocab), -30.0, device="cuda")
+    for r in range(rows):
+        z[r, torch.randperm(vocab, generator=torch.Generator().manual_seed(r))[:8192].cuda()] = 3.0
+    import paper_2505_10526_b200 as mv
+    u = torch.tensor([0.0, 0.3, 0.7, 0.9999], device="cuda")
+    tok = torch.empty((rows,), dtype=torch.int32, device="cuda")
+    q = torch.empty_like(z)
+    # temperature 33 ln 2: the lower level weighs 2^-1 ... of the upper at T = 33 / ln 2 / 40: mass 57344 * 2^-40 of 8192
+    T = 33.0 * 1.4426950408889634 / 40.0
+    mv.massv_sample_top_p(z, u, tok, T, top_p, q, None)
+    torch.cuda.synchronize()
+    for r in range(rows):
+        heavy = torch.nonzero(z[r] > 0).flatten()
+        members = torch.nonzero(q[r] > 0).flatten()
+        # the light entries weigh 57,344 * 2^-40 = 5e-8 of one heavy one: at top_p below 1 the prefix ends inside the heavy ones, one
+        # more than top_p * 8192 where the light mass tips the ceiling; at 1 it takes everything
+        if top_p < 1.0:
+            k = members.numel()
+            assert k in (int(top_p * 8192), int(top_p * 8192) + 1)
+            assert torch.equal(members, heavy[:k])
+            assert int(tok[r]) == int(heavy[int(float(u[r]) * k)])
+        else:
+            assert members.numel() == vocab
+
+
+def test_rows_without_a_finite_logit():
+    import paper_2505_10526_b200 as mv
+    z = torch.randn((5, 60000), device="cuda")
+    z[3] = -float("inf")
+    tok = torch.full((5,), -5, dtype=torch.int32, device="cuda")
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    mv.massv_sample_top_p(z, torch.full((5,), 0.5, device="cuda"), tok, 1.0, 0.9, None, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == -1 and int(tok[3]) == 0 and int(tok.min()) >= 0
