@@ -421,7 +421,7 @@ size_t massv_tvd_workspace_size(const massv_accept_desc* desc) {
 }
 
 static int tvd_call(const massv_accept_desc* desc, const float* logits, const float* draft_probs, const float* row_stats, float* tvd_out,
-                    float* accept_prob_out, void* workspace, size_t workspace_bytes, massv_stream_t stream) {
+                    float* accept_prob_out, void* workspace, size_t workspace_bytes, int32_t* dev_status, massv_stream_t stream) {
     const int rc = check_accept_desc(desc);
     if (rc != MASSV_OK) return rc;
     if (desc->gamma < 1 || !(desc->temperature > 0.f)) return MASSV_ERR_INVALID_ARG;
@@ -433,34 +433,31 @@ static int tvd_call(const massv_accept_desc* desc, const float* logits, const fl
     char* ws = static_cast<char*>(workspace);
     TvdParams t;
     t.B = desc->batch; t.gamma = desc->gamma; t.V = desc->vocab; t.inv_T = 1.f / desc->temperature;
-    t.slice_len = ((desc->vocab + kTvdSlices - 1) / kTvdSlices + 3) / 4 * 4;      // 16-byte aligned slices (V % 8 == 0)
     t.logits = logits; t.draft_probs = draft_probs; t.tvd_out = tvd_out; t.accept_prob_out = accept_prob_out;
     t.slice_max = reinterpret_cast<float*>(ws);
     const size_t off = align_up(rows * kTvdSlices * sizeof(float), kAlign), step = align_up(rows * kTvdSlices * sizeof(double), kAlign);
     t.slice_sum = reinterpret_cast<double*>(ws + off);
     t.slice_abs = reinterpret_cast<double*>(ws + off + step);
     t.slice_min = reinterpret_cast<double*>(ws + off + 2 * step);
-    t.row_stats = row_stats;
+    t.row_stats = row_stats; t.dev_status = dev_status;
     return launch_tvd(t, reinterpret_cast<cudaStream_t>(stream)) == cudaSuccess ? MASSV_OK : MASSV_ERR_CUDA;
 }
 
 int massv_tvd(const massv_accept_desc* desc, const float* logits, const float* draft_probs, float* tvd_out,
               float* accept_prob_out, void* workspace, size_t workspace_bytes, int32_t* dev_status, massv_stream_t stream) {
-    (void)dev_status;
-    return tvd_call(desc, logits, draft_probs, nullptr, tvd_out, accept_prob_out, workspace, workspace_bytes, stream);
+    return tvd_call(desc, logits, draft_probs, nullptr, tvd_out, accept_prob_out, workspace, workspace_bytes, dev_status, stream);
 }
 
 int massv_tvd_after_accept(const massv_accept_desc* desc, const float* logits, const float* draft_probs,
                            const void* accept_workspace, size_t accept_workspace_bytes, float* tvd_out, float* accept_prob_out,
                            void* workspace, size_t workspace_bytes, int32_t* dev_status, massv_stream_t stream) {
-    (void)dev_status;
     const int rc = check_accept_desc(desc);
     if (rc != MASSV_OK) return rc;
     const AcceptLayout l = accept_layout(*desc);
     if (!accept_workspace || (reinterpret_cast<uintptr_t>(accept_workspace) % kAlign) != 0 || accept_workspace_bytes < l.total)
         return MASSV_ERR_WORKSPACE;
     const float* row_stats = reinterpret_cast<const float*>(static_cast<const char*>(accept_workspace) + l.off_rowstat);
-    return tvd_call(desc, logits, draft_probs, row_stats, tvd_out, accept_prob_out, workspace, workspace_bytes, stream);
+    return tvd_call(desc, logits, draft_probs, row_stats, tvd_out, accept_prob_out, workspace, workspace_bytes, dev_status, stream);
 }
 
 int massv_tvd_histogram(int64_t n, const float* tvd, int32_t bins, int64_t* counts, massv_stream_t stream) {

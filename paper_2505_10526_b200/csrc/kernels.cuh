@@ -135,15 +135,15 @@ struct PublishParams {
 cudaError_t launch_shard_publish(const PublishParams& p, cudaStream_t stream);
 
 // ---------------------------------------------------------------- TVD diagnostic
-constexpr int kTvdSlices = 16;      // vocabulary slices per row
+constexpr int kTvdSlices = 16;      // shares of a row's result the workspace has room for
 struct TvdParams {
     int B, gamma, V;
     float inv_T;
-    int slice_len;                  // entries per slice
     const float *logits, *draft_probs;
     float *tvd_out, *accept_prob_out;
     float* slice_max;               // [B*gamma, kTvdSlices]
     double *slice_sum, *slice_abs, *slice_min;
+    int32_t* dev_status;
     const float* row_stats = nullptr;   // [B*(gamma+1), 2] left by the acceptance scan: then the statistics pass is skipped
 };
 cudaError_t launch_tvd(const TvdParams& p, cudaStream_t stream);

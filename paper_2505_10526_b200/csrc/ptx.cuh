@@ -64,6 +64,27 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 
+// ---- a row held by the CTAs of one cluster (1 .. 16): barrier of all their threads, loads from a peer's shared memory
+__device__ __forceinline__ void row_barrier(int n_ctas) {        // all threads of the row's CTAs
+    if (n_ctas == 1) { __syncthreads(); return; }
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_smem(const void* local, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local)), "r"((uint32_t)rank));
+    return r;
+}
+__device__ __forceinline__ unsigned long long peer_load_u64(const void* local, int rank) {
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(peer_smem(local, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t peer_load_u32(const void* local, int rank) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(peer_smem(local, rank)) : "memory");
+    return v;
+}
+
 // Host: 2-D bf16 tensor map over [rows, cols] (cols contiguous) with a box of
 // [box_rows, 64 cols] and the 128-byte swizzle.  Returns false if the driver
 // entry point is unavailable or rejects the shape.

@@ -349,26 +349,6 @@ constexpr int kRowMaxSlice = 48 * 1024;
 static_assert(kRowThreads == kTopPBins && kRowThreads >= kRowMaxCluster * kRowCand, "one thread per bin, one per candidate");
 static_assert(kRowMaxSlice * kRowMaxCluster <= (1 << 19), "fixed point with 44 bits");
 
-__device__ __forceinline__ void row_barrier(int n_ctas) {        // all threads of the row's CTAs
-    if (n_ctas == 1) { __syncthreads(); return; }
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t peer_smem(const void* local, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local)), "r"((uint32_t)rank));
-    return r;
-}
-__device__ __forceinline__ unsigned long long peer_load_u64(const void* local, int rank) {
-    unsigned long long v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(peer_smem(local, rank)) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint32_t peer_load_u32(const void* local, int rank) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(peer_smem(local, rank)) : "memory");
-    return v;
-}
-
 // What a CTA lets the rest of its cluster read.
 struct RowPublished {
     unsigned long long hist[2][kTopPBins];   // two levels of the threshold search take turns
