@@ -4,9 +4,10 @@
 //
 // The scan over the cache is bound by HBM.  All G*(gamma+1) query rows that share
 // a KV head are processed by the same CTA so that every K/V byte is read once.
-// Work item = (sequence, KV head, chunk of kv_chunk positions); grid =
-// (max_chunks, Hkv, B) and CTAs whose chunk lies beyond the sequence retire at
-// once, so the hardware scheduler balances ragged lengths.  Inside a CTA a
+// Two schedules (see launch_verify_attn): work items = (sequence, KV head, chunk of
+// kv_chunk positions) on a grid (max_chunks, Hkv, B), where CTAs whose chunk lies beyond
+// the sequence retire at once; or, at head_dim 256, a persistent grid that cuts the line of
+// all tiles into equal ranges (attn_flat_kernel).  Inside a CTA a
 // producer warp streams 64-token (32-token at d = 256) K/V tiles page by page with TMA (16 x 64 boxes,
 // 128-byte swizzle) into an mbarrier ring; consumer warps run
 // Q K^T and P V on warp-level tensor-core MMAs (m16n8k16, bf16 -> fp32) with an
@@ -62,6 +63,133 @@ struct AttnCfg {
     static constexpr int kStages = DEEP ? 6 : ((D == 64) ? 4 : 3);
 };
 
+// One tile of K/V for a warp: its 16 query rows (group mt) against its TILE/TS tokens (slice ts) of the tile at `kst` (K, then
+// V), the online softmax carried in (o, m_run, l_run).  page_of(position) is the page that holds it (asked for the block's
+// own positions only: they are appended here).
+template <int D, int MT, int TS, int TILE, typename PageOf>
+__device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, int L, int c_end, int tile_start, uint8_t* kst, uint32_t q_base,
+                                            const uint32_t (&qf)[D <= 128 ? D / 16 : 1][4], int mt, int ts, int lane, int j0, int j1, float scale_log2,
+                                            PageOf&& page_of, float (&o)[D / 8][4], float (&m_run)[2], float (&l_run)[2]) {
+    constexpr int kTile = TILE, NT = TILE / TS, RP = MT * 16;
+    constexpr int kRegion = TILE * 128, kBytesK = (D / 64) * kRegion;
+    constexpr bool kQInRegs = D <= 128;
+    const int n_ctx = L + p.R;
+    const int lm = lane >> 3, lr = lane & 7;      // ldmatrix lane roles: matrix (lane >> 3), row (lane & 7) inside it
+    const int valid = min(kTile, c_end - tile_start);
+    uint8_t* vst = kst + kBytesK;
+    if (tile_start + kTile > L) {
+        constexpr int UPR = D / 8;
+        // Append: the block's K/V rows (positions L .. L+gamma) are not in the cache yet.
+        // The warp that owns those tokens puts them into the tile in shared memory, and
+        // the mt == 0 warp also stores them to their page slots.
+        const int p_first = max(L, tile_start + ts * NT), p_last = min(n_ctx, tile_start + ts * NT + NT);
+        for (int i = lane; i < (p_last - p_first) * UPR; i += 32) {
+            const int pos = p_first + i / UPR, u = i % UPR, row = pos - tile_start;
+            const size_t src = (((size_t)b * p.R + (pos - L)) * p.Hkv + g) * D + u * 8;
+            const uint4 kv = *reinterpret_cast<const uint4*>(p.k_new + src);
+            const uint4 vv = *reinterpret_cast<const uint4*>(p.v_new + src);
+            *reinterpret_cast<uint4*>(kst + (u / 8) * kRegion + swz(row, u % 8)) = kv;
+            *reinterpret_cast<uint4*>(vst + (u / 8) * kRegion + swz(row, u % 8)) = vv;
+            if (mt == 0) {
+                const int pid = page_of(pos);
+                if (pid >= 0 && pid < p.num_pages) {
+                    const size_t dst = (((size_t)pid * p.Hkv + g) * kPageSize + (pos % kPageSize)) * D + u * 8;
+                    *reinterpret_cast<uint4*>(p.k_pages + dst) = kv;
+                    *reinterpret_cast<uint4*>(p.v_pages + dst) = vv;
+                }
+            }
+        }
+        // Rows past the end of the context hold stale bytes; their weights are zero, but
+        // 0 * NaN would still poison P V, so clear the V rows this warp will read.
+        const int first = max(valid, ts * NT), last = ts * NT + NT;
+        for (int i = lane; i < (last - first) * UPR; i += 32) {
+            const int row = first + i / UPR, u = i % UPR;
+            *reinterpret_cast<uint4*>(vst + (u / 8) * kRegion + swz(row, u % 8)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncwarp();
+    }
+    const uint32_t k_base = smem_u32(kst), v_base = smem_u32(vst);
+
+    // ---- S = Q K^T for this warp's 16 rows x NT tokens
+    float sacc[NT / 8][4];
+#pragma unroll
+    for (int n = 0; n < NT / 8; ++n) { sacc[n][0] = sacc[n][1] = sacc[n][2] = sacc[n][3] = 0.f; }
+#pragma unroll
+    for (int kk = 0; kk < D / 16; ++kk) {
+        uint32_t a[4];
+        if (kQInRegs) {
+            a[0] = qf[kk][0]; a[1] = qf[kk][1]; a[2] = qf[kk][2]; a[3] = qf[kk][3];
+        } else {
+            const int row = mt * 16 + (lm & 1) * 8 + lr, unit = (kk & 3) * 2 + (lm >> 1);
+            ldmatrix_x4(a, q_base + (kk >> 2) * (RP * 128) + swz(row, unit));
+        }
+#pragma unroll
+        for (int tg = 0; tg < NT / 16; ++tg) {
+            uint32_t bf[4];
+            const int tok = ts * NT + tg * 16 + (lm >> 1) * 8 + lr, unit = (kk & 3) * 2 + (lm & 1);
+            ldmatrix_x4(bf, k_base + (kk >> 2) * kRegion + swz(tok, unit));
+            mma_bf16(sacc[2 * tg], a, bf[0], bf[1]);
+            mma_bf16(sacc[2 * tg + 1], a, bf[2], bf[3]);
+        }
+    }
+
+    // ---- scale, causal mask, online softmax
+    // some position in the tile is hidden from some block row: ahead of row 0, or (with a
+    // window) older than the last row's lower bound
+    const bool need_mask = tile_start + kTile > L + 1 || (p.window > 0 && tile_start < n_ctx - p.window);
+    float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+    for (int n = 0; n < NT / 8; ++n) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float sv = sacc[n][e] * scale_log2;
+            if (need_mask) {
+                const int pos = tile_start + ts * NT + n * 8 + 2 * (lane & 3) + (e & 1);
+                const int row_pos = L + (e < 2 ? j0 : j1);
+                if (pos > row_pos || (p.window > 0 && pos < row_pos - p.window + 1)) sv = -INFINITY;
+            }
+            sacc[n][e] = sv;
+            if (e < 2) mx0 = fmaxf(mx0, sv); else mx1 = fmaxf(mx1, sv);
+        }
+    }
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
+    const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
+    const float ms0 = mn0 == -INFINITY ? 0.f : mn0, ms1 = mn1 == -INFINITY ? 0.f : mn1;
+    const float corr0 = exp2f(m_run[0] - ms0), corr1 = exp2f(m_run[1] - ms1);
+    m_run[0] = mn0; m_run[1] = mn1;
+    float ls0 = 0.f, ls1 = 0.f;
+    uint32_t pa[NT / 16][4];
+#pragma unroll
+    for (int n = 0; n < NT / 8; ++n) {
+        const float p0 = exp2f(sacc[n][0] - ms0), p1 = exp2f(sacc[n][1] - ms0);
+        const float p2 = exp2f(sacc[n][2] - ms1), p3 = exp2f(sacc[n][3] - ms1);
+        ls0 += p0 + p1; ls1 += p2 + p3;
+        // accumulator layout -> A-operand layout of the P V product
+        pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16(p0, p1);
+        pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16(p2, p3);
+    }
+    l_run[0] = l_run[0] * corr0 + ls0;
+    l_run[1] = l_run[1] * corr1 + ls1;
+#pragma unroll
+    for (int n = 0; n < D / 8; ++n) { o[n][0] *= corr0; o[n][1] *= corr0; o[n][2] *= corr1; o[n][3] *= corr1; }
+
+    // ---- O += P V
+#pragma unroll
+    for (int tk = 0; tk < NT / 16; ++tk) {
+#pragma unroll
+        for (int dp = 0; dp < D / 16; ++dp) {
+            uint32_t bf[4];
+            const int tok = ts * NT + tk * 16 + (lm & 1) * 8 + lr, du = dp * 2 + (lm >> 1);
+            ldmatrix_x4_trans(bf, v_base + (du >> 3) * kRegion + swz(tok, du & 7));
+            mma_bf16(o[2 * dp], pa[tk], bf[0], bf[1]);
+            mma_bf16(o[2 * dp + 1], pa[tk], bf[2], bf[3]);
+        }
+    }
+}
+
 // Two CTAs should share an SM (one CTA's set-up and merge hide behind the other's
 // streaming).  Each scheduler owns a quarter of the register file and a CTA's warps are
 // dealt round-robin, so that needs at most four warps per CTA, producer included.
@@ -71,7 +199,6 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     using Cfg = AttnCfg<D, TILE, (MT * TS + 1 > 4)>;
     constexpr int kTile = TILE;
     constexpr int NW = MT * TS;            // consumer warps
-    constexpr int NT = kTile / TS;         // tokens of a tile owned by one warp
     constexpr int RP = MT * 16;            // padded query rows
     constexpr int NCH = Cfg::kChunks;
     constexpr bool kQInRegs = D <= 128;
@@ -193,120 +320,8 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             const uint32_t ph = ((uint32_t)(t / Cfg::kStages)) & 1u;
             if (!mbar_wait(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
             const int tile_start = c_begin + t * kTile;
-            const int valid = min(kTile, c_end - tile_start);
-            uint8_t* kst = smem + (size_t)s * Cfg::kStageBytes;
-            uint8_t* vst = kst + Cfg::kBytesK;
-            if (tile_start + kTile > L) {
-                constexpr int UPR = D / 8;
-                // Append: the block's K/V rows (positions L .. L+gamma) are not in the cache yet.
-                // The warp that owns those tokens puts them into the tile in shared memory, and
-                // the mt == 0 warp also stores them to their page slots.
-                const int p_first = max(L, tile_start + ts * NT), p_last = min(n_ctx, tile_start + ts * NT + NT);
-                for (int i = lane; i < (p_last - p_first) * UPR; i += 32) {
-                    const int pos = p_first + i / UPR, u = i % UPR, row = pos - tile_start;
-                    const size_t src = (((size_t)b * p.R + (pos - L)) * p.Hkv + g) * D + u * 8;
-                    const uint4 kv = *reinterpret_cast<const uint4*>(p.k_new + src);
-                    const uint4 vv = *reinterpret_cast<const uint4*>(p.v_new + src);
-                    *reinterpret_cast<uint4*>(kst + (u / 8) * Cfg::kRegion + swz(row, u % 8)) = kv;
-                    *reinterpret_cast<uint4*>(vst + (u / 8) * Cfg::kRegion + swz(row, u % 8)) = vv;
-                    if (mt == 0) {
-                        const int pid = s_pages[(pos - c_begin) / kPageSize];
-                        if (pid >= 0 && pid < p.num_pages) {
-                            const size_t dst = (((size_t)pid * p.Hkv + g) * kPageSize + (pos % kPageSize)) * D + u * 8;
-                            *reinterpret_cast<uint4*>(p.k_pages + dst) = kv;
-                            *reinterpret_cast<uint4*>(p.v_pages + dst) = vv;
-                        }
-                    }
-                }
-                // Rows past the end of the context hold stale bytes; their weights are zero, but
-                // 0 * NaN would still poison P V, so clear the V rows this warp will read.
-                const int first = max(valid, ts * NT), last = ts * NT + NT;
-                for (int i = lane; i < (last - first) * UPR; i += 32) {
-                    const int row = first + i / UPR, u = i % UPR;
-                    *reinterpret_cast<uint4*>(vst + (u / 8) * Cfg::kRegion + swz(row, u % 8)) = make_uint4(0u, 0u, 0u, 0u);
-                }
-                __syncwarp();
-            }
-            const uint32_t k_base = smem_u32(kst), v_base = smem_u32(vst);
-
-            // ---- S = Q K^T for this warp's 16 rows x NT tokens
-            float sacc[NT / 8][4];
-#pragma unroll
-            for (int n = 0; n < NT / 8; ++n) { sacc[n][0] = sacc[n][1] = sacc[n][2] = sacc[n][3] = 0.f; }
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                uint32_t a[4];
-                if (kQInRegs) {
-                    a[0] = qf[kk][0]; a[1] = qf[kk][1]; a[2] = qf[kk][2]; a[3] = qf[kk][3];
-                } else {
-                    const int row = mt * 16 + (lm & 1) * 8 + lr, unit = (kk & 3) * 2 + (lm >> 1);
-                    ldmatrix_x4(a, q_base + (kk >> 2) * (RP * 128) + swz(row, unit));
-                }
-#pragma unroll
-                for (int tg = 0; tg < NT / 16; ++tg) {
-                    uint32_t bf[4];
-                    const int tok = ts * NT + tg * 16 + (lm >> 1) * 8 + lr, unit = (kk & 3) * 2 + (lm & 1);
-                    ldmatrix_x4(bf, k_base + (kk >> 2) * Cfg::kRegion + swz(tok, unit));
-                    mma_bf16(sacc[2 * tg], a, bf[0], bf[1]);
-                    mma_bf16(sacc[2 * tg + 1], a, bf[2], bf[3]);
-                }
-            }
-
-            // ---- scale, causal mask, online softmax
-            // some position in the tile is hidden from some block row: ahead of row 0, or (with a
-            // window) older than the last row's lower bound
-            const bool need_mask = tile_start + kTile > L + 1 || (p.window > 0 && tile_start < n_ctx - p.window);
-            float mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll
-            for (int n = 0; n < NT / 8; ++n) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float sv = sacc[n][e] * scale_log2;
-                    if (need_mask) {
-                        const int pos = tile_start + ts * NT + n * 8 + 2 * (lane & 3) + (e & 1);
-                        const int row_pos = L + (e < 2 ? j0 : j1);
-                        if (pos > row_pos || (p.window > 0 && pos < row_pos - p.window + 1)) sv = -INFINITY;
-                    }
-                    sacc[n][e] = sv;
-                    if (e < 2) mx0 = fmaxf(mx0, sv); else mx1 = fmaxf(mx1, sv);
-                }
-            }
-            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-            const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
-            const float ms0 = mn0 == -INFINITY ? 0.f : mn0, ms1 = mn1 == -INFINITY ? 0.f : mn1;
-            const float corr0 = exp2f(m_run[0] - ms0), corr1 = exp2f(m_run[1] - ms1);
-            m_run[0] = mn0; m_run[1] = mn1;
-            float ls0 = 0.f, ls1 = 0.f;
-            uint32_t pa[NT / 16][4];
-#pragma unroll
-            for (int n = 0; n < NT / 8; ++n) {
-                const float p0 = exp2f(sacc[n][0] - ms0), p1 = exp2f(sacc[n][1] - ms0);
-                const float p2 = exp2f(sacc[n][2] - ms1), p3 = exp2f(sacc[n][3] - ms1);
-                ls0 += p0 + p1; ls1 += p2 + p3;
-                // accumulator layout -> A-operand layout of the P V product
-                pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16(p0, p1);
-                pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16(p2, p3);
-            }
-            l_run[0] = l_run[0] * corr0 + ls0;
-            l_run[1] = l_run[1] * corr1 + ls1;
-#pragma unroll
-            for (int n = 0; n < D / 8; ++n) { o[n][0] *= corr0; o[n][1] *= corr0; o[n][2] *= corr1; o[n][3] *= corr1; }
-
-            // ---- O += P V
-#pragma unroll
-            for (int tk = 0; tk < NT / 16; ++tk) {
-#pragma unroll
-                for (int dp = 0; dp < D / 16; ++dp) {
-                    uint32_t bf[4];
-                    const int tok = ts * NT + tk * 16 + (lm & 1) * 8 + lr, du = dp * 2 + (lm >> 1);
-                    ldmatrix_x4_trans(bf, v_base + (du >> 3) * Cfg::kRegion + swz(tok, du & 7));
-                    mma_bf16(o[2 * dp], pa[tk], bf[0], bf[1]);
-                    mma_bf16(o[2 * dp + 1], pa[tk], bf[2], bf[3]);
-                }
-            }
+            attend_tile<D, MT, TS, TILE>(p, b, g, L, c_end, tile_start, smem + (size_t)s * Cfg::kStageBytes, q_base, qf, mt, ts, lane, j0, j1, scale_log2,
+                                         [&](int pos) { return s_pages[(pos - c_begin) / kPageSize]; }, o, m_run, l_run);
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty_bar[s]);
         }
@@ -376,6 +391,292 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     }
 }
 
+// ---- The balanced schedule (as in attn_umma.cu): the tiles of all (sequence, KV head) pairs form one line ordered by
+// (sequence, head, position), a persistent grid cuts it into equal ranges, and a CTA leaves at most two pieces of cut pairs to
+// attn_flat_combine_kernel, in the layout the accumulators have in registers.  The ring runs on across the pairs of a
+// range: while the compute warps merge and write one pair, the producer is already filling the next one's tiles.
+// Against a grid of fixed chunks every CTA streams the same bytes whatever the mix of lengths and window bounds, and pays
+// its set-up once.
+template <int D, int MT, int TILE>
+struct FlatCfg {
+    static constexpr int kTS = 2;                          // warps that share 16 query rows, each with half of a tile's tokens
+    static constexpr int kWarps = MT * kTS;
+    static constexpr int kChunks = D / 64;
+    static constexpr int kRegion = TILE * 128;
+    static constexpr int kBytesK = kChunks * kRegion;
+    static constexpr int kStageBytes = 2 * kBytesK;
+    // up to 16 rows: two CTAs per SM with three stages each; above, one CTA needs the shared memory and the warps alone
+    static constexpr int kStages = MT == 1 ? 3 : (MT == 4 ? 5 : 6);
+    static constexpr int kCtasPerSm = MT == 1 ? 2 : 1;
+    static constexpr int kQBytes = MT * 16 * D * 2;
+    static constexpr int kSmem = kStages * kStageBytes + kQBytes + 1024;      // and (B + 1) ints
+};
+
+template <int D, int MT, int TILE>
+__global__ void __launch_bounds__((FlatCfg<D, MT, TILE>::kWarps + 1) * 32, FlatCfg<D, MT, TILE>::kCtasPerSm)
+attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_q,
+                 const AttnParams p) {
+    using Cfg = FlatCfg<D, MT, TILE>;
+    static_assert(D == 256, "the exchange between the two warps of a row group goes through the query rows' space");
+    constexpr int NW = Cfg::kWarps, RP = MT * 16, TS = Cfg::kTS, E = Cfg::kStages, NCH = Cfg::kChunks, UPR = D / 8;
+    constexpr int PPT = TILE / kPageSize, GROUP = 32 / PPT;           // pages per tile; tiles whose page ids fit one register per lane
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[E], empty_bar[E];
+    __shared__ float s_m[NW][16], s_l[NW][16];
+    __shared__ int abort_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int G = p.Hq / p.Hkv, rows = G * p.R;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* q_smem = smem + E * Cfg::kStageBytes;                   // [NCH][RP rows][128 B], swizzled
+    int* s_cum = reinterpret_cast<int*>(q_smem + Cfg::kQBytes);      // tiles of sequences 0 .. b-1 (per KV head)
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < E; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], NW); }
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    pdl_wait();
+
+    // tiles per pair of every sequence, then an exclusive prefix sum over the batch
+    auto first_tile = [&](int L) { return (p.window > 0 ? max(0, L - p.window + 1) : 0) / TILE; };
+    for (int i = threadIdx.x; i < p.B; i += blockDim.x) {
+        const int L = p.seq_lens[i];
+        int n = 0;
+        if (L < 0 || L + p.R > p.max_pages * kPageSize) {            // no room for the block: skip the sequence
+            if (blockIdx.x == 0) set_status(p.dev_status, MASSV_ERR_CAPACITY);
+        } else {
+            n = (L + p.R + TILE - 1) / TILE - first_tile(L);
+        }
+        s_cum[i + 1] = n;
+    }
+    if (threadIdx.x == 0) s_cum[0] = 0;
+    __syncthreads();
+    if (warp == 0) {
+        const int per = (p.B + 31) / 32;
+        const int i0 = min(p.B, lane * per), i1 = min(p.B, i0 + per);
+        int local = 0;
+        for (int i = i0; i < i1; ++i) local += s_cum[i + 1];
+        int incl = local;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        int run = incl - local;
+        for (int i = i0; i < i1; ++i) { run += s_cum[i + 1]; s_cum[i + 1] = run; }
+    }
+    __syncthreads();
+    const int total = s_cum[p.B] * p.Hkv;
+    const int per_cta = max(1, (total + (int)gridDim.x - 1) / (int)gridDim.x);
+    if (blockIdx.x == 0) {          // what the merge kernel needs to find the pieces of a pair
+        for (int i = threadIdx.x; i <= p.B; i += blockDim.x) p.flat_meta[2 + i] = s_cum[i];
+        if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = total; }
+    }
+    const int f_first = min(total, (int)blockIdx.x * per_cta), f_end = min(total, f_first + per_cta);
+    volatile int* abort_ptr = &abort_flag;
+
+    // Piece of work at tile f of the line: a run of tiles of one pair, up to this CTA's end.
+    struct Piece { int b, g, L, c_begin, c_end, n_tiles; bool whole; };
+    int b_hint = 0;
+    auto piece_at = [&](int f) {
+        int lo = b_hint, hi = p.B - 1;                               // largest b with Hkv * cum[b] <= f
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_cum[mid] * p.Hkv <= f) lo = mid; else hi = mid - 1;
+        }
+        b_hint = lo;
+        const int n_b = s_cum[lo + 1] - s_cum[lo], off = f - s_cum[lo] * p.Hkv;
+        const int t0 = off % n_b, t1 = min(n_b, t0 + (f_end - f));
+        Piece w;
+        w.b = lo; w.g = off / n_b; w.L = p.seq_lens[lo];
+        const int tile_lo = first_tile(w.L);
+        w.c_begin = (tile_lo + t0) * TILE;
+        w.c_end = min(w.L + p.R, (tile_lo + t1) * TILE);
+        w.n_tiles = t1 - t0;
+        w.whole = t0 == 0 && t1 == n_b;
+        return w;
+    };
+
+    if (warp == NW) {
+        // ------------------------------------------------ TMA producer: one box per lane (16 per full tile)
+        uint64_t policy;
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int f = f_first; f < f_end && ok;) {
+            const Piece w = piece_at(f);
+            f += w.n_tiles;
+            // page ids travel in registers, lane l holding page 32 * group + l; the next group's are fetched a group ahead
+            const int32_t* pt = p.page_table + (size_t)w.b * p.max_pages + w.c_begin / kPageSize;
+            const int n_pages = (w.c_end - w.c_begin + kPageSize - 1) / kPageSize;
+            int pid_cur = lane < n_pages ? pt[lane] : 0, pid_next = 32 + lane < n_pages ? pt[32 + lane] : 0;
+            {
+                // The pair's query rows travel through the ring ahead of its tiles (row r = block_row * G + head_in_group, and the
+                // G heads of a block row are adjacent in memory: one box per block row and 64-element column group).
+                int freed = 0;
+                if (lane == 0) freed = mbar_wait(&empty_bar[s], ph ^ 1u, abort_ptr) ? 1 : 0;
+                if (!__shfl_sync(0xffffffffu, freed, 0)) { ok = false; break; }
+                if (lane == 0) mbar_expect_tx(&full_bar[s], (uint32_t)(rows * D * 2));
+                __syncwarp();
+                static_assert(kMaxRows * NCH <= 32, "one box per lane");
+                const int j = lane / NCH, dc = lane % NCH;
+                if (j < p.R)
+                    tma_load_2d(smem + (size_t)s * Cfg::kStageBytes + dc * (RP * 128) + j * G * 128, &map_q, dc * 64, (w.b * p.R + j) * p.Hq + w.g * G,
+                                &full_bar[s], policy);
+                if (++s == E) { s = 0; ph ^= 1u; }
+            }
+            for (int t = 0; t < w.n_tiles; ++t) {
+                if (t > 0 && t % GROUP == 0) {
+                    pid_cur = pid_next;
+                    const int nxt = (t / GROUP + 1) * 32 + lane;
+                    pid_next = nxt < n_pages ? pt[nxt] : 0;
+                }
+                int freed = 0;
+                if (lane == 0) freed = mbar_wait(&empty_bar[s], ph ^ 1u, abort_ptr) ? 1 : 0;
+                if (!__shfl_sync(0xffffffffu, freed, 0)) { ok = false; break; }
+                const int n_pg = min(PPT, n_pages - t * PPT);
+                uint8_t* dst = smem + (size_t)s * Cfg::kStageBytes;
+                if (lane == 0) mbar_expect_tx(&full_bar[s], (uint32_t)(n_pg * NCH * 2048 * 2));
+                __syncwarp();
+                const int is_v = lane & 1, dc = (lane >> 1) % NCH, pg = lane / (2 * NCH);
+                static_assert(2 * NCH * PPT <= 32, "one box per lane");
+                int pid = __shfl_sync(0xffffffffu, pid_cur, (t % GROUP) * PPT + min(pg, PPT - 1));
+                if (pg < n_pg) {
+                    if (pid < 0 || pid >= p.num_pages) { set_status(p.dev_status, MASSV_ERR_CAPACITY); pid = 0; }
+                    tma_load_2d(dst + is_v * Cfg::kBytesK + dc * Cfg::kRegion + pg * 2048, is_v ? &map_v : &map_k, dc * 64,
+                                (pid * p.Hkv + w.g) * kPageSize, &full_bar[s], policy);
+                }
+                if (++s == E) { s = 0; ph ^= 1u; }
+            }
+        }
+        if (!ok && lane == 0) {
+            for (int i = 0; i < 64; ++i) __nanosleep(2000);          // let copies in flight land
+        }
+    } else {
+        // ------------------------------------------------ compute warps (one that gave up waiting still meets the barriers)
+        auto sync_warps = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NW * 32) : "memory"); };
+        const int mt = warp / TS, ts = warp % TS;
+        const float scale_log2 = p.scale * 1.4426950408889634f;
+        const int r0 = mt * 16 + (lane >> 2), r1 = r0 + 8;
+        // block row of each of this thread's two query rows (padding rows behave like the last block row)
+        const int j0 = r0 < rows ? r0 / G : p.R - 1, j1 = r1 < rows ? r1 / G : p.R - 1;
+        const uint32_t q_base = smem_u32(q_smem);
+        float4* exchange = reinterpret_cast<float4*>(q_smem + mt * 16 * D * 2) + lane;     // half of the columns of 16 rows
+        const uint32_t no_q[1][4] = {{0u, 0u, 0u, 0u}};
+        int s = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int f = f_first; f < f_end;) {
+            const Piece w = piece_at(f);
+            const size_t slot = (size_t)blockIdx.x * 2 + (f == f_first ? 0 : 1);
+            f += w.n_tiles;
+            // the pair's query rows, from their ring stage to their place (same layout; zeros past the last row)
+            if (ok && !mbar_wait_warp(&full_bar[s], ph, abort_ptr)) ok = false;
+            for (int i = threadIdx.x; i < RP * UPR; i += NW * 32) {
+                const int r = (i / 8) % RP;
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (r < rows) v = *reinterpret_cast<const uint4*>(smem + (size_t)s * Cfg::kStageBytes + (size_t)i * 16);
+                *reinterpret_cast<uint4*>(q_smem + (size_t)i * 16) = v;
+            }
+            sync_warps();
+            if (lane == 0) mbar_arrive(&empty_bar[s]);
+            if (++s == E) { s = 0; ph ^= 1u; }
+            float o[D / 8][4];
+#pragma unroll
+            for (int n = 0; n < D / 8; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
+            float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+            for (int t = 0; t < w.n_tiles && ok; ++t) {
+                if (!mbar_wait_warp(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
+                attend_tile<D, MT, TS, TILE>(p, w.b, w.g, w.L, w.c_end, w.c_begin + t * TILE, smem + (size_t)s * Cfg::kStageBytes, q_base, no_q, mt, ts,
+                                             lane, j0, j1, scale_log2, [&](int pos) { return p.page_table[(size_t)w.b * p.max_pages + pos / kPageSize]; },
+                                             o, m_run, l_run);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty_bar[s]);
+                if (++s == E) { s = 0; ph ^= 1u; }
+            }
+            l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 1);
+            l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 2);
+            l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 1);
+            l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 2);
+            if ((lane & 3) == 0) {
+                s_m[warp][lane >> 2] = m_run[0]; s_l[warp][lane >> 2] = l_run[0];
+                s_m[warp][(lane >> 2) + 8] = m_run[1]; s_l[warp][(lane >> 2) + 8] = l_run[1];
+            }
+            sync_warps();                      // the query rows have been read: their space carries the exchange
+            // the second warp of a row group hands its accumulator over, half of the columns at a time
+            float own[2], other[2], M[2];
+            {
+                const int peer = warp ^ 1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int r = (lane >> 2) + 8 * h;
+                    const float mo = s_m[peer][r];
+                    M[h] = fmaxf(m_run[h], mo);
+                    own[h] = m_run[h] == -INFINITY ? 0.f : exp2f(m_run[h] - M[h]);
+                    other[h] = mo == -INFINITY ? 0.f : exp2f(mo - M[h]);
+                    l_run[h] = l_run[h] * own[h] + s_l[peer][r] * other[h];
+                }
+            }
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                if (ts == 1) {
+#pragma unroll
+                    for (int k = 0; k < D / 16; ++k) {
+                        const int n = half * (D / 16) + k;
+                        exchange[k * 32] = make_float4(o[n][0], o[n][1], o[n][2], o[n][3]);
+                    }
+                }
+                sync_warps();
+                if (ts == 0) {
+#pragma unroll
+                    for (int k = 0; k < D / 16; ++k) {
+                        const int n = half * (D / 16) + k;
+                        const float4 v = exchange[k * 32];
+                        o[n][0] = o[n][0] * own[0] + v.x * other[0]; o[n][1] = o[n][1] * own[0] + v.y * other[0];
+                        o[n][2] = o[n][2] * own[1] + v.z * other[1]; o[n][3] = o[n][3] * own[1] + v.w * other[1];
+                    }
+                }
+                sync_warps();
+            }
+            if (ts != 0 || mt * 16 >= rows || !ok) continue;
+            if (!w.whole) {
+                // unit (mt * D/8 + n) * 32 + lane of the piece: (row r0: columns c, c+1; row r1: the same), c = 8 n + 2 (lane % 4)
+                size_t at = slot;
+                if (!MASSV_IN_BOUNDS(at, 2 * kFlatMaxCtas, p.dev_status)) at = 0;
+                float4* dst = reinterpret_cast<float4*>(p.flat_part_o + at * RP * D) + mt * (D / 8) * 32 + lane;
+#pragma unroll
+                for (int n = 0; n < D / 8; ++n) dst[n * 32] = make_float4(o[n][0], o[n][1], o[n][2], o[n][3]);
+                if ((lane & 3) == 0) {
+                    float2* ml = reinterpret_cast<float2*>(p.flat_part_ml + at * RP * 2);
+                    ml[r0] = make_float2(M[0], l_run[0]);
+                    ml[r1] = make_float2(M[1], l_run[1]);
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int r = h ? r1 : r0;
+                    if (r >= rows) continue;
+                    const size_t row_out = ((size_t)w.b * p.R + r / G) * p.Hq + w.g * G + r % G;
+                    const float inv = 1.f / l_run[h];
+#pragma unroll
+                    for (int n = 0; n < D / 8; ++n) {
+                        const float x = o[n][2 * h] * inv, y = o[n][2 * h + 1] * inv;
+                        const size_t at = row_out * D + n * 8 + 2 * (lane & 3);
+                        *reinterpret_cast<uint32_t*>(p.out + at) = pack_bf16(x, y);
+                        if (p.out_f32) *reinterpret_cast<float2*>(p.out_f32 + at) = make_float2(x, y);
+                    }
+                    if (p.lse && (lane & 3) == 0) p.lse[row_out] = (M[h] + log2f(l_run[h])) * 0.6931471805599453f;
+                }
+            }
+        }
+    }
+    pdl_trigger();
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_flag) set_status(p.dev_status, MASSV_ERR_TIMEOUT);
+}
+
 // Merge the chunks of sequences that span more than one: one CTA per
 // (sequence, KV head, query row), one thread per channel.
 constexpr int kCombineMaxChunks = 1024;
@@ -438,6 +739,21 @@ cudaError_t launch_split(const AttnParams& p, const CUtensorMap& mk, const CUten
     return launch_pdl(attn_split_kernel<D, MT, TS, TILE>, dim3(p.max_chunks, p.Hkv, p.B), dim3((MT * TS + 1) * 32), smem, stream, mk, mv, p);
 }
 
+template <int D, int MT, int TILE>
+cudaError_t launch_flat(const AttnParams& p, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t stream, int* ctas) {
+    using Cfg = FlatCfg<D, MT, TILE>;
+    const size_t smem = (size_t)Cfg::kSmem + (size_t)(p.B + 1) * sizeof(int);
+    static_assert(Cfg::kSmem + (kFlatMaxBatchMeta + 1) * 4 <= 226 * 1024, "ring, query rows and tile counts fit shared memory");
+    cudaError_t e = cudaFuncSetAttribute(attn_flat_kernel<D, MT, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    *ctas = device_sm_count() * Cfg::kCtasPerSm;
+    if (*ctas > kFlatMaxCtas) *ctas = kFlatMaxCtas;
+    // the query rows as a [B * R * Hq, D] matrix; a box is the G adjacent heads of one block row
+    CUtensorMap mq;
+    if (!make_tensor_map_bf16_2d(&mq, p.q, (uint64_t)p.B * p.R * p.Hq, D, (uint32_t)(p.Hq / p.Hkv))) return cudaErrorInvalidValue;
+    return launch_pdl(attn_flat_kernel<D, MT, TILE>, dim3(*ctas), dim3((Cfg::kWarps + 1) * 32), smem, stream, mk, mv, mq, p);
+}
+
 template <int D>
 cudaError_t launch_split_d(const AttnParams& p, int mt, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t stream) {
     switch (mt) {
@@ -466,6 +782,22 @@ bool attn_use_umma(const AttnParams& p) {
     return p.d <= 128;
 }
 
+// Balanced schedule or chunk grid for the warp-MMA kernel at head_dim 256.  The balanced one wins wherever a pair's tiles
+// are many or pairs are few (batch 32 x 8 heads: contexts 2k - 8k 228 -> 207 us, window 1,024 72 -> 57 us; batch 2, 1,000
+// positions 20 -> 16 us; 36 query rows 284 -> 176 us).  It loses where a pair is a few tiles and there are enough pairs
+// to occupy the chip one by one: a grid of one-pair CTAs has no ranges to cut and no pieces to merge (64 x 8 pairs: up to
+// 100 positions 21 against 29 us, up to 512 43 against 48, up to 1,024 75 against 71; 16 x 8 pairs up to 512: 19 against
+// 21).  From 17 rows up the balanced kernel's two warps per row group outweigh that except for the shortest
+// (64 x 4 pairs of 36 rows, up to 100 positions: 40 against 45 us, up to 256: 51 against 46).
+static bool use_flat_warp_mma(const AttnParams& p, int mt) {
+    if (p.d != 256 || p.chunk_forced || p.B > kFlatMaxBatchMeta) return false;
+    long tokens = (long)p.max_pages * kPageSize;                     // the most a pair can need
+    if (p.window > 0 && p.window + p.R + 64 < tokens) tokens = p.window + p.R + 64;
+    const long pairs = (long)p.B * p.Hkv, ctas = (long)device_sm_count() * (mt == 1 ? 2 : 1);
+    if (mt == 1) return tokens > 544 || pairs * 5 < ctas * 2;
+    return tokens > 128 || pairs < ctas;
+}
+
 cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream) {
     if (p.kv_chunk % kChunkAlign != 0 || p.kv_chunk > kMaxChunkPages * kPageSize) return cudaErrorInvalidValue;
     CUtensorMap mk, mv;
@@ -487,6 +819,21 @@ cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream) {
             count_launches(launched);
             return cudaGetLastError();
         }
+    } else if (use_flat_warp_mma(p, mt)) {
+        int ctas = 0;
+        switch (mt) {
+            case 1: e = launch_flat<256, 1, 32>(p, mk, mv, stream, &ctas); break;
+            case 2: e = launch_flat<256, 2, 32>(p, mk, mv, stream, &ctas); break;
+            case 3: e = launch_flat<256, 3, 32>(p, mk, mv, stream, &ctas); break;
+            case 4: e = launch_flat<256, 4, 32>(p, mk, mv, stream, &ctas); break;
+            default: return cudaErrorInvalidValue;
+        }
+        if (e != cudaSuccess) return e;
+        if (hooks.attn_stop && cudaEventRecord(hooks.attn_stop, stream) != cudaSuccess) return cudaGetLastError();
+        e = launch_flat_combine(p, ctas, stream);
+        if (e != cudaSuccess) return e;
+        count_launches(2);
+        return cudaGetLastError();
     } else {
         switch (p.d) {
             case 64: e = launch_split_d<64>(p, mt, mk, mv, stream); break;

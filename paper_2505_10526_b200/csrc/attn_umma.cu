@@ -864,6 +864,25 @@ int flat_sm_count() {
     return n;
 }
 
+}  // namespace
+
+cudaError_t launch_flat_combine(const AttnParams& p, int ctas, cudaStream_t stream) {
+    const int rows = (p.Hq / p.Hkv) * p.R;
+    // enough CTAs to fill the machine: a pair's groups of 16 rows go to separate CTAs, and with few pairs a
+    // group's units (d/64 * 256 of them) are cut further into 2, 4, 8 or 16 parts
+    const int pairs = p.B * p.Hkv, rows_pad = attn_rows_pad(rows), n_qd = rows_pad / 16, units_per_qd = (p.d / 64) * 256;
+    int parts = 1;
+    while (parts < 16 && units_per_qd / (parts * 2) >= 32 && pairs * n_qd * parts < 2 * flat_sm_count()) parts *= 2;
+    // (max, sum) and weight of 16 rows for at most `ctas` pieces of a pair (a pair can span every CTA)
+    const size_t comb_smem = (2 * (size_t)ctas + 1) * 16 * sizeof(float) + kFlatCombineThreads * sizeof(float4);
+    const cudaError_t e = cudaFuncSetAttribute(attn_flat_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)comb_smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(attn_flat_combine_kernel, dim3(pairs, n_qd * parts), dim3(kFlatCombineThreads), comb_smem, stream, p, rows_pad, parts,
+                      units_per_qd / parts);
+}
+
+namespace {
+
 template <int D, int TILE>
 cudaError_t launch_umma(const AttnParams& p, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t stream, bool flat, int* launched,
                         cudaEvent_t split_done) {
@@ -882,18 +901,7 @@ cudaError_t launch_umma(const AttnParams& p, const CUtensorMap& mk, const CUtens
         e = launch_pdl(attn_umma_kernel<D, TILE, true>, dim3(ctas), dim3(kUmmaThreads), (size_t)Cfg::kSmem, stream, mk, mv, mq, p);
         if (e != cudaSuccess) return e;
         if (split_done && cudaEventRecord(split_done, stream) != cudaSuccess) return cudaGetLastError();
-        const int rows = (p.Hq / p.Hkv) * p.R;
-        // enough CTAs to fill the machine: a pair's groups of 16 rows go to separate CTAs, and with few pairs a
-        // group's units (D/64 * 256 of them) are cut further into 2, 4, 8 or 16 parts
-        const int pairs = p.B * p.Hkv, rows_pad = attn_rows_pad(rows), n_qd = rows_pad / 16, units_per_qd = (D / 64) * 256;
-        int parts = 1;
-        while (parts < 16 && units_per_qd / (parts * 2) >= 32 && pairs * n_qd * parts < 2 * flat_sm_count()) parts *= 2;
-        // (max, sum) and weight of 16 rows for at most `ctas` pieces of a pair (a pair can span every CTA)
-        const size_t comb_smem = (2 * (size_t)ctas + 1) * 16 * sizeof(float) + kFlatCombineThreads * sizeof(float4);
-        e = cudaFuncSetAttribute(attn_flat_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)comb_smem);
-        if (e != cudaSuccess) return e;
-        e = launch_pdl(attn_flat_combine_kernel, dim3(pairs, n_qd * parts), dim3(kFlatCombineThreads), comb_smem, stream, p, rows_pad, parts,
-                       units_per_qd / parts);
+        e = launch_flat_combine(p, ctas, stream);
         *launched = 2;
         return e;
     }

@@ -25,7 +25,7 @@ struct AttnParams {
     int32_t* dev_status;
     int path;          // 0: choose by shape, 1: warp-level MMA kernel, 2: tcgen05 kernel
     bool chunk_forced; // the caller fixed kv_chunk: keep the (chunk, KV head, sequence) grid
-    // flat schedule of the tcgen05 kernel: two partial slots per resident CTA, and what the merge needs
+    // flat schedules: two partial slots per resident CTA, and what the merge needs
     float* flat_part_o;    // [kFlatMaxCtas * 2, rows_pad, d]
     float* flat_part_ml;   // [kFlatMaxCtas * 2, rows_pad, 2]
     int32_t* flat_meta;    // [0] tiles per CTA, [1] tiles in all, [2 + b] tiles of sequences 0 .. b-1 (per KV head)
@@ -34,6 +34,8 @@ constexpr int kFlatMaxCtas = 320;      // resident CTAs of the flat schedule (tw
 constexpr int kFlatMaxBatchMeta = 1024;
 int attn_rows_pad(int group_rows);                 // query rows per KV head, padded to the MMA tile
 cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream);
+// Merge of the pieces a flat schedule of `ctas` CTAs left (attn_umma.cu; the warp-MMA kernel's flat schedule uses it too).
+cudaError_t launch_flat_combine(const AttnParams& p, int ctas, cudaStream_t stream);
 // tcgen05 variant of the split kernel (attn_umma.cu); the tensor maps are the ones the warp-MMA kernel uses
 bool attn_umma_supported(const AttnParams& p);
 bool attn_umma_flat_supported(const AttnParams& p);

@@ -1,0 +1,76 @@
+"""The balanced schedule of the warp-MMA kernel at head_dim 256: pairs cut between CTAs and ranges of several pairs, every
+number of row groups, windows, lengths from zero, ragged ends, against attention in fp32 on the same bf16 values."""
+import math
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(batch, gamma, q_heads, kv_heads, lens, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    R, d = gamma + 1, 256
+    max_pages = (max(lens) + R + 15) // 16
+    n_pages = batch * max_pages + 2
+    bf = dict(dtype=torch.bfloat16, device="cuda", generator=g)
+    table = torch.randperm(n_pages, generator=g, device="cuda")[:batch * max_pages].view(batch, max_pages).to(torch.int32)
+    return dict(q=torch.randn((batch, R, q_heads, d), **bf), k_new=torch.randn((batch, R, kv_heads, d), **bf),
+                v_new=torch.randn((batch, R, kv_heads, d), **bf), k_pages=torch.randn((n_pages, kv_heads, 16, d), **bf),
+                v_pages=torch.randn((n_pages, kv_heads, 16, d), **bf), page_table=table.contiguous(),
+                seq_lens=torch.tensor(lens, dtype=torch.int32, device="cuda"))
+
+
+def _reference(w, window):
+    B, R, hq, d = w["q"].shape
+    hkv = w["k_new"].shape[2]
+    G = hq // hkv
+    out, lse = torch.empty((B, R, hq, d), device="cuda"), torch.empty((B, R, hq), device="cuda")
+    for b, n in enumerate(w["seq_lens"].tolist()):
+        pages = w["page_table"][b].long()
+        k, v = (torch.cat([w[p][pages].transpose(0, 1).reshape(hkv, -1, d)[:, :n], w[x][b].transpose(0, 1)], dim=1).double()
+                for p, x in (("k_pages", "k_new"), ("v_pages", "v_new")))
+        q = w["q"][b].double().view(R, hkv, G, d).permute(1, 0, 2, 3).reshape(hkv, R * G, d)
+        s = q @ k.transpose(1, 2) / math.sqrt(d)
+        pos, row = torch.arange(n + R, device="cuda"), n + torch.arange(R, device="cuda").repeat_interleave(G)
+        hidden = pos[None] > row[:, None]
+        if window:
+            hidden |= pos[None] <= row[:, None] - window
+        s.masked_fill_(hidden[None], -math.inf)
+        out[b] = (torch.softmax(s, -1) @ v).view(hkv, R, G, d).permute(1, 0, 2, 3).reshape(R, hq, d)
+        lse[b] = torch.logsumexp(s, -1).view(hkv, R, G).permute(1, 0, 2).reshape(R, hq)
+    return out, lse
+
+
+@pytest.mark.parametrize("batch,gamma,q_heads,kv_heads,lo,hi,window", [
+    (1, 5, 2, 1, 0, 0, 0), (3, 0, 4, 4, 31, 33, 0), (2, 5, 16, 8, 9000, 9100, 0), (48, 5, 16, 8, 100, 1500, 0), (40, 3, 16, 8, 700, 2000, 512),
+    (64, 1, 8, 8, 0, 100, 0), (20, 3, 32, 4, 0, 900, 0), (24, 5, 32, 4, 300, 900, 0), (9, 7, 8, 1, 5, 2500, 0), (30, 7, 16, 2, 600, 1800, 300),
+    (150, 2, 4, 2, 0, 700, 0), (5, 5, 16, 8, 2000, 3000, 1)])
+def test_against_fp32(batch, gamma, q_heads, kv_heads, lo, hi, window):
+    import paper_2505_10526_b200 as mv
+    g = torch.Generator().manual_seed(batch + hi)
+    lens = torch.randint(lo, hi + 1, (batch,), generator=g).tolist()
+    w = _inputs(batch, gamma, q_heads, kv_heads, lens, seed=hi + gamma)
+    want, want_lse = _reference(w, window)
+    desc = mv.attn_desc(batch, gamma, q_heads, kv_heads, 256, w["page_table"].shape[1], w["k_pages"].shape[0], window=window)
+    ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda")
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+
+    def run():
+        out = torch.full_like(w["q"], float("nan"))
+        f32 = torch.full(out.shape, float("nan"), device="cuda")
+        lse = torch.full(out.shape[:3], float("nan"), device="cuda")
+        mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, lse, ws, status)
+        return out, f32, lse
+
+    out, f32, lse = run()
+    again = run()
+    assert int(status.item()) == 0
+    # softmax weights carry bf16's 2^-9; values of a few units, weights that sum to one: 5e-3 of the fp32 output, bf16 on top of it
+    assert float((f32 - want).abs().max()) < 1e-2 and float((out.float() - want).abs().max()) < 3e-2
+    assert float((lse - want_lse).abs().max()) < 1e-3
+    assert all(torch.equal(a, b) for a, b in zip((out, f32, lse), again))
+    for b, n in enumerate(lens):                          # the block's rows are in their slots
+        for j in range(gamma + 1):
+            page, at = int(w["page_table"][b, (n + j) // 16]), (n + j) % 16
+            assert torch.equal(w["k_pages"][page, :, at], w["k_new"][b, j]) and torch.equal(w["v_pages"][page, :, at], w["v_new"][b, j])
