@@ -827,31 +827,54 @@ __global__ void shard_publish_kernel(PublishParams p) {
     }
 }
 
-// Dense probabilities for callers that ask for them (diagnostics / tests).
-__global__ void probs_kernel(AcceptParams p) {
-    const int R = p.gamma + 1, M = p.B * R;
-    const int row = blockIdx.y;
-    pdl_wait();
-    if (row >= M) return;
+// Dense p = softmax(z / T) for callers that ask for it (a drafter's own step: its distribution is the next verify step's
+// q).  One CTA per 4,096 entries of a row, four 16-byte loads in flight per thread; the row's statistics are the scan's.
+// It runs beside the draw kernel: that one lets it start after its own wait, i.e. when the scan has completed, and
+// nothing here depends on the draw (so the results of earlier kernels are read past L1, and the wait at the end only keeps
+// this grid from completing before the draw).  What bounds it is HBM, 8 B per entry, where there are many rows; 16 rows of
+// 152,064: 23 us behind the draw with one 4-byte load per thread and iteration.
+constexpr int kProbsThreads = 256, kProbsGroups = 4, kProbsChunk = kProbsThreads * kProbsGroups * 4;
+__global__ void __launch_bounds__(kProbsThreads) probs_kernel(AcceptParams p) {
+    const int M = p.B * (p.gamma + 1), row = blockIdx.y, t = threadIdx.x;
+    pdl_trigger();
     const float inv_T = 1.f / p.T;
-    __shared__ Stat red[256];
-    __shared__ Stat rs;
-    Stat acc{-INFINITY, 0.f, 0x7fffffff};
-    for (int i = threadIdx.x; i < p.n_part; i += blockDim.x) {
-        Stat x{p.part_max[(size_t)i * M + row], p.part_sum[(size_t)i * M + row], p.part_idx[(size_t)i * M + row]};
-        acc = combine(acc, x, inv_T);
+    const int n4 = p.V / 4, i0 = blockIdx.x * (kProbsChunk / 4) + t;            // V is a multiple of 8
+    const float4* z = reinterpret_cast<const float4*>(p.logits + (size_t)row * p.V);
+    float4 x[kProbsGroups];
+#pragma unroll
+    for (int k = 0; k < kProbsGroups; ++k) {
+        const int i = i0 + k * kProbsThreads;
+        x[k] = i < n4 ? __ldcg(z + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] = combine(red[threadIdx.x], red[threadIdx.x + w], inv_T);
+    float m, inv_sum;
+    if (p.row_stats) {
+        const float2 ms = __ldcg(reinterpret_cast<const float2*>(p.row_stats) + row);
+        m = ms.x; inv_sum = 1.f / ms.y;
+    } else {
+        // no room for merged statistics in the caller's scratch: merge the LM head's partial slots
+        __shared__ Stat red[kProbsThreads];
+        Stat acc{-INFINITY, 0.f, 0x7fffffff};
+        for (int i = t; i < p.n_part; i += kProbsThreads) {
+            const size_t at = (size_t)i * M + row;
+            acc = combine(acc, Stat{__ldcg(p.part_max + at), __ldcg(p.part_sum + at), __ldcg(p.part_idx + at)}, inv_T);
+        }
+        red[t] = acc;
         __syncthreads();
+        for (int w = kProbsThreads / 2; w > 0; w >>= 1) {
+            if (t < w) red[t] = combine(red[t], red[t + w], inv_T);
+            __syncthreads();
+        }
+        m = red[0].m; inv_sum = 1.f / red[0].s;
     }
-    if (threadIdx.x == 0) rs = red[0];
-    __syncthreads();
-    const float inv_sum = 1.f / rs.s;
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < p.V; v += gridDim.x * blockDim.x)
-        p.probs_out[(size_t)row * p.V + v] = expf((p.logits[(size_t)row * p.V + v] - rs.m) * inv_T) * inv_sum;
+    float4* out = reinterpret_cast<float4*>(p.probs_out + (size_t)row * p.V);
+#pragma unroll
+    for (int k = 0; k < kProbsGroups; ++k) {
+        const int i = i0 + k * kProbsThreads;
+        if (i < n4)
+            out[i] = make_float4(expf((x[k].x - m) * inv_T) * inv_sum, expf((x[k].y - m) * inv_T) * inv_sum,
+                                 expf((x[k].z - m) * inv_T) * inv_sum, expf((x[k].w - m) * inv_T) * inv_sum);
+    }
+    pdl_wait();
 }
 
 __global__ void kv_commit_kernel(int B, int gamma, const int32_t* accept_len, int32_t* seq_lens, int32_t* dev_status) {
@@ -880,7 +903,7 @@ cudaError_t launch_accept(const AcceptParams& p, cudaStream_t stream) {
         count_launches(1);
         if (p.probs_out) {
             const int M = p.B * (p.gamma + 1);
-            if (launch_pdl(probs_kernel, dim3(16, M), dim3(256), 0, stream, p) != cudaSuccess) return cudaGetLastError();
+            if (launch_pdl(probs_kernel, dim3((p.V + kProbsChunk - 1) / kProbsChunk, M), dim3(kProbsThreads), 0, stream, p) != cudaSuccess) return cudaGetLastError();
             count_launches(1);
         }
     }
