@@ -117,7 +117,9 @@ def _ptr(t, dtype=None):
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    # the handle itself: torch.cuda.current_stream() builds a Stream object around it (3.5 us a call against 0.3 us, three
+    # calls a step, on a step whose launches take 18 us)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def massv_version() -> int:
