@@ -6,6 +6,7 @@
 //                           extra token is drawn from (residual max(p-q,0) after
 //                           a rejection, p itself for the bonus token), as chunk
 //                           masses followed by an inverse-CDF walk in fp64;
+//   accept_row_kernel       T > 0 with few sequences: both of the above in one launch, a cluster of CTAs per sequence;
 //   probs_kernel            optional dense p = softmax(z/T) output;
 //   kv_commit_kernel        advance the committed cache lengths.
 // All reductions run in a fixed order, so results are bit-identical run to run.
@@ -44,62 +45,113 @@ __device__ __forceinline__ Stat combine(Stat a, Stat b, float inv_T) {
     return r;
 }
 
-// One CTA per sequence, one warp per block row.  Each lane merges a strided
-// share of the partial slots (independent loads), a butterfly merges the lanes,
-// and warp 0 then evaluates all gamma accept tests at once (lane j = draft j) and
-// takes the first failure.
+// The step's inputs at the drafted tokens of sequence b, lane j = draft j: they are not results of the kernel before this
+// one, so they are fetched while that kernel drains (two dependent cold reads).
+struct DraftInputs {
+    int x = -1;
+    float u = 0.f, q = 0.f;
+    __device__ __forceinline__ void fetch(const AcceptParams& p, int b, int lane, bool greedy) {
+        if (lane >= p.gamma) return;
+        x = p.draft_tokens[(size_t)b * p.gamma + lane];
+        if (greedy) return;
+        u = p.u_accept[(size_t)b * p.gamma + lane];
+        if (!p.q_at_draft && x >= 0 && x < p.V) q = p.draft_probs[((size_t)b * p.gamma + lane) * p.V + x];
+    }
+};
+
+// Softmax statistics of one block row, by one warp: lanes hold a strided share of the partial slots (independent loads);
+// first the maximum and the lowest index that attains it, then the sums relative to it.  The same value in every lane.
+// (Little code on purpose: it runs once, right after the LM head has streamed a gigabyte of weights through L2, and every
+// line of instructions is fetched from memory.)
+__device__ __forceinline__ Stat merge_partials(const AcceptParams& p, int row, int lane, float inv_T, bool greedy) {
+    const int M = p.B * (p.gamma + 1);
+    Stat acc{-INFINITY, 0.f, 0x7fffffff};
+    for (int i0 = 0; i0 < p.n_part; i0 += 32 * kScanBatch) {
+        Stat x[kScanBatch];
+#pragma unroll
+        for (int k = 0; k < kScanBatch; ++k) {
+            const int i = i0 + k * 32 + lane;
+            x[k] = Stat{-INFINITY, 0.f, 0x7fffffff};
+            if (i < p.n_part) {
+                const size_t at = p.part_per_rank
+                    ? (size_t)(i / p.part_per_rank) * p.rank_stride + (size_t)(i % p.part_per_rank) * M + row
+                    : (size_t)i * M + row;
+                x[k].m = p.part_max[at];
+                if (!greedy) x[k].s = p.part_sum[at];
+                x[k].idx = p.part_idx[at];
+            }
+        }
+        float m = x[0].m;
+#pragma unroll
+        for (int k = 1; k < kScanBatch; ++k) m = fmaxf(m, x[k].m);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        Stat part{m, 0.f, 0x7fffffff};
+#pragma unroll
+        for (int k = 0; k < kScanBatch; ++k) {
+            if (x[k].m == m) part.idx = min(part.idx, x[k].idx);
+            if (!greedy && x[k].m != -INFINITY) part.s += x[k].s * expf((x[k].m - m) * inv_T);
+        }
+        part.idx = __reduce_min_sync(0xffffffffu, part.idx);
+        if (!greedy) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) part.s += __shfl_xor_sync(0xffffffffu, part.s, o);
+        }
+        acc = i0 == 0 ? part : combine(acc, part, inv_T);
+    }
+    return acc;
+}
+
+// The accept tests of sequence b, all at once (lane j = draft j), by one warp: the first rejected draft, or gamma if
+// there is none.  GATHERED: the logits and probabilities at the drafts come from the ranks' exchange buffers.
+template <bool GATHERED>
+__device__ __forceinline__ int first_rejection(const AcceptParams& p, int b, int lane, float inv_T, bool greedy, const Stat* row_stat,
+                                               const DraftInputs& in) {
+    const int R = p.gamma + 1;
+    bool ok = true;
+    if (lane < p.gamma) {
+        if (in.x < 0 || in.x >= p.V) {
+            set_status(p.dev_status, MASSV_ERR_INVALID_ARG);
+            ok = false;
+        } else if (greedy) {
+            ok = (in.x == row_stat[lane].idx);
+        } else {
+            float zx, qx;
+            if (GATHERED && p.z_at_draft) {     // the owner's value is the only one that is not -inf
+                zx = qx = -INFINITY;
+                for (int r = 0; r < p.ranks; ++r) {
+                    zx = fmaxf(zx, p.z_at_draft[r * p.rank_stride + (size_t)b * p.gamma + lane]);
+                    qx = fmaxf(qx, p.q_at_draft[r * p.rank_stride + (size_t)b * p.gamma + lane]);
+                }
+            } else {
+                zx = p.logits[(size_t)(b * R + lane) * p.V + in.x];
+                qx = in.q;
+            }
+            const float px = expf((zx - row_stat[lane].m) * inv_T) / row_stat[lane].s;
+            const float lhs = in.u * qx;
+            ok = lhs < px;
+        }
+    }
+    const unsigned fail = __ballot_sync(0xffffffffu, !ok);
+    return fail ? (__ffs(fail) - 1) : p.gamma;
+}
+
+// One CTA per sequence, one warp per block row; warp 0 then evaluates the accept tests.
 __global__ void __launch_bounds__(kScanThreads) accept_scan_kernel(AcceptParams p) {
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int R = p.gamma + 1, M = p.B * R;
+    const int R = p.gamma + 1;
     const bool greedy = !(p.T > 0.f);
     const float inv_T = greedy ? 1.f : 1.f / p.T;
     __shared__ Stat row_stat[kMaxRows];
     static_assert(kScanThreads / 32 >= kMaxRows, "one warp per block row");
-    // The drafted tokens, their uniforms and the drafter's probabilities at them are inputs of the step, not
-    // results of the kernel before this one: fetch them while that kernel drains (two dependent cold reads).
-    int x_in = -1;
-    float u_in = 0.f, q_in = 0.f;
-    if (warp == 0 && lane < p.gamma) {
-        x_in = p.draft_tokens[(size_t)b * p.gamma + lane];
-        if (!greedy) {
-            u_in = p.u_accept[(size_t)b * p.gamma + lane];
-            if (!p.q_at_draft && x_in >= 0 && x_in < p.V) q_in = p.draft_probs[((size_t)b * p.gamma + lane) * p.V + x_in];
-        }
-    }
+    DraftInputs in;
+    if (warp == 0) in.fetch(p, b, lane, greedy);
     pdl_wait();
     pdl_trigger();
 
     if (warp < R) {
         const int row = b * R + warp;
-        Stat acc{-INFINITY, 0.f, 0x7fffffff};
-        for (int i0 = 0; i0 < p.n_part; i0 += 32 * kScanBatch) {
-            // issue a batch of independent loads before merging them
-            Stat x[kScanBatch];
-#pragma unroll
-            for (int k = 0; k < kScanBatch; ++k) {
-                const int i = i0 + k * 32 + lane;
-                x[k] = Stat{-INFINITY, 0.f, 0x7fffffff};
-                if (i < p.n_part) {
-                    const size_t at = p.part_per_rank
-                        ? (size_t)(i / p.part_per_rank) * p.rank_stride + (size_t)(i % p.part_per_rank) * M + row
-                        : (size_t)i * M + row;
-                    x[k].m = p.part_max[at];
-                    x[k].s = greedy ? 0.f : p.part_sum[at];
-                    x[k].idx = p.part_idx[at];
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < kScanBatch; ++k) acc = combine(acc, x[k], inv_T);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            Stat y;
-            y.m = __shfl_xor_sync(0xffffffffu, acc.m, o);
-            y.s = __shfl_xor_sync(0xffffffffu, acc.s, o);
-            y.idx = __shfl_xor_sync(0xffffffffu, acc.idx, o);
-            // both partners must form the same sum: order the operands by lane
-            acc = (lane & o) ? combine(y, acc, inv_T) : combine(acc, y, inv_T);
-        }
+        const Stat acc = merge_partials(p, row, lane, inv_T, greedy);
         if (lane == 0) {
             row_stat[warp] = acc;
             if (p.row_stats) { p.row_stats[(size_t)row * 2] = acc.m; p.row_stats[(size_t)row * 2 + 1] = acc.s; }
@@ -108,36 +160,9 @@ __global__ void __launch_bounds__(kScanThreads) accept_scan_kernel(AcceptParams 
     __syncthreads();
     if (warp != 0) return;
 
-    bool ok = true;
-    int x = -1;
-    if (lane < p.gamma) {
-        x = x_in;
-        if (x < 0 || x >= p.V) {
-            set_status(p.dev_status, MASSV_ERR_INVALID_ARG);
-            ok = false;
-        } else if (greedy) {
-            ok = (x == row_stat[lane].idx);
-        } else {
-            float zx, qx;
-            if (p.z_at_draft) {                 // the owner's value is the only one that is not -inf
-                zx = qx = -INFINITY;
-                for (int r = 0; r < p.ranks; ++r) {
-                    zx = fmaxf(zx, p.z_at_draft[r * p.rank_stride + (size_t)b * p.gamma + lane]);
-                    qx = fmaxf(qx, p.q_at_draft[r * p.rank_stride + (size_t)b * p.gamma + lane]);
-                }
-            } else {
-                zx = p.logits[(size_t)(b * R + lane) * p.V + x];
-                qx = q_in;
-            }
-            const float px = expf((zx - row_stat[lane].m) * inv_T) / row_stat[lane].s;
-            const float lhs = u_in * qx;
-            ok = lhs < px;
-        }
-    }
-    const unsigned fail = __ballot_sync(0xffffffffu, !ok);
-    const int n = fail ? (__ffs(fail) - 1) : p.gamma;       // first rejected draft, or gamma if none
+    const int n = first_rejection<true>(p, b, lane, inv_T, greedy, row_stat, in);
     int32_t* toks = p.out_tokens + (size_t)b * R;
-    if (lane < R) toks[lane] = lane < n ? x : -1;
+    if (lane < R) toks[lane] = lane < n ? in.x : -1;
     __syncwarp();
     if (lane != 0) return;
     p.accept_len[b] = n + 1;
@@ -679,6 +704,154 @@ __global__ void __launch_bounds__(kResidualThreads, kResidualCtasPerSm) residual
     }
 }
 
+// T > 0 with few sequences: the accept tests and the draw in one launch, a cluster of CTAs per sequence.  Every CTA merges
+// the row statistics and takes the (same) decision; each warp then brings one contiguous segment of the sampled row (and of
+// the drafter's) into shared memory with bulk copies and turns it into masses there, the segments' totals are exchanged
+// once through distributed shared memory, and the warp whose segment holds the target finds the token in its segment.
+// What bounds it is that chain of latencies (statistics, logits at the drafts, the row, one cluster barrier, the pick) and
+// the instructions themselves, which are cold behind a kernel that has streamed a gigabyte through L2: loops stay rolled.
+// The two kernels it replaces add a launch boundary, the arrival counters, and a draw that reads masses back through L2.
+// With gamma = 0 the row is the whole distribution, so probs_out is written here too.
+constexpr int kRowThreads = 512;
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kRowMaxCluster = 8;
+constexpr int kRowMaxBytes = 208 * 1024;             // a CTA's share of the row
+constexpr int kRowPairBytes = 106 * 1024;            // up to here two CTAs share an SM
+
+__global__ void __launch_bounds__(kRowThreads, 2) accept_row_kernel(AcceptParams p, int n_ctas, int warp_groups) {
+    extern __shared__ __align__(128) float4 row_smem[];                   // [warp][warp_groups]: logits, then masses
+    __shared__ __align__(8) uint64_t full_bar[kRowWarps];
+    __shared__ Stat row_stat[kMaxRows];
+    __shared__ double s_pub[kRowWarps];                                   // this CTA's segment totals, read by the cluster
+    __shared__ double s_all[kRowMaxCluster * kRowWarps];
+    __shared__ int s_n, s_pick[2], s_abort;
+    __shared__ double s_base[2];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int rank = blockIdx.x % n_ctas, b = blockIdx.x / n_ctas;
+    const int R = p.gamma + 1;
+    const float inv_T = 1.f / p.T;
+    if (t == 0) {
+        for (int w = 0; w < kRowWarps; ++w) mbar_init(&full_bar[w], 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    DraftInputs in;
+    if (warp == 0) in.fetch(p, b, lane, false);
+    pdl_wait();
+    pdl_trigger();
+
+    // ---- the accept tests
+    if (warp < R) {
+        const int row = b * R + warp;
+        const Stat acc = merge_partials(p, row, lane, inv_T, false);
+        if (lane == 0) {
+            row_stat[warp] = acc;
+            if (p.row_stats && rank == 0) { p.row_stats[(size_t)row * 2] = acc.m; p.row_stats[(size_t)row * 2 + 1] = acc.s; }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const int n = first_rejection<false>(p, b, lane, inv_T, false, row_stat, in);
+        if (lane == 0) s_n = n;
+        if (rank == 0) {
+            // (the extra token's place is left to the draw)
+            if (lane < R && lane != n) p.out_tokens[(size_t)b * R + lane] = lane < n ? in.x : -1;
+            if (lane == 0) p.accept_len[b] = n + 1;
+        }
+    }
+    __syncthreads();
+    const int n = s_n;
+    SeqState st;
+    st.n = n; st.use_q = n < p.gamma ? 1 : 0;
+    st.row_max = row_stat[n].m; st.inv_sum = 1.f / row_stat[n].s;
+    const RowCtx rc(st, inv_T);
+
+    // ---- this warp's segment: groups of four entries g0 .. g0 + count - 1 of the row (V is a multiple of 8)
+    const int n4 = p.V / 4, segment = rank * kRowWarps + warp, n_seg = n_ctas * kRowWarps;
+    const int g0 = min(n4, segment * warp_groups), count = min(n4 - g0, warp_groups);
+    float4* ms = row_smem + (size_t)warp * warp_groups;
+    const float4* q = reinterpret_cast<const float4*>(p.draft_probs + ((size_t)b * p.gamma + n) * p.V) + g0;
+    float4* probs = p.probs_out && p.gamma == 0 ? reinterpret_cast<float4*>(p.probs_out + (size_t)b * p.V) + g0 : nullptr;
+    bool use_q = st.use_q != 0;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (count > 0) {
+            if (lane == 0) {
+                const uint32_t bytes = (uint32_t)count * 16u;
+                mbar_expect_tx(&full_bar[warp], bytes);
+                bulk_load_1d(ms, p.logits + (size_t)(b * R + n) * p.V + 4 * (size_t)g0, bytes, &full_bar[warp]);
+                if (use_q) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(q), "r"(bytes) : "memory");
+            }
+            __syncwarp();
+            if (!mbar_wait_warp(&full_bar[warp], (uint32_t)attempt, &s_abort) && lane == 0) {
+                // report it, and give copies that may still be in flight time to land
+                set_status(p.dev_status, MASSV_ERR_TIMEOUT);
+                for (int i = 0; i < 64; ++i) __nanosleep(2000);
+            }
+            __syncwarp();
+        }
+        double total = 0.0;
+#pragma unroll 2
+        for (int i = lane; i < count; i += 32) {
+            const float4 q4 = use_q ? __ldcs(q + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 z = ms[i];
+            if (probs)
+                probs[i] = make_float4(expf((z.x - st.row_max) * inv_T) * st.inv_sum, expf((z.y - st.row_max) * inv_T) * st.inv_sum,
+                                       expf((z.z - st.row_max) * inv_T) * st.inv_sum, expf((z.w - st.row_max) * inv_T) * st.inv_sum);
+            // (without a residual q4 is zero: max(p - 0, 0) = p)
+            const float4 m = make_float4(fmaxf(rc.prob(z.x) - q4.x, 0.f), fmaxf(rc.prob(z.y) - q4.y, 0.f), fmaxf(rc.prob(z.z) - q4.z, 0.f),
+                                         fmaxf(rc.prob(z.w) - q4.w, 0.f));
+            ms[i] = m;
+            total += ((double)m.x + (double)m.y) + ((double)m.z + (double)m.w);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        if (lane == 0) s_pub[warp] = total;
+        // ---- all segments' totals (segment order is vocabulary order), the segment that holds u * total
+        row_barrier(n_ctas);
+        if (t < n_seg) s_all[t] = __longlong_as_double((long long)peer_load_u64(&s_pub[t % kRowWarps], t / kRowWarps));
+        __syncthreads();
+        if (warp == 0) walk_chunk_masses(s_all, n_seg, (double)p.u_sample[(size_t)b * R + n], s_pick, s_base);
+        row_barrier(n_ctas);               // the pick is visible here, and nobody reads this CTA's totals any more
+        if (s_pick[0] >= 0 || !use_q) break;
+        use_q = false;                     // the residual has no mass (p == q on this row): draw from p
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the masses, ahead of the copy over them
+        __syncthreads();
+    }
+    const int pick = s_pick[0];
+    if (pick < 0) {                        // no mass at all (cannot happen for a softmax row)
+        if (rank == 0 && t == 0) { p.out_tokens[(size_t)b * R + n] = 0; set_status(p.dev_status, MASSV_ERR_INVALID_ARG); }
+    } else if (pick == segment) {
+        // ---- the token: lane l owns a contiguous run of the segment's groups
+        const int per = (count + 31) / 32, i0 = min(count, lane * per), i1 = min(count, i0 + per);
+        double mine = 0.0;
+        for (int i = i0; i < i1; ++i) mine += ((double)ms[i].x + (double)ms[i].y) + ((double)ms[i].z + (double)ms[i].w);
+        double incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const double target = s_base[1];
+        double run = s_base[0] + (incl - mine);
+        int first = 0x7fffffff, last = -1;
+        const float* m = reinterpret_cast<const float*>(ms);
+        for (int i = 4 * i0; i < 4 * i1; ++i) {
+            const float v = m[i];
+            run += (double)v;
+            if (v > 0.f) {
+                last = i;
+                if (first == 0x7fffffff && run > target) first = i;
+            }
+        }
+        first = __reduce_min_sync(0xffffffffu, first);
+        last = __reduce_max_sync(0xffffffffu, last);
+        if (lane == 0) {
+            const int tok = 4 * g0 + (s_pick[1] == 0 && first != 0x7fffffff ? first : last);
+            if (MASSV_IN_BOUNDS(tok, p.V, p.dev_status)) p.out_tokens[(size_t)b * R + n] = tok;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- vocabulary shards
 // The same arithmetic with the vocabulary cut into contiguous shards, one per rank: a shard sees Vs
 // columns of the logits and of q.  Chunks are counted inside the shard; ranks in order are vocabulary order.
@@ -829,13 +1002,14 @@ __global__ void shard_publish_kernel(PublishParams p) {
 
 // Dense p = softmax(z / T) for callers that ask for it (a drafter's own step: its distribution is the next verify step's
 // q).  One CTA per 4,096 entries of a row, four 16-byte loads in flight per thread; the row's statistics are the scan's.
-// It runs beside the draw kernel: that one lets it start after its own wait, i.e. when the scan has completed, and
+// It runs beside the persistent draw kernel: that one lets it start after its own wait, i.e. when the scan has completed, and
 // nothing here depends on the draw (so the results of earlier kernels are read past L1, and the wait at the end only keeps
-// this grid from completing before the draw).  What bounds it is HBM, 8 B per entry, where there are many rows; 16 rows of
+// this grid from completing before the draw).  Behind accept_row_kernel, which makes the statistics itself, it waits first.  What bounds it is HBM, 8 B per entry, where there are many rows; 16 rows of
 // 152,064: 23 us behind the draw with one 4-byte load per thread and iteration.
 constexpr int kProbsThreads = 256, kProbsGroups = 4, kProbsChunk = kProbsThreads * kProbsGroups * 4;
-__global__ void __launch_bounds__(kProbsThreads) probs_kernel(AcceptParams p) {
+__global__ void __launch_bounds__(kProbsThreads) probs_kernel(AcceptParams p, int wait_first) {
     const int M = p.B * (p.gamma + 1), row = blockIdx.y, t = threadIdx.x;
+    if (wait_first) pdl_wait();
     pdl_trigger();
     const float inv_T = 1.f / p.T;
     const int n4 = p.V / 4, i0 = blockIdx.x * (kProbsChunk / 4) + t;            // V is a multiple of 8
@@ -874,7 +1048,7 @@ __global__ void __launch_bounds__(kProbsThreads) probs_kernel(AcceptParams p) {
             out[i] = make_float4(expf((x[k].x - m) * inv_T) * inv_sum, expf((x[k].y - m) * inv_T) * inv_sum,
                                  expf((x[k].z - m) * inv_T) * inv_sum, expf((x[k].w - m) * inv_T) * inv_sum);
     }
-    pdl_wait();
+    if (!wait_first) pdl_wait();
 }
 
 __global__ void kv_commit_kernel(int B, int gamma, const int32_t* accept_len, int32_t* seq_lens, int32_t* dev_status) {
@@ -888,11 +1062,43 @@ __global__ void kv_commit_kernel(int B, int gamma, const int32_t* accept_len, in
 
 }  // namespace
 
+// CTAs per sequence of accept_row_kernel, 0 where it does not apply.  All clusters have to be resident at once: a second wave
+// would repeat the whole latency chain, where the persistent draw kernel overlaps its sequences.
+static int row_cluster(const AcceptParams& p) {
+    for (int c = kRowMaxCluster; c >= 1; c /= 2) {
+        if (c > 1 && p.V < c * 2048) continue;
+        const long bytes = ((long)(p.V + c - 1) / c + 256) * 4;
+        if (bytes > kRowMaxBytes) break;
+        const long slots = bytes <= kRowPairBytes ? 224 : 96;
+        if ((long)p.B * c <= slots) return c;
+    }
+    return 0;
+}
+
 cudaError_t launch_accept(const AcceptParams& p, cudaStream_t stream) {
+    const TimingHooks& hooks = timing_hooks();
+    const int c = p.T > 0.f ? row_cluster(p) : 0;
+    if (c > 0) {
+        const int segments = c * kRowWarps, warp_groups = (p.V / 4 + segments - 1) / segments;
+        if (hooks.residual_start && cudaEventRecord(hooks.residual_start, stream) != cudaSuccess) return cudaGetLastError();
+        const size_t smem = (size_t)kRowWarps * warp_groups * 16;
+        cudaError_t e = cudaFuncSetAttribute(accept_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowMaxBytes + 4096);
+        const dim3 grid((unsigned)(p.B * c));
+        if (e == cudaSuccess)
+            e = c == 1 ? launch_pdl(accept_row_kernel, grid, dim3(kRowThreads), smem, stream, p, c, warp_groups)
+                       : launch_pdl_cluster(accept_row_kernel, grid, dim3(kRowThreads), smem, stream, c, p, c, warp_groups);
+        if (e != cudaSuccess) return e;
+        if (hooks.residual_stop && cudaEventRecord(hooks.residual_stop, stream) != cudaSuccess) return cudaGetLastError();
+        count_launches(1);
+        if (p.probs_out && p.gamma > 0) {
+            if (launch_pdl(probs_kernel, dim3((p.V + kProbsChunk - 1) / kProbsChunk, p.B * (p.gamma + 1)), dim3(kProbsThreads), 0, stream, p, 1) != cudaSuccess) return cudaGetLastError();
+            count_launches(1);
+        }
+        return cudaGetLastError();
+    }
     if (launch_pdl(accept_scan_kernel, dim3(p.B), dim3(kScanThreads), 0, stream, p) != cudaSuccess) return cudaGetLastError();
     count_launches(1);
     if (p.T > 0.f) {
-        const TimingHooks& hooks = timing_hooks();
         if (hooks.residual_start && cudaEventRecord(hooks.residual_start, stream) != cudaSuccess) return cudaGetLastError();
         const size_t ring = (size_t)kResidualStages * 2 * kResidualChunk * sizeof(float);
         if (cudaFuncSetAttribute(residual_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring) != cudaSuccess) return cudaGetLastError();
@@ -902,8 +1108,7 @@ cudaError_t launch_accept(const AcceptParams& p, cudaStream_t stream) {
         if (hooks.residual_stop && cudaEventRecord(hooks.residual_stop, stream) != cudaSuccess) return cudaGetLastError();
         count_launches(1);
         if (p.probs_out) {
-            const int M = p.B * (p.gamma + 1);
-            if (launch_pdl(probs_kernel, dim3((p.V + kProbsChunk - 1) / kProbsChunk, M), dim3(kProbsThreads), 0, stream, p) != cudaSuccess) return cudaGetLastError();
+            if (launch_pdl(probs_kernel, dim3((p.V + kProbsChunk - 1) / kProbsChunk, p.B * (p.gamma + 1)), dim3(kProbsThreads), 0, stream, p, 0) != cudaSuccess) return cudaGetLastError();
             count_launches(1);
         }
     }
