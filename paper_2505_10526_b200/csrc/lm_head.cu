@@ -39,7 +39,6 @@ constexpr int kPairMinTile = 64;            // token rows per tile from which CT
 struct UmmaParams {
     int M, K, V;
     int n_tile;          // token rows per MMA (multiple of 16, <= 256)
-    int n_token_tiles;   // 1 or 2
     int n_groups;        // vocab bands
     int tiles_per_group; // whole 128-row tiles per band
     int stages;
@@ -273,15 +272,12 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
     const int num_kb = p.K / kBlockK;
     const uint32_t pair_rank = PAIR ? cluster_cta_rank() : 0u;
 
-    // which band of vocabulary rows and which token tile this CTA (or pair) owns
-    const int unit = PAIR ? blockIdx.x / 2 : blockIdx.x;
-    const int group = unit / p.n_token_tiles;
-    const int token_tile = unit % p.n_token_tiles;
+    // which band of vocabulary rows this CTA (or pair) owns
+    const int group = PAIR ? blockIdx.x / 2 : blockIdx.x;
     constexpr int tile_rows = PAIR ? 2 * kVocabTile : kVocabTile;       // rows per (super-)tile of the band
     const int row_begin = min(p.V, group * p.tiles_per_group * tile_rows);
     const int row_end = min(p.V, row_begin + p.tiles_per_group * tile_rows);
     const int n_tiles = (row_end - row_begin + tile_rows - 1) / tile_rows;
-    const int tok_base = token_tile * p.n_tile;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -359,7 +355,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                         const uint32_t bar = cluster_addr(&full_bar[s], 0);
                         if (pair_rank == 0) mbar_expect_tx_at(bar, (uint32_t)(2 * kTileBytesW + p.n_tile * 128));
                         tma_load_2d_pair(w_dst, &map_w128, kb * kBlockK, v0, bar, pol_stream);
-                        tma_load_2d_pair(h_dst, &map_h, kb * kBlockK, tok_base + (int)pair_rank * h_rows, bar, pol_keep);
+                        tma_load_2d_pair(h_dst, &map_h, kb * kBlockK, (int)pair_rank * h_rows, bar, pol_keep);
                         w_dst += stage_bytes;
                         if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
                         continue;
@@ -375,7 +371,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                         if (rows & 16) { tma_load_2d(w_dst + r * 128, &map_w16, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 16; }
                         if (rows & 8) { tma_load_2d(w_dst + r * 128, &map_w8, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 8; }
                     }
-                    tma_load_2d(h_dst, &map_h, kb * kBlockK, tok_base, &full_bar[s], pol_keep);
+                    tma_load_2d(h_dst, &map_h, kb * kBlockK, 0, &full_bar[s], pol_keep);
                     w_dst += stage_bytes;
                     if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
                 }
@@ -456,14 +452,14 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
             for (int c = half; c < n_chunks32; c += 2) {
                 const int col = c * 32 + lane;
                 Stat running{run_m[quarter][col], run_s[quarter][col], run_i[quarter][col]};
-                drain_chunk<32>(p, taddr + c * 32, lane, row_in_tile, tile, tok_base + c * 32, running);
+                drain_chunk<32>(p, taddr + c * 32, lane, row_in_tile, tile, c * 32, running);
                 run_m[quarter][col] = running.m; run_s[quarter][col] = running.s; run_i[quarter][col] = running.idx;
             }
             if (tail16 && (n_chunks32 & 1) == half) {
                 // lanes 2c and 2c+1 both end up with column c of the 16-column tail; the even lane keeps it
                 const int col = n_chunks32 * 32 + (lane >> 1);
                 Stat running{run_m[quarter][col], run_s[quarter][col], run_i[quarter][col]};
-                drain_chunk<16>(p, taddr + n_chunks32 * 32, lane, row_in_tile, tile, tok_base + n_chunks32 * 32, running);
+                drain_chunk<16>(p, taddr + n_chunks32 * 32, lane, row_in_tile, tile, n_chunks32 * 32, running);
                 __syncwarp();
                 if ((lane & 1) == 0) { run_m[quarter][col] = running.m; run_s[quarter][col] = running.s; run_i[quarter][col] = running.idx; }
                 __syncwarp();
@@ -481,7 +477,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
     __syncthreads();
     // the CTA's statistics: merge the four lane quarters (ascending rows) into one partial slot
     for (int c = threadIdx.x; c < p.n_tile; c += kThreads) {
-        const int tok = tok_base + c;
+        const int tok = c;
         if (tok < p.M) {
             Stat acc{run_m[0][c], run_s[0][c], run_i[0][c]};
 #pragma unroll
@@ -664,19 +660,25 @@ __device__ __forceinline__ void stats_job64(const UmmaParams& p, uint32_t (&va)[
     }
 }
 
-// ---- One pass over the weights for 257 .. 384 token rows (CTA pairs only).
-// The token rows are cut into two sub-tiles of n_tile <= 192 rows whose accumulators live in tensor memory
-// at the same time (columns 0.. and 192..), so every weight block crosses from L2 into shared memory once
-// and feeds two MMAs (the two-token-tile arrangement of lm_head_umma_kernel streams the weights twice and
-// is bound by that traffic).  Tensor memory has no room for a second pair of accumulators; instead the
-// twelve epilogue warps copy a finished sub-tile into registers (64 columns each) and hand its tensor
+// ---- One pass over the weights for 257 .. 512 token rows (CTA pairs only).
+// The token rows are cut into two sub-tiles of n_tile rows whose accumulators live in tensor memory
+// at the same time, so every weight block crosses from L2 into shared memory once and feeds two MMAs
+// (two token tiles on separate CTA pairs stream the weights twice and are bound by that traffic).
+// Tensor memory has no room for a second pair of accumulators; instead the epilogue warps - PARTS per
+// lane quarter, 64 columns of a sub-tile each - copy a finished sub-tile into registers and hand its tensor
 // memory back before they start on its statistics, which then run from registers while the next tile's
 // MMAs are under way; the second sub-tile follows the same way.
-constexpr int kDuoEpilogueWarps = 12;      // three per TMEM lane quarter
-constexpr int kDuoThreads = (2 + kDuoEpilogueWarps) * 32;
-constexpr int kDuoSubCols = 192;           // tensor-memory columns reserved per sub-tile
-__global__ void __launch_bounds__(kDuoThreads, 1)
+// PARTS = 3: sub-tiles of up to 192 rows (257 .. 384 in all); PARTS = 4: up to 256, all 512 columns.
+template <int PARTS>
+struct DuoCfg {
+    static constexpr int kEpilogueWarps = 4 * PARTS;
+    static constexpr int kThreads = (2 + kEpilogueWarps) * 32;
+    static constexpr int kSubCols = 64 * PARTS;       // tensor-memory columns reserved per sub-tile
+};
+template <int PARTS>
+__global__ void __launch_bounds__(DuoCfg<PARTS>::kThreads, 1)
 lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_constant__ CUtensorMap map_h, const UmmaParams p) {
+    using Cfg = DuoCfg<PARTS>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages];
     __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
@@ -684,9 +686,9 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
     __shared__ __align__(8) uint64_t tmem_empty_bar[2];      // one per sub-tile's accumulator
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
-    __shared__ float run_m[4][2 * kDuoSubCols];
-    __shared__ float run_s[4][2 * kDuoSubCols];
-    __shared__ int run_i[4][2 * kDuoSubCols];
+    __shared__ float run_m[4][2 * Cfg::kSubCols];
+    __shared__ float run_s[4][2 * Cfg::kSubCols];
+    __shared__ int run_i[4][2 * Cfg::kSubCols];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -699,7 +701,8 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
     const int group = blockIdx.x / 2;
     constexpr int tile_rows = 2 * kVocabTile;
     // This pair's tiles: tiles_per_group whole bands (fewer at the end of the vocabulary), then, where the bands
-    // do not divide evenly, one sub-tile of a left-over band (the pair g ^ 1 takes the other sub-tile).
+    // do not divide evenly, one sub-tile of a left-over band (the pair g ^ 1 takes the other sub-tile).  With few
+    // bands every pair takes one sub-tile only (tiles_per_group = 0), and the two pairs of a band share its slot.
     const int n_full = max(0, min(p.tiles_per_group, p.n_bands - group * p.tiles_per_group));
     const int n_tiles = n_full + (group < 2 * p.split_rem ? 1 : 0);
     auto band_of = [&](int t) { return t < n_full ? group * p.tiles_per_group + t : (int)(gridDim.x / 2) * p.tiles_per_group + group / 2; };
@@ -708,7 +711,7 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&tmem_full_bar, 1);
-        for (int q = 0; q < 2; ++q) mbar_init(&tmem_empty_bar[q], 2 * kDuoEpilogueWarps);     // the leader's collect both CTAs' epilogue warps
+        for (int q = 0; q < 2; ++q) mbar_init(&tmem_empty_bar[q], 2 * Cfg::kEpilogueWarps);     // the leader's collect both CTAs' epilogue warps
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -780,7 +783,7 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
                             tc_fence_after();
                         }
                         if (!((subs >> q) & 1)) continue;
-                        const uint32_t d_tmem = tmem_base + (uint32_t)(q * kDuoSubCols);
+                        const uint32_t d_tmem = tmem_base + (uint32_t)(q * Cfg::kSubCols);
                         const uint32_t b_lo = a_lo + (kTileBytesW >> 4) + (uint32_t)q * h_step;
                         if (kb == 0) umma_bf16_pair<false>(d_tmem, a_lo, b_lo, idesc);
                         else umma_bf16_pair<true>(d_tmem, a_lo, b_lo, idesc);
@@ -798,15 +801,15 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
         }
     } else {
         // ------------------------------------------------ epilogue (warps 2..13)
-        // TMEM lanes 32*quarter .. +31 are the only ones warp (quarter = warp % 4) may read; the three warps
+        // TMEM lanes 32*quarter .. +31 are the only ones warp (quarter = warp % 4) may read; the PARTS warps
         // of a quarter take columns 64*part .. 64*part+63 of both sub-tiles.
         const int quarter = warp & 3;
         const int part = (warp - 2) >> 2;
         const int c0 = part * 64;                              // first column (token row within the sub-tile)
-        for (int c = threadIdx.x - 64; c < 4 * 2 * kDuoSubCols; c += kDuoEpilogueWarps * 32) {
+        for (int c = threadIdx.x - 64; c < 4 * 2 * Cfg::kSubCols; c += Cfg::kEpilogueWarps * 32) {
             (&run_m[0][0])[c] = -INFINITY; (&run_s[0][0])[c] = 0.f; (&run_i[0][0])[c] = 0x7fffffff;
         }
-        asm volatile("bar.sync 1, %0;" ::"r"(kDuoEpilogueWarps * 32) : "memory");     // epilogue warps only
+        asm volatile("bar.sync 1, %0;" ::"r"(Cfg::kEpilogueWarps * 32) : "memory");     // epilogue warps only
         bool ok = true;
         for (int t = 0; t < n_tiles && ok; ++t) {
             if (!mbar_wait_warp(&tmem_full_bar, (uint32_t)t & 1u, abort_ptr)) { ok = false; break; }
@@ -822,8 +825,8 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
                 uint32_t va[32], vb[32];
                 const bool live = (subs >> q) & 1;             // a half-tile computes one sub-tile only
                 if (live) {
-                    tmem_load_16x64(taddr + q * kDuoSubCols, va);                              // rows 0-15 of the quarter
-                    tmem_load_16x64(taddr + q * kDuoSubCols + (16u << 16), vb);                // rows 16-31
+                    tmem_load_16x64(taddr + q * Cfg::kSubCols, va);                              // rows 0-15 of the quarter
+                    tmem_load_16x64(taddr + q * Cfg::kSubCols + (16u << 16), vb);                // rows 16-31
                     tmem_wait_ld<32>(va);
                     tmem_wait_ld<32>(vb);
                 }
@@ -833,7 +836,7 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
                 if (!live) continue;
                 const int n_cols = min(64, sub - c0);
                 if (n_cols > 0) {                               // the same in every lane
-                    const int col = q * kDuoSubCols + c0;
+                    const int col = q * Cfg::kSubCols + c0;
                     stats_job64(p, va, vb, lane, quarter, tile, q * sub + c0, n_cols, &run_m[quarter][col], &run_s[quarter][col], &run_i[quarter][col]);
                 }
             }
@@ -843,14 +846,14 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
     tc_fence_before();
     __syncthreads();
     // the CTA's statistics: merge the four lane quarters (ascending rows) into one partial slot
-    for (int i = threadIdx.x; i < 2 * sub; i += kDuoThreads) {
-        const int c = (i / sub) * kDuoSubCols + i % sub, tok = i;
-        if (tok < p.M) {
+    for (int i = threadIdx.x; i < 2 * sub; i += Cfg::kThreads) {
+        const int c = (i / sub) * Cfg::kSubCols + i % sub, tok = i;
+        if (tok < p.M && (p.tiles_per_group > 0 || i / sub == (group & 1))) {
             Stat acc{run_m[0][c], run_s[0][c], run_i[0][c]};
 #pragma unroll
             for (int qd = 1; qd < 4; ++qd)
                 acc = stat_combine(acc, Stat{run_m[qd][c], run_s[qd][c], run_i[qd][c]}, p.scale_log2, p.greedy != 0);
-            const size_t slot = (size_t)(group * 2 + (int)pair_rank) * p.M;
+            const size_t slot = (size_t)((p.tiles_per_group > 0 ? group : group / 2) * 2 + (int)pair_rank) * p.M;
             if (MASSV_IN_BOUNDS(slot + tok, (size_t)p.n_part * p.M, p.dev_status)) {
                 p.part_max[slot + tok] = acc.m;
                 p.part_sum[slot + tok] = p.greedy ? 0.f : acc.s;
@@ -886,22 +889,33 @@ int lm_head_num_partials(int M, int V) {
     return slots < kMaxCtas ? slots : kMaxCtas;
 }
 
-// 257 .. 384 token rows: two sub-tiles, one pass over the weights (lm_head_duo_kernel).
+// 257 .. 512 token rows: two sub-tiles, one pass over the weights (lm_head_duo_kernel).
+template <int PARTS>
 static cudaError_t launch_lm_head_duo(const LmHeadParams& q, UmmaParams p, int ctas, cudaStream_t stream, int* n_part_used) {
-    p.n_token_tiles = 1;
-    p.n_tile = ((q.M + 1) / 2 + 15) / 16 * 16;        // rows per sub-tile, <= 192
+    using Cfg = DuoCfg<PARTS>;
+    p.n_tile = ((q.M + 1) / 2 + 15) / 16 * 16;        // rows per sub-tile, <= Cfg::kSubCols
     const int bands = (q.V + 2 * kVocabTile - 1) / (2 * kVocabTile);
     int groups = ctas / 2;
-    if (groups > bands) groups = bands;
-    // Whole bands per pair; a few left-over bands are cut into their two sub-tiles and dealt to the first pairs
-    // (594 bands on 74 pairs: 8 each, and 4 pairs take half a band more - not 9 each on 66 pairs).
     p.n_bands = bands;
-    p.tiles_per_group = bands / groups;
-    p.split_rem = bands - p.tiles_per_group * groups;
-    if (2 * p.split_rem > groups) {
-        p.tiles_per_group = (bands + groups - 1) / groups;
-        groups = (bands + p.tiles_per_group - 1) / p.tiles_per_group;
-        p.split_rem = 0;
+    int slots;
+    if (2 * bands <= groups) {
+        // so few bands that a pair per band leaves half of the chip idle: a pair per sub-tile of a band
+        groups = 2 * bands;
+        p.tiles_per_group = 0;
+        p.split_rem = bands;
+        slots = groups;
+    } else {
+        if (groups > bands) groups = bands;
+        // Whole bands per pair; a few left-over bands are cut into their two sub-tiles and dealt to the first pairs
+        // (594 bands on 74 pairs: 8 each, and 4 pairs take half a band more - not 9 each on 66 pairs).
+        p.tiles_per_group = bands / groups;
+        p.split_rem = bands - p.tiles_per_group * groups;
+        if (2 * p.split_rem > groups) {
+            p.tiles_per_group = (bands + groups - 1) / groups;
+            groups = (bands + p.tiles_per_group - 1) / p.tiles_per_group;
+            p.split_rem = 0;
+        }
+        slots = groups * 2;
     }
     p.n_groups = groups;
     const int h_rows = p.n_tile / 2;
@@ -909,8 +923,7 @@ static cudaError_t launch_lm_head_duo(const LmHeadParams& q, UmmaParams p, int c
     int stages = kRingBytes / stage_bytes;
     if (stages > kMaxStages) stages = kMaxStages;
     p.stages = stages;
-    p.tmem_cols = 512;                                 // two accumulators at columns 0 and 192
-    const int slots = groups * 2;
+    p.tmem_cols = 512;                                 // two accumulators at columns 0 and kSubCols
     if (slots > q.n_part) return cudaErrorInvalidValue;
     *n_part_used = slots;
     CUtensorMap map_w, map_h;
@@ -919,9 +932,9 @@ static cudaError_t launch_lm_head_duo(const LmHeadParams& q, UmmaParams p, int c
     const size_t smem = (size_t)stages * stage_bytes + 1024;
     const TimingHooks& hooks = timing_hooks();
     if (hooks.lm_head_start && cudaEventRecord(hooks.lm_head_start, stream) != cudaSuccess) return cudaGetLastError();
-    cudaError_t e = cudaFuncSetAttribute(lm_head_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(lm_head_duo_kernel<PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = launch_pdl_cluster(lm_head_duo_kernel, dim3(groups * 2), dim3(kDuoThreads), smem, stream, 2, map_w, map_h, p);
+    e = launch_pdl_cluster(lm_head_duo_kernel<PARTS>, dim3(groups * 2), dim3(Cfg::kThreads), smem, stream, 2, map_w, map_h, p);
     if (e != cudaSuccess) return e;
     if (hooks.lm_head_stop && cudaEventRecord(hooks.lm_head_stop, stream) != cudaSuccess) return cudaGetLastError();
     count_launches(1);
@@ -940,10 +953,10 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     p.dev_status = q.dev_status;
     p.idx_offset = q.idx_offset;
     p.test_skip_stage = q.test_skip_stage;
-    if (q.M > 256 && q.M <= 2 * kDuoSubCols) return launch_lm_head_duo(q, p, ctas, stream, n_part_used);
-    p.n_token_tiles = q.M > 256 ? 2 : 1;
-    const int per_tile = (q.M + p.n_token_tiles - 1) / p.n_token_tiles;
-    p.n_tile = (per_tile + 15) / 16 * 16;
+    if (q.M > 2 * DuoCfg<4>::kSubCols) return cudaErrorInvalidValue;
+    if (q.M > 2 * DuoCfg<3>::kSubCols) return launch_lm_head_duo<4>(q, p, ctas, stream, n_part_used);
+    if (q.M > 256) return launch_lm_head_duo<3>(q, p, ctas, stream, n_part_used);
+    p.n_tile = (q.M + 15) / 16 * 16;
     // From 64 token rows up, pairs of CTAs (cta_group::2) share the hidden-state tile: the traffic
     // from L2 into shared memory per weight byte drops from 1 + N/128 to 1 + N/256.
     const bool pair = p.n_tile >= kPairMinTile;
@@ -951,7 +964,7 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     // Whole tiles per CTA (pair): a band with a short tail tile would run a full K loop with almost
     // nothing in flight.  Use the fewest CTAs that still reach the minimal tiles-per-CTA count
     // (1188 tiles on 148 SMs: 132 CTAs x 9 tiles).
-    int groups = ctas / (p.n_token_tiles * (pair ? 2 : 1));
+    int groups = ctas / (pair ? 2 : 1);
     const int bands = (q.V + band_rows - 1) / band_rows;
     if (groups > bands) groups = bands;
     p.tiles_per_group = (bands + groups - 1) / groups;
@@ -987,12 +1000,12 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     if (pair) {
         e = cudaFuncSetAttribute(lm_head_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * p.n_token_tiles * 2), dim3(kThreads), smem, stream, 2,
+        e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * 2), dim3(kThreads), smem, stream, 2,
                                map_w[0], map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
     } else {
         e = cudaFuncSetAttribute(lm_head_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups * p.n_token_tiles), dim3(kThreads), smem, stream, map_w[0],
+        e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups), dim3(kThreads), smem, stream, map_w[0],
                        map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
     }
     if (e != cudaSuccess) return e;

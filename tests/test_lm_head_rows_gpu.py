@@ -1,0 +1,39 @@
+"""The LM head with more than 256 rows (two sub-tiles over one pass of the weights) at the edges of its sub-tiles and of the way
+it deals the vocabulary out: one band, bands that take a pair per sub-tile and the first count that does not, left-over bands,
+ragged ends; logits against 64 bits, greedy tokens against the logits' own argmax, probabilities from the merged statistics."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch,gamma", [(257, 0), (68, 3), (64, 5), (77, 4), (100, 3), (73, 6), (64, 7)])
+@pytest.mark.parametrize("vocab", [8, 264, 9472, 9480, 18944, 19208, 40008])
+def test_rows(batch, gamma, vocab):
+    import paper_2505_10526_b200 as mv
+    K, R = 192, gamma + 1
+    g = torch.Generator(device="cuda").manual_seed(batch * 7 + vocab)
+    hidden = (5.0 * torch.randn((batch, R, K), generator=g, device="cuda")).to(torch.bfloat16)
+    w = (0.05 * torch.randn((vocab, K), generator=g, device="cuda")).to(torch.bfloat16)
+    exact = torch.matmul(hidden.view(-1, K).double(), w.double().t()).view(batch, R, vocab)
+    drafts = exact[:, :gamma].argmax(-1).to(torch.int32).contiguous()          # every draft is right: the extra token is row gamma's
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    tokens = torch.empty((batch, R), dtype=torch.int32, device="cuda"); lens = torch.empty((batch,), dtype=torch.int32, device="cuda")
+    for T in (0.0, 1.0):
+        logits = torch.full((batch, R, vocab), float("nan"), device="cuda")
+        probs = torch.full((batch, R, vocab), float("nan"), device="cuda") if T > 0 else None
+        q = torch.full((batch, gamma, vocab), 1e-9, device="cuda")
+        desc = mv.accept_desc(batch, gamma, K, vocab, T)
+        ws = mv.alloc_workspace(mv.massv_accept_workspace_size(desc), "cuda").fill_(0xff)
+        mv.massv_accept(desc, hidden, w, drafts, q if T > 0 else None, torch.full((batch, gamma), 0.5, device="cuda") if T > 0 else None,
+                        torch.full((batch, R), 0.5, device="cuda") if T > 0 else None, tokens, lens, logits, probs, ws, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        # fp32 sums of 192 products of size about 0.25: 1e-5
+        assert float((logits.double() - exact).abs().max()) < 1e-4
+        assert lens.tolist() == [R] * batch
+        if T == 0:
+            assert torch.equal(tokens[:, gamma].long(), logits[:, gamma].argmax(-1))
+            assert torch.equal(tokens[:, :gamma], logits[:, :gamma].argmax(-1).to(torch.int32))
+        else:
+            assert float((probs.double() - torch.softmax(exact, -1)).abs().max()) < 1e-4
