@@ -10,7 +10,7 @@
 // streamed exactly once: each persistent CTA owns a contiguous band of whole
 // 128-row vocabulary tiles and walks K in 64-element blocks through a TMA ->
 // shared memory ring.  Warp roles: warp 0 issues TMA loads, warp 1 issues MMAs and owns
-// the TMEM allocation, warps 2-9 drain finished accumulators (double buffered)
+// the TMEM allocation, the others drain finished accumulators (double buffered)
 // with tcgen05.ld, store fp32 logits when they are needed, and keep running
 // (max, sum exp((z-max)/T), argmax) per token row in shared memory (warp-wide
 // integer max reduction on order-preserving keys, ballot for the argmax, a
@@ -26,8 +26,10 @@ namespace massv {
 
 namespace {
 
-constexpr int kEpilogueWarps = 8;          // two per TMEM lane quarter
-constexpr int kThreads = (2 + kEpilogueWarps) * 32;
+// Epilogue warps: two per TMEM lane quarter for single-CTA tiles (16 columns at a time), four for CTA pairs (64 columns each,
+// so that the epilogue of a 256-row tile keeps up with short K loops too).
+__host__ __device__ constexpr int epilogue_warps(bool pair) { return pair ? 16 : 8; }
+__host__ __device__ constexpr int lm_head_threads(bool pair) { return (2 + epilogue_warps(pair)) * 32; }
 constexpr int kBlockK = 64;                 // bf16 elements per 128-byte swizzled row
 constexpr int kTileBytesW = kVocabTile * kBlockK * 2;
 constexpr int kMaxStages = 12;
@@ -42,7 +44,7 @@ struct UmmaParams {
     int n_groups;        // vocab bands
     int tiles_per_group; // whole 128-row tiles per band
     int stages;
-    int tmem_cols;       // power of two >= 2 * n_tile
+    int tmem_cols;       // power of two; two accumulators, half each
     int greedy;
     float scale_log2;    // log2(e) / T
     float* logits;       // [M, V] or nullptr
@@ -107,18 +109,6 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 
 template <int C>
 __device__ __forceinline__ void tmem_load(uint32_t taddr, uint32_t (&r)[C]);
-template <>
-__device__ __forceinline__ void tmem_load<32>(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-}
 template <>
 __device__ __forceinline__ void tmem_load<16>(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
@@ -243,264 +233,6 @@ __device__ __forceinline__ void drain_chunk(const UmmaParams& p, uint32_t taddr,
         mine.s = sums[0];
     }
     running = stat_combine(running, mine, p.scale_log2, greedy);
-}
-
-// PAIR: the grid is made of 2-CTA clusters; a pair works on 256-row vocabulary super-tiles (CTA rank r
-// owns rows 128 r .. 128 r + 127 and half of the token rows of the hidden-state tile), which halves the
-// hidden-state traffic per weight byte compared with one CTA per 128 rows.
-template <bool PAIR>
-__global__ void __launch_bounds__(kThreads, 1)
-lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_constant__ CUtensorMap map_w64,
-                    const __grid_constant__ CUtensorMap map_w32, const __grid_constant__ CUtensorMap map_w16,
-                    const __grid_constant__ CUtensorMap map_w8, const __grid_constant__ CUtensorMap map_h,
-                    const UmmaParams p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[kMaxStages];
-    __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
-    __shared__ __align__(8) uint64_t tmem_full_bar[2];
-    __shared__ __align__(8) uint64_t tmem_empty_bar[2];
-    __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
-    __shared__ float run_m[4][256];
-    __shared__ float run_s[4][256];
-    __shared__ int run_i[4][256];
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int h_rows = PAIR ? p.n_tile / 2 : p.n_tile;       // hidden-state rows this CTA loads per K block
-    const int stage_bytes = kTileBytesW + h_rows * 128;
-    const int num_kb = p.K / kBlockK;
-    const uint32_t pair_rank = PAIR ? cluster_cta_rank() : 0u;
-
-    // which band of vocabulary rows this CTA (or pair) owns
-    const int group = PAIR ? blockIdx.x / 2 : blockIdx.x;
-    constexpr int tile_rows = PAIR ? 2 * kVocabTile : kVocabTile;       // rows per (super-)tile of the band
-    const int row_begin = min(p.V, group * p.tiles_per_group * tile_rows);
-    const int row_end = min(p.V, row_begin + p.tiles_per_group * tile_rows);
-    const int n_tiles = (row_end - row_begin + tile_rows - 1) / tile_rows;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        // in a pair the leader's tmem_empty barriers collect both CTAs' epilogue warps
-        for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full_bar[b], 1); mbar_init(&tmem_empty_bar[b], (PAIR ? 2 : 1) * kEpilogueWarps); }
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    if (warp == 1) {
-        __syncwarp();
-        if constexpr (PAIR) {
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                         "r"((uint32_t)p.tmem_cols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                         "r"((uint32_t)p.tmem_cols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if constexpr (PAIR) cluster_sync_all();      // the peer's barriers exist before anything signals them
-    tc_fence_after();
-    const uint32_t tmem_base = tmem_base_slot;
-    volatile int* abort_ptr = &abort_flag;
-    // The weights do not depend on the kernel before this one: while it drains, an epilogue warp (idle
-    // until the first accumulator is ready) asks L2 for the first boxes of this CTA's first tile.
-    // Single-CTA tiles only: with CTA pairs the hints cost more than they bring.  Depth by measurement:
-    // the step gains up to 32 boxes (-2.4 %), beyond 40 the hinted boxes are fetched twice too often.
-    if constexpr (!PAIR) {
-        if (warp == 2 && lane == 0 && n_tiles > 0) {
-            const int n_pf = min(num_kb, kPrefetchBlocks);
-            for (int kb = 0; kb < n_pf; ++kb) tma_prefetch_2d(&map_w128, kb * kBlockK, row_begin);
-        }
-    }
-    pdl_wait();          // everything above overlapped with the tail of the previous kernel
-    // The acceptance kernels behind this one are small: let them become resident now, fetch the inputs that
-    // do not depend on this grid, and wait for it there.
-    pdl_trigger();
-
-    if (warp == 0) {
-        // ------------------------------------------------ TMA producer
-        if (lane == 0) {
-            uint64_t pol_stream, pol_keep;
-            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
-            asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
-            int s = 0;
-            uint32_t ph = 0;
-            uint8_t* w_dst = smem;
-            bool ok = true;
-            for (int t = 0; t < n_tiles && ok; ++t) {
-                const int v0 = row_begin + t * tile_rows + (int)pair_rank * kVocabTile;
-                const int rows = PAIR ? kVocabTile : min(tile_rows, row_end - v0);
-                const uint32_t tx_bytes = (uint32_t)(rows * 128 + p.n_tile * 128);
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!mbar_wait(&empty_bar[s], ph ^ 1u, abort_ptr)) { ok = false; break; }
-#ifdef MASSV_TEST_HOOKS
-                    if (p.test_skip_stage && t == 0 && kb == 1) {
-                        // nothing is announced and nothing is copied for this stage: the MMA thread's wait for it
-                        // must give up by itself
-                        w_dst += stage_bytes;
-                        if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
-                        continue;
-                    }
-#endif
-                    uint8_t* h_dst = w_dst + kTileBytesW;
-                    if constexpr (PAIR) {
-                        // Both CTAs' copies complete on the leader's barrier; the leader announces the
-                        // bytes of the pair (two 128-row weight boxes, two halves of the hidden-state tile;
-                        // rows past the end of either matrix are filled with zeros and still counted).
-                        const uint32_t bar = cluster_addr(&full_bar[s], 0);
-                        if (pair_rank == 0) mbar_expect_tx_at(bar, (uint32_t)(2 * kTileBytesW + p.n_tile * 128));
-                        tma_load_2d_pair(w_dst, &map_w128, kb * kBlockK, v0, bar, pol_stream);
-                        tma_load_2d_pair(h_dst, &map_h, kb * kBlockK, (int)pair_rank * h_rows, bar, pol_keep);
-                        w_dst += stage_bytes;
-                        if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
-                        continue;
-                    }
-                    mbar_expect_tx(&full_bar[s], tx_bytes);
-                    if (rows == kVocabTile) {
-                        tma_load_2d(w_dst, &map_w128, kb * kBlockK, v0, &full_bar[s], pol_stream);
-                    } else {
-                        // rows is a multiple of 8 below 128: one box per set bit
-                        int r = 0;
-                        if (rows & 64) { tma_load_2d(w_dst + r * 128, &map_w64, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 64; }
-                        if (rows & 32) { tma_load_2d(w_dst + r * 128, &map_w32, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 32; }
-                        if (rows & 16) { tma_load_2d(w_dst + r * 128, &map_w16, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 16; }
-                        if (rows & 8) { tma_load_2d(w_dst + r * 128, &map_w8, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 8; }
-                    }
-                    tma_load_2d(h_dst, &map_h, kb * kBlockK, 0, &full_bar[s], pol_keep);
-                    w_dst += stage_bytes;
-                    if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
-                }
-            }
-            if (!ok) {
-                // let copies that are still in flight land before the CTA retires
-                for (int i = 0; i < 64; ++i) __nanosleep(2000);
-            }
-        }
-    } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer
-        if (lane == 0 && pair_rank == 0) {       // in a pair only the leader issues
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.n_tile >> 3) << 17) |
-                                   ((uint32_t)((PAIR ? 2 * kVocabTile : kVocabTile) >> 4) << 24);
-            // The issuing thread must stay far below the 64..128 cycles one MMA takes, so the
-            // loop carries only 32-bit descriptor words and a stage counter.
-            const uint32_t lo_step = (uint32_t)stage_bytes >> 4;
-            const uint32_t a_lo0 = umma_desc_lo(smem_u32(smem));
-            int s = 0;
-            uint32_t ph = 0, a_lo = a_lo0;
-            bool ok = true;
-            for (int t = 0; t < n_tiles && ok; ++t) {
-                const int buf = t & 1;
-                if (!mbar_wait(&tmem_empty_bar[buf], (((uint32_t)t >> 1) & 1u) ^ 1u, abort_ptr)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * p.n_tile);
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    if (!mbar_wait(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t b_lo = a_lo + (kTileBytesW >> 4);
-                    // four K slices of 16 elements (32 bytes, i.e. 2 descriptor units) each
-                    if constexpr (PAIR) {
-                        if (kb == 0) umma_bf16_pair<false>(d_tmem, a_lo, b_lo, idesc);
-                        else umma_bf16_pair<true>(d_tmem, a_lo, b_lo, idesc);
-                        umma_bf16_pair<true>(d_tmem, a_lo + 2, b_lo + 2, idesc);
-                        umma_bf16_pair<true>(d_tmem, a_lo + 4, b_lo + 4, idesc);
-                        umma_bf16_pair<true>(d_tmem, a_lo + 6, b_lo + 6, idesc);
-                        umma_commit_pair(&empty_bar[s]);     // frees the stage in both CTAs
-                    } else {
-                        if (kb == 0) umma_bf16<false>(d_tmem, a_lo, b_lo, idesc);
-                        else umma_bf16<true>(d_tmem, a_lo, b_lo, idesc);
-                        umma_bf16<true>(d_tmem, a_lo + 2, b_lo + 2, idesc);
-                        umma_bf16<true>(d_tmem, a_lo + 4, b_lo + 4, idesc);
-                        umma_bf16<true>(d_tmem, a_lo + 6, b_lo + 6, idesc);
-                        umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
-                    }
-                    a_lo += lo_step;
-                    if (++s == p.stages) { s = 0; ph ^= 1u; a_lo = a_lo0; }
-                }
-                if (ok) {
-                    if constexpr (PAIR) umma_commit_pair(&tmem_full_bar[buf]);
-                    else umma_commit(&tmem_full_bar[buf]);
-                }
-            }
-        }
-    } else {
-        // ------------------------------------------------ epilogue (warps 2..9)
-        // TMEM lanes 32*quarter .. +31 are the only ones warp (quarter = warp % 4) may read; the two
-        // warps that share a quarter take alternate column chunks.
-        const int quarter = warp & 3;
-        const int half = (warp - 2) >> 2;
-        const int row_in_tile = quarter * 32 + lane;
-        const int n_chunks32 = p.n_tile / 32;
-        const bool tail16 = (p.n_tile % 32) != 0;
-        // running statistics per (quarter, column); each column is touched by exactly one lane of one warp
-        if (half == 0)
-            for (int c = lane; c < 256; c += 32) { run_m[quarter][c] = -INFINITY; run_s[quarter][c] = 0.f; run_i[quarter][c] = 0x7fffffff; }
-        asm volatile("bar.sync 1, %0;" ::"r"(kEpilogueWarps * 32) : "memory");     // epilogue warps only
-        bool ok = true;
-        for (int t = 0; t < n_tiles && ok; ++t) {
-            const int buf = t & 1;
-            if (!mbar_wait(&tmem_full_bar[buf], ((uint32_t)t >> 1) & 1u, abort_ptr)) { ok = false; break; }
-            tc_fence_after();
-            TileCtx tile;
-            tile.v0 = row_begin + t * tile_rows + (int)pair_rank * kVocabTile;     // this CTA's 128 rows
-            tile.rows = max(0, min(kVocabTile, row_end - tile.v0));
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.n_tile);
-            for (int c = half; c < n_chunks32; c += 2) {
-                const int col = c * 32 + lane;
-                Stat running{run_m[quarter][col], run_s[quarter][col], run_i[quarter][col]};
-                drain_chunk<32>(p, taddr + c * 32, lane, row_in_tile, tile, c * 32, running);
-                run_m[quarter][col] = running.m; run_s[quarter][col] = running.s; run_i[quarter][col] = running.idx;
-            }
-            if (tail16 && (n_chunks32 & 1) == half) {
-                // lanes 2c and 2c+1 both end up with column c of the 16-column tail; the even lane keeps it
-                const int col = n_chunks32 * 32 + (lane >> 1);
-                Stat running{run_m[quarter][col], run_s[quarter][col], run_i[quarter][col]};
-                drain_chunk<16>(p, taddr + n_chunks32 * 32, lane, row_in_tile, tile, n_chunks32 * 32, running);
-                __syncwarp();
-                if ((lane & 1) == 0) { run_m[quarter][col] = running.m; run_s[quarter][col] = running.s; run_i[quarter][col] = running.idx; }
-                __syncwarp();
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                if constexpr (PAIR) mbar_arrive_at(cluster_addr(&tmem_empty_bar[buf], 0));   // the leader waits for both CTAs
-                else mbar_arrive(&tmem_empty_bar[buf]);
-            }
-        }
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    // the CTA's statistics: merge the four lane quarters (ascending rows) into one partial slot
-    for (int c = threadIdx.x; c < p.n_tile; c += kThreads) {
-        const int tok = c;
-        if (tok < p.M) {
-            Stat acc{run_m[0][c], run_s[0][c], run_i[0][c]};
-#pragma unroll
-            for (int qd = 1; qd < 4; ++qd)
-                acc = stat_combine(acc, Stat{run_m[qd][c], run_s[qd][c], run_i[qd][c]}, p.scale_log2, p.greedy != 0);
-            const size_t slot = (size_t)(PAIR ? group * 2 + (int)pair_rank : group) * p.M;
-            if (MASSV_IN_BOUNDS(slot + tok, (size_t)p.n_part * p.M, p.dev_status)) {
-                p.part_max[slot + tok] = acc.m;
-                p.part_sum[slot + tok] = p.greedy ? 0.f : acc.s;
-                p.part_idx[slot + tok] = acc.idx == 0x7fffffff ? acc.idx : acc.idx + p.idx_offset;
-            }
-        }
-    }
-    if constexpr (PAIR) cluster_sync_all();      // neither CTA frees TMEM or leaves while the other may still use it
-    if (warp == 1) {
-        __syncwarp();
-        tc_fence_after();
-        if constexpr (PAIR)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
-        else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
-    }
-    if (threadIdx.x == 0 && abort_flag) set_status(p.dev_status, MASSV_ERR_TIMEOUT);
 }
 
 // 16 TMEM lanes x 64 columns -> 32 registers per thread.  Register 4k+e holds row (lane/4 + 8*(e>>1)) of the
@@ -658,6 +390,271 @@ __device__ __forceinline__ void stats_job64(const UmmaParams& p, uint32_t (&va)[
             if (!greedy) run_s[c] = rs;
         }
     }
+}
+
+// PAIR: the grid is made of 2-CTA clusters; a pair works on 256-row vocabulary super-tiles (CTA rank r
+// owns rows 128 r .. 128 r + 127 and half of the token rows of the hidden-state tile), which halves the
+// hidden-state traffic per weight byte compared with one CTA per 128 rows.
+template <bool PAIR>
+__global__ void __launch_bounds__(lm_head_threads(PAIR), 1)
+lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_constant__ CUtensorMap map_w64,
+                    const __grid_constant__ CUtensorMap map_w32, const __grid_constant__ CUtensorMap map_w16,
+                    const __grid_constant__ CUtensorMap map_w8, const __grid_constant__ CUtensorMap map_h,
+                    const UmmaParams p) {
+    constexpr int kEpilogueWarps = epilogue_warps(PAIR), kThreads = lm_head_threads(PAIR);
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kMaxStages];
+    __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
+    __shared__ __align__(8) uint64_t tmem_full_bar[2];
+    __shared__ __align__(8) uint64_t tmem_empty_bar[2];
+    __shared__ uint32_t tmem_base_slot;
+    __shared__ int abort_flag;
+    __shared__ float run_m[4][256];
+    __shared__ float run_s[4][256];
+    __shared__ int run_i[4][256];
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int h_rows = PAIR ? p.n_tile / 2 : p.n_tile;       // hidden-state rows this CTA loads per K block
+    const int stage_bytes = kTileBytesW + h_rows * 128;
+    const int num_kb = p.K / kBlockK;
+    const uint32_t pair_rank = PAIR ? cluster_cta_rank() : 0u;
+
+    // which band of vocabulary rows this CTA (or pair) owns
+    const int group = PAIR ? blockIdx.x / 2 : blockIdx.x;
+    constexpr int tile_rows = PAIR ? 2 * kVocabTile : kVocabTile;       // rows per (super-)tile of the band
+    const int row_begin = min(p.V, group * p.tiles_per_group * tile_rows);
+    const int row_end = min(p.V, row_begin + p.tiles_per_group * tile_rows);
+    const int n_tiles = (row_end - row_begin + tile_rows - 1) / tile_rows;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+        // in a pair the leader's tmem_empty barriers collect both CTAs' epilogue warps
+        for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full_bar[b], 1); mbar_init(&tmem_empty_bar[b], (PAIR ? 2 : 1) * kEpilogueWarps); }
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        __syncwarp();
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
+                         "r"((uint32_t)p.tmem_cols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
+                         "r"((uint32_t)p.tmem_cols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();      // the peer's barriers exist before anything signals them
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_slot;
+    volatile int* abort_ptr = &abort_flag;
+    // The weights do not depend on the kernel before this one: while it drains, an epilogue warp (idle
+    // until the first accumulator is ready) asks L2 for the first boxes of this CTA's first tile.
+    // Single-CTA tiles only: with CTA pairs the hints cost more than they bring.  Depth by measurement:
+    // the step gains up to 32 boxes (-2.4 %), beyond 40 the hinted boxes are fetched twice too often.
+    if constexpr (!PAIR) {
+        if (warp == 2 && lane == 0 && n_tiles > 0) {
+            const int n_pf = min(num_kb, kPrefetchBlocks);
+            for (int kb = 0; kb < n_pf; ++kb) tma_prefetch_2d(&map_w128, kb * kBlockK, row_begin);
+        }
+    }
+    pdl_wait();          // everything above overlapped with the tail of the previous kernel
+    // The acceptance kernels behind this one are small: let them become resident now, fetch the inputs that
+    // do not depend on this grid, and wait for it there.
+    pdl_trigger();
+
+    if (warp == 0) {
+        // ------------------------------------------------ TMA producer
+        if (lane == 0) {
+            uint64_t pol_stream, pol_keep;
+            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
+            asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
+            int s = 0;
+            uint32_t ph = 0;
+            uint8_t* w_dst = smem;
+            bool ok = true;
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                const int v0 = row_begin + t * tile_rows + (int)pair_rank * kVocabTile;
+                const int rows = PAIR ? kVocabTile : min(tile_rows, row_end - v0);
+                const uint32_t tx_bytes = (uint32_t)(rows * 128 + p.n_tile * 128);
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    if (!mbar_wait(&empty_bar[s], ph ^ 1u, abort_ptr)) { ok = false; break; }
+#ifdef MASSV_TEST_HOOKS
+                    if (p.test_skip_stage && t == 0 && kb == 1) {
+                        // nothing is announced and nothing is copied for this stage: the MMA thread's wait for it
+                        // must give up by itself
+                        w_dst += stage_bytes;
+                        if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
+                        continue;
+                    }
+#endif
+                    uint8_t* h_dst = w_dst + kTileBytesW;
+                    if constexpr (PAIR) {
+                        // Both CTAs' copies complete on the leader's barrier; the leader announces the
+                        // bytes of the pair (two 128-row weight boxes, two halves of the hidden-state tile;
+                        // rows past the end of either matrix are filled with zeros and still counted).
+                        const uint32_t bar = cluster_addr(&full_bar[s], 0);
+                        if (pair_rank == 0) mbar_expect_tx_at(bar, (uint32_t)(2 * kTileBytesW + p.n_tile * 128));
+                        tma_load_2d_pair(w_dst, &map_w128, kb * kBlockK, v0, bar, pol_stream);
+                        tma_load_2d_pair(h_dst, &map_h, kb * kBlockK, (int)pair_rank * h_rows, bar, pol_keep);
+                        w_dst += stage_bytes;
+                        if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
+                        continue;
+                    }
+                    mbar_expect_tx(&full_bar[s], tx_bytes);
+                    if (rows == kVocabTile) {
+                        tma_load_2d(w_dst, &map_w128, kb * kBlockK, v0, &full_bar[s], pol_stream);
+                    } else {
+                        // rows is a multiple of 8 below 128: one box per set bit
+                        int r = 0;
+                        if (rows & 64) { tma_load_2d(w_dst + r * 128, &map_w64, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 64; }
+                        if (rows & 32) { tma_load_2d(w_dst + r * 128, &map_w32, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 32; }
+                        if (rows & 16) { tma_load_2d(w_dst + r * 128, &map_w16, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 16; }
+                        if (rows & 8) { tma_load_2d(w_dst + r * 128, &map_w8, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 8; }
+                    }
+                    tma_load_2d(h_dst, &map_h, kb * kBlockK, 0, &full_bar[s], pol_keep);
+                    w_dst += stage_bytes;
+                    if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
+                }
+            }
+            if (!ok) {
+                // let copies that are still in flight land before the CTA retires
+                for (int i = 0; i < 64; ++i) __nanosleep(2000);
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        if (lane == 0 && pair_rank == 0) {       // in a pair only the leader issues
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.n_tile >> 3) << 17) |
+                                   ((uint32_t)((PAIR ? 2 * kVocabTile : kVocabTile) >> 4) << 24);
+            // The issuing thread must stay far below the 64..128 cycles one MMA takes, so the
+            // loop carries only 32-bit descriptor words and a stage counter.
+            const uint32_t lo_step = (uint32_t)stage_bytes >> 4;
+            const uint32_t a_lo0 = umma_desc_lo(smem_u32(smem));
+            int s = 0;
+            uint32_t ph = 0, a_lo = a_lo0;
+            bool ok = true;
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                const int buf = t & 1;
+                if (!mbar_wait(&tmem_empty_bar[buf], (((uint32_t)t >> 1) & 1u) ^ 1u, abort_ptr)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * p.tmem_cols / 2);
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    if (!mbar_wait(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t b_lo = a_lo + (kTileBytesW >> 4);
+                    // four K slices of 16 elements (32 bytes, i.e. 2 descriptor units) each
+                    if constexpr (PAIR) {
+                        if (kb == 0) umma_bf16_pair<false>(d_tmem, a_lo, b_lo, idesc);
+                        else umma_bf16_pair<true>(d_tmem, a_lo, b_lo, idesc);
+                        umma_bf16_pair<true>(d_tmem, a_lo + 2, b_lo + 2, idesc);
+                        umma_bf16_pair<true>(d_tmem, a_lo + 4, b_lo + 4, idesc);
+                        umma_bf16_pair<true>(d_tmem, a_lo + 6, b_lo + 6, idesc);
+                        umma_commit_pair(&empty_bar[s]);     // frees the stage in both CTAs
+                    } else {
+                        if (kb == 0) umma_bf16<false>(d_tmem, a_lo, b_lo, idesc);
+                        else umma_bf16<true>(d_tmem, a_lo, b_lo, idesc);
+                        umma_bf16<true>(d_tmem, a_lo + 2, b_lo + 2, idesc);
+                        umma_bf16<true>(d_tmem, a_lo + 4, b_lo + 4, idesc);
+                        umma_bf16<true>(d_tmem, a_lo + 6, b_lo + 6, idesc);
+                        umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+                    }
+                    a_lo += lo_step;
+                    if (++s == p.stages) { s = 0; ph ^= 1u; a_lo = a_lo0; }
+                }
+                if (ok) {
+                    if constexpr (PAIR) umma_commit_pair(&tmem_full_bar[buf]);
+                    else umma_commit(&tmem_full_bar[buf]);
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------ epilogue
+        // TMEM lanes 32*quarter .. +31 are the only ones warp (quarter = warp % 4) may read.  Pairs: the four warps of a
+        // quarter take 64 columns each, copy them to registers and give the accumulator back before they compute.
+        // Single CTAs (tiles of up to 48 columns): the two warps of a quarter take alternate chunks of 16 columns.
+        const int quarter = warp & 3;
+        const int part = (warp - 2) >> 2;
+        // running statistics per (quarter, column); each column is touched by exactly one lane of one warp
+        for (int c = threadIdx.x - 64; c < 4 * 256; c += kEpilogueWarps * 32) {
+            (&run_m[0][0])[c] = -INFINITY; (&run_s[0][0])[c] = 0.f; (&run_i[0][0])[c] = 0x7fffffff;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");     // epilogue warps only
+        bool ok = true;
+        for (int t = 0; t < n_tiles && ok; ++t) {
+            const int buf = t & 1;
+            if (!mbar_wait_warp(&tmem_full_bar[buf], ((uint32_t)t >> 1) & 1u, abort_ptr)) { ok = false; break; }
+            tc_fence_after();
+            TileCtx tile;
+            tile.v0 = row_begin + t * tile_rows + (int)pair_rank * kVocabTile;     // this CTA's 128 rows
+            tile.rows = max(0, min(kVocabTile, row_end - tile.v0));
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.tmem_cols / 2);
+            if constexpr (PAIR) {
+                const int c0 = part * 64, n_cols = min(64, p.n_tile - c0);
+                uint32_t va[32], vb[32];
+                if (n_cols > 0) {                                  // the same in every lane
+                    tmem_load_16x64(taddr + c0, va);               // rows 0-15 of the quarter
+                    tmem_load_16x64(taddr + c0 + (16u << 16), vb); // rows 16-31
+                    tmem_wait_ld<32>(va);
+                    tmem_wait_ld<32>(vb);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_at(cluster_addr(&tmem_empty_bar[buf], 0));   // the leader waits for both CTAs
+                if (n_cols > 0)
+                    stats_job64(p, va, vb, lane, quarter, tile, c0, n_cols, &run_m[quarter][c0], &run_s[quarter][c0], &run_i[quarter][c0]);
+            } else {
+                for (int c0 = part * 16; c0 < p.n_tile; c0 += 32) {
+                    // lanes 2c and 2c+1 both end up with column c of the 16; the even lane keeps it
+                    const int col = c0 + (lane >> 1);
+                    Stat running{run_m[quarter][col], run_s[quarter][col], run_i[quarter][col]};
+                    drain_chunk<16>(p, taddr + c0, lane, quarter * 32 + lane, tile, c0, running);
+                    __syncwarp();
+                    if ((lane & 1) == 0) { run_m[quarter][col] = running.m; run_s[quarter][col] = running.s; run_i[quarter][col] = running.idx; }
+                    __syncwarp();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tmem_empty_bar[buf]);
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    // the CTA's statistics: merge the four lane quarters (ascending rows) into one partial slot
+    for (int c = threadIdx.x; c < p.n_tile; c += kThreads) {
+        const int tok = c;
+        if (tok < p.M) {
+            Stat acc{run_m[0][c], run_s[0][c], run_i[0][c]};
+#pragma unroll
+            for (int qd = 1; qd < 4; ++qd)
+                acc = stat_combine(acc, Stat{run_m[qd][c], run_s[qd][c], run_i[qd][c]}, p.scale_log2, p.greedy != 0);
+            const size_t slot = (size_t)(PAIR ? group * 2 + (int)pair_rank : group) * p.M;
+            if (MASSV_IN_BOUNDS(slot + tok, (size_t)p.n_part * p.M, p.dev_status)) {
+                p.part_max[slot + tok] = acc.m;
+                p.part_sum[slot + tok] = p.greedy ? 0.f : acc.s;
+                p.part_idx[slot + tok] = acc.idx == 0x7fffffff ? acc.idx : acc.idx + p.idx_offset;
+            }
+        }
+    }
+    if constexpr (PAIR) cluster_sync_all();      // neither CTA frees TMEM or leaves while the other may still use it
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)p.tmem_cols) : "memory");
+    }
+    if (threadIdx.x == 0 && abort_flag) set_status(p.dev_status, MASSV_ERR_TIMEOUT);
 }
 
 // ---- One pass over the weights for 257 .. 512 token rows (CTA pairs only).
@@ -975,8 +972,9 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     int stages = kRingBytes / stage_bytes;
     if (stages > kMaxStages) stages = kMaxStages;
     p.stages = stages;
+    // two accumulators, each in half of the allocation (pairs read 64 columns at a time)
     int cols = 32;
-    while (cols < 2 * p.n_tile) cols *= 2;
+    while (cols < 2 * (pair ? (p.n_tile + 63) / 64 * 64 : p.n_tile)) cols *= 2;
     p.tmem_cols = cols;
     p.greedy = q.greedy;
     p.scale_log2 = q.inv_T_log2e;
@@ -1000,12 +998,12 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     if (pair) {
         e = cudaFuncSetAttribute(lm_head_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * 2), dim3(kThreads), smem, stream, 2,
+        e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * 2), dim3(lm_head_threads(true)), smem, stream, 2,
                                map_w[0], map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
     } else {
         e = cudaFuncSetAttribute(lm_head_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups), dim3(kThreads), smem, stream, map_w[0],
+        e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups), dim3(lm_head_threads(false)), smem, stream, map_w[0],
                        map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
     }
     if (e != cudaSuccess) return e;

@@ -1,4 +1,4 @@
-"""The LM head with more than 256 rows (two sub-tiles over one pass of the weights) at the edges of its sub-tiles and of the way
+"""The LM head at the edges of its row tiles (16-column chunks of single CTAs, 64-column jobs of CTA pairs, the two sub-tiles above 256 rows) and of the way
 it deals the vocabulary out: one band, bands that take a pair per sub-tile and the first count that does not, left-over bands,
 ragged ends; logits against 64 bits, greedy tokens against the logits' own argmax, probabilities from the merged statistics."""
 import pytest
@@ -7,7 +7,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("batch,gamma", [(257, 0), (68, 3), (64, 5), (77, 4), (100, 3), (73, 6), (64, 7)])
+@pytest.mark.parametrize("batch,gamma", [(1, 0), (17, 0), (11, 2), (48, 0), (49, 0), (16, 3), (13, 4), (16, 5), (43, 2), (32, 5), (51, 4), (64, 3), (257, 0), (68, 3), (64, 5), (77, 4), (100, 3), (73, 6), (64, 7)])
 @pytest.mark.parametrize("vocab", [8, 264, 9472, 9480, 18944, 19208, 40008])
 def test_rows(batch, gamma, vocab):
     import paper_2505_10526_b200 as mv
