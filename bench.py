@@ -267,7 +267,7 @@ def roofline_block(kernel, bound, algorithmic, ms, peaks, peak_src, family):
          "ms_per_launch_best": ms["best"]}
     if bound == "tensor" and peaks.get("bf16_tflops_sustained"):
         r["frac_of_sustained"] = achieved / peaks["bf16_tflops_sustained"]
-    key = {"attn_umma_kernel": "attn", "attn_split_kernel": "attn", "lm_head_umma_kernel": "lm_head", "lm_head_duo_kernel": "lm_head",
+    key = {"attn_umma_kernel": "attn", "attn_split_kernel": "attn", "attn_flat_kernel": "attn", "accept_row_kernel": "residual", "lm_head_umma_kernel": "lm_head", "lm_head_duo_kernel": "lm_head",
            "residual_sample_kernel": "residual"}[kernel]
     ratio = NCU_TRAFFIC_RATIO.get((key, family))
     r["traffic"] = None if (ratio is None or bound == "tensor") else ratio * algorithmic
@@ -376,16 +376,18 @@ def measure(mv, cfg, dev, K, W, attn_kernel, peaks, peak_src, world, sampler=Non
     lm_flops = 2.0 * cfg.m * cfg.vocab * cfg.hidden
     attn_bytes = kv_bytes(cfg, seq0.tolist())
     ridge = peaks["bf16_tflops"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
-    attn_name = "attn_umma_kernel" if (attn_kernel == 2 or (attn_kernel == 0 and cfg.head_dim <= 128)) else "attn_split_kernel"
+    attn_name = "attn_umma_kernel" if (attn_kernel == 2 or (attn_kernel == 0 and cfg.head_dim <= 128)) else "attn_flat_kernel"
     rl = {"attn": roofline_block(attn_name, "hbm", attn_bytes, t_attn_k, peaks, peak_src, family),
-          # 257 .. 384 token rows take the one-pass kernel (two sub-tiles of the rows in tensor memory at once)
-          "lm_head": roofline_block("lm_head_duo_kernel" if 256 < cfg.m <= 384 else "lm_head_umma_kernel", "tensor" if cfg.m > ridge else "hbm",
+          # more than 256 token rows take the one-pass kernel (two sub-tiles of the rows in tensor memory at once)
+          "lm_head": roofline_block("lm_head_duo_kernel" if cfg.m > 256 else "lm_head_umma_kernel", "tensor" if cfg.m > ridge else "hbm",
                                     lm_flops if cfg.m > ridge else lm_bytes, t_lm, peaks, peak_src, family)}
     rl["attn"]["frac_whole_call"] = attn_bytes / (t_attn["mean"] * 1e-3) / 1e9 / peaks["hbm_gbs"]
     rl["lm_head"]["frac_whole_accept_call"] = rl["lm_head"]["algorithmic"] / (t_accept["mean"] * 1e-3) / \
         (1e12 if cfg.m > ridge else 1e9) / rl["lm_head"]["peak"]
     if sampling:
-        rl["residual"] = roofline_block("residual_sample_kernel", "hbm", cfg.batch * cfg.vocab * 8, t_res, peaks, peak_src, family)
+        # few sequences: the accept tests and the draw are one launch (accept_row_kernel), timed as a whole
+        one_launch = cfg.batch * 8 <= (224 if cfg.vocab <= 8 * 26880 else 96)
+        rl["residual"] = roofline_block("accept_row_kernel" if one_launch else "residual_sample_kernel", "hbm", cfg.batch * cfg.vocab * 8, t_res, peaks, peak_src, family)
     shares = {"attn": t_attn_k["mean"], "lm_head": t_lm["mean"]}
     if sampling:
         shares["residual"] = t_res["mean"]

@@ -235,8 +235,8 @@ size_t massv_tvd_workspace_size(const massv_accept_desc *desc);
  *   logits        fp32 [B, R, V]   (the logits_out of massv_accept; rows 0..gamma-1 are used)
  *   draft_probs   fp32 [B, gamma, V]
  *   tvd_out       fp32 [B, gamma];  accept_prob_out  optional fp32 [B, gamma]
- * Needs T > 0 and gamma >= 1.  Reads every drafted row once (B*gamma*V*8 bytes),
- * twice for the logits; sums run in fp64 in a fixed order.
+ * Needs T > 0 and gamma >= 1.  Reads every drafted row once (B*gamma*V*8 bytes), the
+ * logits of many rows a second time; sums run in fp64 in a fixed order.
  */
 int massv_tvd(const massv_accept_desc *desc, const float *logits, const float *draft_probs,
               float *tvd_out, float *accept_prob_out,
@@ -403,7 +403,8 @@ int massv_set_timing_events(massv_event_t lm_head_start, massv_event_t lm_head_s
 
 /* The same hook, one kernel at a time: `kernel` is one of MASSV_TIMED_*; NULL for both events
  * switches that kernel's hook off.  MASSV_TIMED_RESIDUAL is the residual / bonus draw of
- * massv_accept at T > 0 (the one pass over the vocabulary row the extra token is drawn from). */
+ * massv_accept at T > 0 (the one pass over the vocabulary row the extra token is drawn from; with few
+ * sequences the acceptance tests are part of the same launch). */
 #define MASSV_TIMED_LM_HEAD 0
 #define MASSV_TIMED_ATTN 1
 #define MASSV_TIMED_RESIDUAL 2
