@@ -106,6 +106,9 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
             const int row = first + i / UPR, u = i % UPR;
             *reinterpret_cast<uint4*>(vst + (u / 8) * kRegion + swz(row, u % 8)) = make_uint4(0u, 0u, 0u, 0u);
         }
+        // The balanced schedule refills this stage for its next pair: these stores have to be ordered ahead of the TMA's
+        // (async-proxy) writes to the same bytes, which the mbarrier between the two does not do.
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
     }
     const uint32_t k_base = smem_u32(kst), v_base = smem_u32(vst);

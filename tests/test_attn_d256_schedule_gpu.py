@@ -8,10 +8,10 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-def _inputs(batch, gamma, q_heads, kv_heads, lens, seed):
+def _inputs(batch, gamma, q_heads, kv_heads, lens, seed, max_pages=0):
     g = torch.Generator(device="cuda").manual_seed(seed)
     R, d = gamma + 1, 256
-    max_pages = (max(lens) + R + 15) // 16
+    max_pages = max_pages or (max(lens) + R + 15) // 16
     n_pages = batch * max_pages + 2
     bf = dict(dtype=torch.bfloat16, device="cuda", generator=g)
     table = torch.randperm(n_pages, generator=g, device="cuda")[:batch * max_pages].view(batch, max_pages).to(torch.int32)
@@ -74,3 +74,30 @@ def test_against_fp32(batch, gamma, q_heads, kv_heads, lo, hi, window):
         for j in range(gamma + 1):
             page, at = int(w["page_table"][b, (n + j) // 16]), (n + j) % 16
             assert torch.equal(w["k_pages"][page, :, at], w["k_new"][b, j]) and torch.equal(w["v_pages"][page, :, at], w["v_new"][b, j])
+
+
+@pytest.mark.parametrize("batch,gamma,q_heads,kv_heads,hi", [(300, 5, 16, 8, 40), (300, 0, 8, 8, 90), (300, 3, 32, 4, 30), (200, 7, 8, 1, 60), (260, 7, 16, 2, 25)])
+def test_many_short_pairs_per_cta(batch, gamma, q_heads, kv_heads, hi):
+    """Contexts far below the page table's capacity: a CTA's range is many pairs of one to three tiles, so every stage of its ring
+    is patched (block rows, zeros past the end) and refilled with another pair's query rows or tiles over and over."""
+    import paper_2505_10526_b200 as mv
+    g = torch.Generator().manual_seed(batch + hi)
+    lens = torch.randint(0, hi + 1, (batch,), generator=g).tolist()
+    w = _inputs(batch, gamma, q_heads, kv_heads, lens, seed=hi + gamma, max_pages=40)
+    want, want_lse = _reference(w, 0)
+    desc = mv.attn_desc(batch, gamma, q_heads, kv_heads, 256, 40, w["k_pages"].shape[0])
+    ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda")
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    first = None
+    for _ in range(5):
+        out = torch.full_like(w["q"], float("nan"))
+        f32 = torch.full(out.shape, float("nan"), device="cuda")
+        lse = torch.full(out.shape[:3], float("nan"), device="cuda")
+        mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, lse, ws, status)
+        assert int(status.item()) == 0
+        # an output row is a sum of w_i v_i whose weights carry bf16's 2^-9 each: 2^-9 of the row's norm for independent values
+        assert float(((f32 - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 4e-3
+        # the weights' sum is taken before that rounding: fp32 scores of a few units, fp32 exponentials
+        assert float((lse - want_lse).abs().max()) < 2e-5
+        first = out if first is None else first
+        assert torch.equal(out, first)
