@@ -25,6 +25,7 @@ namespace {
 
 constexpr int kChunkAlign = 64;      // kv_chunk granularity (a multiple of every tile size)
 constexpr int kMaxChunkPages = 256;  // kv_chunk <= 4096 tokens
+constexpr float kRefDrop = 6.f;      // binary orders that a slice's reference may lie below the running maximum
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -48,6 +49,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+// 2^x in one instruction (results below 2^-126 are zero): for factors between maxima.
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Byte offset of the 16-byte unit `unit` (0..7) of row `row` inside a region of
 // 128-byte rows laid out with the 128-byte swizzle (what TMA writes).
 __device__ __forceinline__ uint32_t swz(int row, int unit) { return (uint32_t)(row * 128 + ((unit ^ (row & 7)) << 4)); }
@@ -64,12 +72,17 @@ struct AttnCfg {
 };
 
 // One tile of K/V for a warp: its 16 query rows (group mt) against its TILE/TS tokens (slice ts) of the tile at `kst` (K, then
-// V), the online softmax carried in (o, m_run, l_run).  page_of(position) is the page that holds it (asked for the block's
+// V), the online softmax carried in (o, m_run, l_run, r_run): l_run is relative to the running maximum m_run, o to r_run, the
+// maximum of the latest slice (kept within kRefDrop binary orders of m_run, so that o cannot outgrow its range).  The
+// largest weight of every slice is then exactly 1, and it is the heaviest weights whose rounding to bf16 shows in the
+// output.  With the running maximum as the reference only the maxima of a prefix were exact, so the error of a row depended
+// on the number of cuts its context had (32 x 8 pairs of 2k - 8k positions, error against 64 bits relative to the norm: 1.43e-3
+// with the fixed chunks, 1.47e-3 with the longer runs of the balanced schedule, 1.02e-3 with either now).  page_of(position) is the page that holds it (asked for the block's
 // own positions only: they are appended here).
 template <int D, int MT, int TS, int TILE, typename PageOf>
 __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, int L, int c_end, int tile_start, uint8_t* kst, uint32_t q_base,
                                             const uint32_t (&qf)[D <= 128 ? D / 16 : 1][4], int mt, int ts, int lane, int j0, int j1, float scale_log2,
-                                            PageOf&& page_of, float (&o)[D / 8][4], float (&m_run)[2], float (&l_run)[2]) {
+                                            PageOf&& page_of, float (&o)[D / 8][4], float (&m_run)[2], float (&l_run)[2], float (&r_run)[2]) {
     constexpr int kTile = TILE, NT = TILE / TS, RP = MT * 16;
     constexpr int kRegion = TILE * 128, kBytesK = (D / 64) * kRegion;
     constexpr bool kQInRegs = D <= 128;
@@ -160,9 +173,10 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
     mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
     const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
-    const float ms0 = mn0 == -INFINITY ? 0.f : mn0, ms1 = mn1 == -INFINITY ? 0.f : mn1;
-    const float corr0 = exp2f(m_run[0] - ms0), corr1 = exp2f(m_run[1] - ms1);
-    m_run[0] = mn0; m_run[1] = mn1;
+    const float rn0 = fmaxf(mx0, mn0 - kRefDrop), rn1 = fmaxf(mx1, mn1 - kRefDrop);
+    const float ms0 = rn0 == -INFINITY ? 0.f : rn0, ms1 = rn1 == -INFINITY ? 0.f : rn1;
+    const float corr0 = ex2(r_run[0] - ms0), corr1 = ex2(r_run[1] - ms1);
+    r_run[0] = rn0; r_run[1] = rn1;
     float ls0 = 0.f, ls1 = 0.f;
     uint32_t pa[NT / 16][4];
 #pragma unroll
@@ -174,8 +188,13 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
         pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16(p0, p1);
         pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16(p2, p3);
     }
-    l_run[0] = l_run[0] * corr0 + ls0;
-    l_run[1] = l_run[1] * corr1 + ls1;
+    const float mt0 = mn0 == -INFINITY ? 0.f : mn0, mt1 = mn1 == -INFINITY ? 0.f : mn1;
+    if (__any_sync(0xffffffffu, mn0 > m_run[0] || mn1 > m_run[1])) {
+        l_run[0] *= ex2(m_run[0] - mt0); l_run[1] *= ex2(m_run[1] - mt1);
+        m_run[0] = mn0; m_run[1] = mn1;
+    }
+    l_run[0] += ls0 * ex2(rn0 - mt0);
+    l_run[1] += ls1 * ex2(rn1 - mt1);
 #pragma unroll
     for (int n = 0; n < D / 8; ++n) { o[n][0] *= corr0; o[n][1] *= corr0; o[n][2] *= corr1; o[n][3] *= corr1; }
 
@@ -191,6 +210,14 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
             mma_bf16(o[2 * dp + 1], pa[tk], bf[2], bf[3]);
         }
     }
+}
+
+// The accumulator relative to the running maximum, as the merges take it.
+template <int D>
+__device__ __forceinline__ void settle(float (&o)[D / 8][4], const float (&m_run)[2], const float (&r_run)[2]) {
+    const float f0 = m_run[0] == -INFINITY ? 0.f : exp2f(r_run[0] - m_run[0]), f1 = m_run[1] == -INFINITY ? 0.f : exp2f(r_run[1] - m_run[1]);
+#pragma unroll
+    for (int n = 0; n < D / 8; ++n) { o[n][0] *= f0; o[n][1] *= f0; o[n][2] *= f1; o[n][3] *= f1; }
 }
 
 // Two CTAs should share an SM (one CTA's set-up and merge hide behind the other's
@@ -264,7 +291,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     volatile int* abort_ptr = &abort_flag;
 
     float o[D / 8][4];
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, r_run[2] = {-INFINITY, -INFINITY};
     const int mt = warp / TS, ts = warp % TS;
 
     if (warp == NW) {
@@ -324,10 +351,11 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             if (!mbar_wait(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
             const int tile_start = c_begin + t * kTile;
             attend_tile<D, MT, TS, TILE>(p, b, g, L, c_end, tile_start, smem + (size_t)s * Cfg::kStageBytes, q_base, qf, mt, ts, lane, j0, j1, scale_log2,
-                                         [&](int pos) { return s_pages[(pos - c_begin) / kPageSize]; }, o, m_run, l_run);
+                                         [&](int pos) { return s_pages[(pos - c_begin) / kPageSize]; }, o, m_run, l_run, r_run);
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty_bar[s]);
         }
+        settle<D>(o, m_run, r_run);
         l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 1);
         l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 2);
         l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 1);
@@ -589,16 +617,17 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
             float o[D / 8][4];
 #pragma unroll
             for (int n = 0; n < D / 8; ++n) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f; }
-            float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+            float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, r_run[2] = {-INFINITY, -INFINITY};
             for (int t = 0; t < w.n_tiles && ok; ++t) {
                 if (!mbar_wait_warp(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
                 attend_tile<D, MT, TS, TILE>(p, w.b, w.g, w.L, w.c_end, w.c_begin + t * TILE, smem + (size_t)s * Cfg::kStageBytes, q_base, no_q, mt, ts,
                                              lane, j0, j1, scale_log2, [&](int pos) { return p.page_table[(size_t)w.b * p.max_pages + pos / kPageSize]; },
-                                             o, m_run, l_run);
+                                             o, m_run, l_run, r_run);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty_bar[s]);
                 if (++s == E) { s = 0; ph ^= 1u; }
             }
+            settle<D>(o, m_run, r_run);
             l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 1);
             l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 2);
             l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 1);
