@@ -49,6 +49,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
 // 2^x in one instruction (results below 2^-126 are zero): for factors between maxima.
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -96,19 +100,22 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
         // The warp that owns those tokens puts them into the tile in shared memory, and
         // the mt == 0 warp also stores them to their page slots.
         const int p_first = max(L, tile_start + ts * NT), p_last = min(n_ctx, tile_start + ts * NT + NT);
+        // (All rows in flight at once: one after the other through registers, a pair of six rows took six memory latencies.)
         for (int i = lane; i < (p_last - p_first) * UPR; i += 32) {
             const int pos = p_first + i / UPR, u = i % UPR, row = pos - tile_start;
             const size_t src = (((size_t)b * p.R + (pos - L)) * p.Hkv + g) * D + u * 8;
-            const uint4 kv = *reinterpret_cast<const uint4*>(p.k_new + src);
-            const uint4 vv = *reinterpret_cast<const uint4*>(p.v_new + src);
-            *reinterpret_cast<uint4*>(kst + (u / 8) * kRegion + swz(row, u % 8)) = kv;
-            *reinterpret_cast<uint4*>(vst + (u / 8) * kRegion + swz(row, u % 8)) = vv;
-            if (mt == 0) {
+            cp_async_16(kst + (u / 8) * kRegion + swz(row, u % 8), p.k_new + src);
+            cp_async_16(vst + (u / 8) * kRegion + swz(row, u % 8), p.v_new + src);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (mt == 0) {
+            for (int i = lane; i < (p_last - p_first) * UPR; i += 32) {          // the units this lane has copied
+                const int pos = p_first + i / UPR, u = i % UPR, row = pos - tile_start;
                 const int pid = page_of(pos);
                 if (pid >= 0 && pid < p.num_pages) {
                     const size_t dst = (((size_t)pid * p.Hkv + g) * kPageSize + (pos % kPageSize)) * D + u * 8;
-                    *reinterpret_cast<uint4*>(p.k_pages + dst) = kv;
-                    *reinterpret_cast<uint4*>(p.v_pages + dst) = vv;
+                    *reinterpret_cast<uint4*>(p.k_pages + dst) = *reinterpret_cast<const uint4*>(kst + (u / 8) * kRegion + swz(row, u % 8));
+                    *reinterpret_cast<uint4*>(p.v_pages + dst) = *reinterpret_cast<const uint4*>(vst + (u / 8) * kRegion + swz(row, u % 8));
                 }
             }
         }
@@ -428,6 +435,11 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 // range: while the compute warps merge and write one pair, the producer is already filling the next one's tiles.
 // Against a grid of fixed chunks every CTA streams the same bytes whatever the mix of lengths and window bounds, and pays
 // its set-up once.
+// The line is measured in tiles, and a pair's set-up and merge count as kPairUnits tiles ahead of its own: a sequence of a few
+// positions is one tile for each of its heads, and a CTA that got a dozen such pairs for a dozen tiles of one long pair held
+// all others up.  64 x 8 pairs of 1 - 512 positions: 81 us with 0 units, 58, 51, 50 and 50 with 2, 4, 6 and 8; 32 x 8 of
+// 2k - 8k: 225, 225, 223, 223, 231; the same with a window of 1,024: 61.3, 62.1, 62.0, 63.3, 63.7.
+constexpr int kPairUnits = 4;
 template <int D, int MT, int TILE>
 struct FlatCfg {
     static constexpr int kTS = 2;                          // warps that share 16 query rows, each with half of a tile's tokens
@@ -469,7 +481,7 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
     }
     pdl_wait();
 
-    // tiles per pair of every sequence, then an exclusive prefix sum over the batch
+    // units per pair of every sequence, then an exclusive prefix sum over the batch
     auto first_tile = [&](int L) { return (p.window > 0 ? max(0, L - p.window + 1) : 0) / TILE; };
     for (int i = threadIdx.x; i < p.B; i += blockDim.x) {
         const int L = p.seq_lens[i];
@@ -477,7 +489,7 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         if (L < 0 || L + p.R > p.max_pages * kPageSize) {            // no room for the block: skip the sequence
             if (blockIdx.x == 0) set_status(p.dev_status, MASSV_ERR_CAPACITY);
         } else {
-            n = (L + p.R + TILE - 1) / TILE - first_tile(L);
+            n = (L + p.R + TILE - 1) / TILE - first_tile(L) + kPairUnits;
         }
         s_cum[i + 1] = n;
     }
@@ -502,13 +514,13 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
     const int per_cta = max(1, (total + (int)gridDim.x - 1) / (int)gridDim.x);
     if (blockIdx.x == 0) {          // what the merge kernel needs to find the pieces of a pair
         for (int i = threadIdx.x; i <= p.B; i += blockDim.x) p.flat_meta[2 + i] = s_cum[i];
-        if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = total; }
+        if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = kPairUnits; }
     }
     const int f_first = min(total, (int)blockIdx.x * per_cta), f_end = min(total, f_first + per_cta);
     volatile int* abort_ptr = &abort_flag;
 
-    // Piece of work at tile f of the line: a run of tiles of one pair, up to this CTA's end.
-    struct Piece { int b, g, L, c_begin, c_end, n_tiles; bool whole; };
+    // Piece of work at unit f of the line: a run of tiles of one pair, up to this CTA's end (none where that lies ahead of them).
+    struct Piece { int b, g, L, c_begin, c_end, n_tiles, n_units; bool whole; };
     int b_hint = 0;
     auto piece_at = [&](int f) {
         int lo = b_hint, hi = p.B - 1;                               // largest b with Hkv * cum[b] <= f
@@ -518,14 +530,15 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         }
         b_hint = lo;
         const int n_b = s_cum[lo + 1] - s_cum[lo], off = f - s_cum[lo] * p.Hkv;
-        const int t0 = off % n_b, t1 = min(n_b, t0 + (f_end - f));
+        const int u0 = off % n_b, u1 = min(n_b, u0 + (f_end - f)), t0 = max(0, u0 - kPairUnits), t1 = max(0, u1 - kPairUnits);
         Piece w;
         w.b = lo; w.g = off / n_b; w.L = p.seq_lens[lo];
         const int tile_lo = first_tile(w.L);
         w.c_begin = (tile_lo + t0) * TILE;
         w.c_end = min(w.L + p.R, (tile_lo + t1) * TILE);
         w.n_tiles = t1 - t0;
-        w.whole = t0 == 0 && t1 == n_b;
+        w.n_units = u1 - u0;
+        w.whole = t0 == 0 && u1 == n_b;
         return w;
     };
 
@@ -538,7 +551,8 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         bool ok = true;
         for (int f = f_first; f < f_end && ok;) {
             const Piece w = piece_at(f);
-            f += w.n_tiles;
+            f += w.n_units;
+            if (w.n_tiles == 0) continue;
             // page ids travel in registers, lane l holding page 32 * group + l; the next group's are fetched a group ahead
             const int32_t* pt = p.page_table + (size_t)w.b * p.max_pages + w.c_begin / kPageSize;
             const int n_pages = (w.c_end - w.c_begin + kPageSize - 1) / kPageSize;
@@ -602,7 +616,8 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         for (int f = f_first; f < f_end;) {
             const Piece w = piece_at(f);
             const size_t slot = (size_t)blockIdx.x * 2 + (f == f_first ? 0 : 1);
-            f += w.n_tiles;
+            f += w.n_units;
+            if (w.n_tiles == 0) continue;
             // the pair's query rows, from their ring stage to their place (same layout; zeros past the last row)
             if (ok && !mbar_wait_warp(&full_bar[s], ph, abort_ptr)) ok = false;
             for (int i = threadIdx.x; i < RP * UPR; i += NW * 32) {
@@ -814,20 +829,21 @@ bool attn_use_umma(const AttnParams& p) {
     return p.d <= 128;
 }
 
-// Balanced schedule or chunk grid for the warp-MMA kernel at head_dim 256.  The balanced one wins wherever a pair's tiles
-// are many or pairs are few (batch 32 x 8 heads: contexts 2k - 8k 228 -> 207 us, window 1,024 72 -> 57 us; batch 2, 1,000
-// positions 20 -> 16 us; 36 query rows 284 -> 176 us).  It loses where a pair is a few tiles and there are enough pairs
-// to occupy the chip one by one: a grid of one-pair CTAs has no ranges to cut and no pieces to merge (64 x 8 pairs: up to
-// 100 positions 21 against 29 us, up to 512 43 against 48, up to 1,024 75 against 71; 16 x 8 pairs up to 512: 19 against
-// 21).  From 17 rows up the balanced kernel's two warps per row group outweigh that except for the shortest
-// (64 x 4 pairs of 36 rows, up to 100 positions: 40 against 45 us, up to 256: 51 against 46).
+// Balanced schedule or chunk grid for the warp-MMA kernel at head_dim 256.  The balanced one wins wherever the grid would cut
+// a pair into chunks, since that costs CTAs that retire at once and a merge as well (times of a call, page table for 8,192
+// positions: 32 x 8 pairs of 2k - 8k positions 243 -> 224 us, of 100 - 900 50 -> 38, of 1 - 100 24 -> 23; a window of 1,024 on long
+// contexts 79 -> 62; 2 x 8 pairs of 1,000 positions 18.5 -> 16.6).  Where the table holds no more than one chunk, a grid of
+// one-pair CTAs has no ranges to cut and nothing to merge: it wins as long as its CTAs are resident at once (30 x 8 pairs of
+// 1 - 104 positions 17 against 23 us, of 400 - 600 34 against 38; 18 x 8 of 160 - 312 19 against 23), and up to about 544 positions
+// beyond that (64 x 8 pairs of 1 - 184: 35 against 37, of 272 - 536: 59 against 57, of 600 - 792: 89 against 81).  From 17
+// query rows up the balanced kernel's two warps per row group decide it (24 x 8 pairs of 24 rows, 1 - 54 positions: 33 -> 20 us;
+// 64 x 4 pairs of 36 rows, 2k - 6k: 412 -> 268).
 static bool use_flat_warp_mma(const AttnParams& p, int mt) {
     if (p.d != 256 || p.chunk_forced || p.B > kFlatMaxBatchMeta) return false;
+    if (mt > 1 || p.max_chunks > 1) return true;
     long tokens = (long)p.max_pages * kPageSize;                     // the most a pair can need
     if (p.window > 0 && p.window + p.R + 64 < tokens) tokens = p.window + p.R + 64;
-    const long pairs = (long)p.B * p.Hkv, ctas = (long)device_sm_count() * (mt == 1 ? 2 : 1);
-    if (mt == 1) return tokens > 544 || pairs * 5 < ctas * 2;
-    return tokens > 128 || pairs < ctas;
+    return tokens > 544 && (long)p.B * p.Hkv > 2L * device_sm_count();
 }
 
 cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream) {

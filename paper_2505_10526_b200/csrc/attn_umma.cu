@@ -212,7 +212,7 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         const int per_cta = max(1, (total + (int)gridDim.x - 1) / (int)gridDim.x);
         if (blockIdx.x == 0) {      // what the merge kernel needs to find the pieces of a pair
             for (int i = threadIdx.x; i <= p.B; i += blockDim.x) p.flat_meta[2 + i] = s_cum[i];
-            if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = total; }
+            if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = 0; }
         }
         f = min(total, (int)blockIdx.x * per_cta);
         f_end = min(total, f + per_cta);
@@ -761,11 +761,11 @@ __global__ void __launch_bounds__(kFlatCombineThreads) attn_flat_combine_kernel(
     const int qd = blockIdx.y / parts, part = blockIdx.y % parts;
     pdl_wait();
     pdl_trigger();
-    const int per_cta = p.flat_meta[0];
+    const int per_cta = p.flat_meta[0], ahead = p.flat_meta[1];     // units of a pair ahead of its first tile
     const int cum_b = p.flat_meta[2 + b], n_b = p.flat_meta[2 + b + 1] - cum_b;
     if (n_b <= 0) return;
     const int start = cum_b * p.Hkv + g * n_b, end = start + n_b;
-    const int c_first = start / per_cta, c_last = (end - 1) / per_cta;
+    const int c_first = (start + ahead) / per_cta, c_last = (end - 1) / per_cta;
     if (c_first == c_last) return;                 // the pair was finished by one CTA
     const int n = c_last - c_first + 1;
     auto slot_of = [&](int i) -> size_t { const int c = c_first + i; return (size_t)c * 2 + (start <= c * per_cta ? 0 : 1); };

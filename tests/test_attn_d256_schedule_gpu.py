@@ -122,3 +122,30 @@ def test_long_rows_are_as_exact_as_in_chunks(batch, gamma, q_heads, kv_heads, lo
         mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, lse, ws, None)
         assert float((f32 - want).norm() / want.norm()) < 1.2e-3
         assert float((lse - want_lse).abs().max()) < 2e-5
+
+
+@pytest.mark.parametrize("batch,gamma,q_heads,kv_heads,long_at", [(70, 5, 16, 8, (3, 40)), (33, 1, 8, 4, (32,)), (41, 5, 32, 4, (0, 20)), (300, 7, 16, 2, (150,)), (9, 7, 8, 1, (4,))])
+def test_a_few_long_contexts_among_very_short_ones(batch, gamma, q_heads, kv_heads, long_at):
+    """Cuts that fall inside a long pair, between pairs of one tile, and among the units that stand for a pair's set-up; one sequence
+    has no room for its block and is skipped."""
+    import paper_2505_10526_b200 as mv
+    lens = [b % 3 for b in range(batch)]
+    for i, b in enumerate(long_at):
+        lens[b] = 2500 + 700 * i
+    w = _inputs(batch, gamma, q_heads, kv_heads, lens, seed=batch)
+    full = batch // 2 + 3
+    capacity = w["page_table"].shape[1] * 16
+    want, want_lse = _reference(w, 0)
+    w["seq_lens"][full] = capacity - gamma                       # one position short of room
+    desc = mv.attn_desc(batch, gamma, q_heads, kv_heads, 256, w["page_table"].shape[1], w["k_pages"].shape[0])
+    ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda").fill_(0xff)
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    out = torch.full_like(w["q"], 7.0)
+    f32 = torch.full(out.shape, 7.0, device="cuda")
+    lse = torch.full(out.shape[:3], 7.0, device="cuda")
+    mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, lse, ws, status)
+    assert int(status.item()) == -3
+    assert bool((out[full] == 7.0).all()) and bool((f32[full] == 7.0).all())
+    rest = [b for b in range(batch) if b != full]
+    assert float(((f32 - want).norm(dim=-1) / want.norm(dim=-1))[rest].max()) < 4e-3        # 2^-8 per weight
+    assert float((lse - want_lse)[rest].abs().max()) < 2e-5
