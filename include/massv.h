@@ -159,6 +159,8 @@ size_t massv_accept_workspace_size(const massv_accept_desc *desc);
  * T == 0: draft j is accepted iff x equals argmax_v z_j[v] (lowest index on
  *   ties); the extra token is argmax_v z_n[v].  draft_probs, u_accept and
  *   u_sample are ignored and may be NULL.
+ * A row n without any logit above -inf (a hidden state that has gone NaN), and at T > 0 one whose
+ * probabilities are not numbers, yields token 0 and MASSV_ERR_INVALID_ARG in dev_status.
  *
  *   hidden        bf16 [B, R, K]
  *   lm_head       bf16 [V, K]

@@ -167,7 +167,10 @@ __global__ void __launch_bounds__(kScanThreads) accept_scan_kernel(AcceptParams 
     if (lane != 0) return;
     p.accept_len[b] = n + 1;
     if (greedy) {
-        toks[n] = row_stat[n].idx;
+        // (a row without a logit to compare, all of them NaN or -inf, has no index)
+        const int top = row_stat[n].idx;
+        if (top < 0 || top >= p.V) set_status(p.dev_status, MASSV_ERR_INVALID_ARG);
+        toks[n] = top >= 0 && top < p.V ? top : 0;
     } else {
         SeqState st;
         st.n = n;

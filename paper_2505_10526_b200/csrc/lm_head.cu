@@ -218,7 +218,7 @@ __device__ __forceinline__ void drain_chunk(const UmmaParams& p, uint32_t taddr,
 #pragma unroll
     for (int j = 0; j < C; ++j) {
         const float z = row_ok ? __uint_as_float(r[j]) + 0.f : -INFINITY;     // + 0 folds -0 into +0
-        const uint32_t key = float_key(z);
+        const uint32_t key = float_key(fmaxf(z, -INFINITY));                  // a NaN never wins (it still reaches the sum)
         const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
         const unsigned hit = __ballot_sync(0xffffffffu, key == kmax);
         const float mx = key_float(kmax);
