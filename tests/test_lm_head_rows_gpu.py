@@ -37,3 +37,29 @@ def test_rows(batch, gamma, vocab):
             assert torch.equal(tokens[:, :gamma], logits[:, :gamma].argmax(-1).to(torch.int32))
         else:
             assert float((probs.double() - torch.softmax(exact, -1)).abs().max()) < 1e-4
+
+
+@pytest.mark.parametrize("batch,gamma", [(1, 5), (16, 3), (16, 5), (40, 5), (50, 5), (100, 4)])        # 6, 64, 96, 240, 300, 500 token rows
+@pytest.mark.parametrize("std,shift,T", [(5.0, 0.0, 1.0), (5.0, 100.0, 1.0), (20.0, 0.0, 0.1), (5.0, -400.0, 0.3)])
+def test_sums_of_exponentials(batch, gamma, std, shift, T):
+    """The largest probability of a row is 1 / sum exp((z - max) / T), so its relative error is the sum's: terms of a few 2^-24 (one
+    product, one exponential), added 32 at a time, by tiles and by slots.  1.5e-6 is twice what a chain of a dozen fp32 sums gives."""
+    import paper_2505_10526_b200 as mv
+    K, R, vocab = 256, gamma + 1, 40008
+    g = torch.Generator(device="cuda").manual_seed(batch + gamma)
+    hidden = (std / 0.05 / 16.0 * torch.randn((batch, R, K), generator=g, device="cuda")).to(torch.bfloat16)
+    w = (0.05 * torch.randn((vocab, K), generator=g, device="cuda")).to(torch.bfloat16)
+    hidden[:, :, 0], w[:, 0] = shift, 1.0                   # every logit moved by the same amount
+    q = torch.full((batch, gamma, vocab), 1e-9, device="cuda")
+    desc = mv.accept_desc(batch, gamma, K, vocab, T)
+    ws = mv.alloc_workspace(mv.massv_accept_workspace_size(desc), "cuda")
+    logits, probs = torch.empty((batch, R, vocab), device="cuda"), torch.empty((batch, R, vocab), device="cuda")
+    tokens = torch.empty((batch, R), dtype=torch.int32, device="cuda"); lens = torch.empty((batch,), dtype=torch.int32, device="cuda")
+    mv.massv_accept(desc, hidden, w, torch.zeros((batch, gamma), dtype=torch.int32, device="cuda"), q, torch.full((batch, gamma), 0.5, device="cuda"),
+                    torch.full((batch, R), 0.5, device="cuda"), tokens, lens, logits, probs, ws, None)
+    worst = 0.0
+    for b in range(batch):
+        top = torch.softmax(logits[b].double() / T, dim=-1).max(-1).values
+        worst = max(worst, float((probs[b].max(-1).values.double() / top - 1).abs().max()))
+    print("worst", worst)
+    assert worst < 1.5e-6
