@@ -172,7 +172,8 @@ size_t massv_accept_workspace_size(const massv_accept_desc *desc);
  *   accept_len    int32 [B]: n + 1, the tokens gained by this target pass
  *                 (its batch mean is the paper's mean accepted length tau)
  *   logits_out    optional fp32 [B, R, V]: z
- *   probs_out     optional fp32 [B, R, V]: p (T > 0 only; must be NULL at T == 0)
+ *   probs_out     optional fp32 [B, R, V]: p (T > 0 only; must be NULL at T == 0); may be the buffer of
+ *                 logits_out, which then holds p when the call is through
  * Math: bf16 x bf16 products accumulated in fp32 on the tensor cores.
  */
 int massv_accept(const massv_accept_desc *desc, const void *hidden, const void *lm_head,

@@ -1007,7 +1007,8 @@ __global__ void shard_publish_kernel(PublishParams p) {
 // q).  One CTA per 4,096 entries of a row, four 16-byte loads in flight per thread; the row's statistics are the scan's.
 // It runs beside the persistent draw kernel: that one lets it start after its own wait, i.e. when the scan has completed, and
 // nothing here depends on the draw (so the results of earlier kernels are read past L1, and the wait at the end only keeps
-// this grid from completing before the draw).  Behind accept_row_kernel, which makes the statistics itself, it waits first.  What bounds it is HBM, 8 B per entry, where there are many rows; 16 rows of
+// this grid from completing before the draw).  Behind accept_row_kernel, which makes the statistics itself, it waits first, and so it
+// does where the distribution goes over the logits or the drafter's probabilities, which the draw reads.  What bounds it is HBM, 8 B per entry, where there are many rows; 16 rows of
 // 152,064: 23 us behind the draw with one 4-byte load per thread and iteration.
 constexpr int kProbsThreads = 256, kProbsGroups = 4, kProbsChunk = kProbsThreads * kProbsGroups * 4;
 __global__ void __launch_bounds__(kProbsThreads) probs_kernel(AcceptParams p, int wait_first) {
@@ -1078,6 +1079,11 @@ static int row_cluster(const AcceptParams& p) {
     return 0;
 }
 
+static bool overlaps(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + b_bytes && y < x + a_bytes;
+}
+
 cudaError_t launch_accept(const AcceptParams& p, cudaStream_t stream) {
     const TimingHooks& hooks = timing_hooks();
     const int c = p.T > 0.f ? row_cluster(p) : 0;
@@ -1111,7 +1117,9 @@ cudaError_t launch_accept(const AcceptParams& p, cudaStream_t stream) {
         if (hooks.residual_stop && cudaEventRecord(hooks.residual_stop, stream) != cudaSuccess) return cudaGetLastError();
         count_launches(1);
         if (p.probs_out) {
-            if (launch_pdl(probs_kernel, dim3((p.V + kProbsChunk - 1) / kProbsChunk, p.B * (p.gamma + 1)), dim3(kProbsThreads), 0, stream, p, 0) != cudaSuccess) return cudaGetLastError();
+            const size_t row = (size_t)p.V * sizeof(float), out_bytes = (size_t)p.B * (p.gamma + 1) * row;
+            const int wait_first = overlaps(p.probs_out, out_bytes, p.logits, out_bytes) || overlaps(p.probs_out, out_bytes, p.draft_probs, (size_t)p.B * p.gamma * row);
+            if (launch_pdl(probs_kernel, dim3((p.V + kProbsChunk - 1) / kProbsChunk, p.B * (p.gamma + 1)), dim3(kProbsThreads), 0, stream, p, wait_first) != cudaSuccess) return cudaGetLastError();
             count_launches(1);
         }
     }

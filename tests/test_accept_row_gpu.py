@@ -91,3 +91,27 @@ def test_no_residual_mass(vocab):
         cdf = torch.cumsum(p[b, 0], 0)
         tok = int(r["tokens"][b, 0])
         assert (float(cdf[tok - 1]) if tok else 0.0) - 2e-6 <= 0.4 <= float(cdf[tok]) + 2e-6
+
+
+@pytest.mark.parametrize("batch,gamma,vocab", [(3, 2, 10008), (5, 0, 50264), (300, 0, 4096), (128, 2, 65536), (150, 1, 32000)])
+def test_distribution_in_place_of_the_logits(batch, gamma, vocab):
+    """probs_out in the buffer of logits_out: the tokens are drawn before the row is overwritten."""
+    import paper_2505_10526_b200 as mv
+    K, R, T = 128, gamma + 1, 0.8
+    g = torch.Generator(device="cuda").manual_seed(vocab)
+    hidden = (20.0 * torch.randn((batch, R, K), generator=g, device="cuda")).to(torch.bfloat16)
+    w = (0.02 * torch.randn((vocab, K), generator=g, device="cuda")).to(torch.bfloat16)
+    q = torch.softmax(4.0 * torch.randn((batch, gamma, vocab), generator=g, device="cuda"), dim=-1).contiguous()
+    drafts = torch.randint(0, vocab, (batch, gamma), generator=g, device="cuda", dtype=torch.int32)
+    ua, us = torch.rand((batch, gamma), generator=g, device="cuda"), torch.rand((batch, R), generator=g, device="cuda")
+    desc = mv.accept_desc(batch, gamma, K, vocab, T)
+    ws = mv.alloc_workspace(mv.massv_accept_workspace_size(desc), "cuda")
+    res = []
+    for shared in (False, True, True):
+        logits = torch.empty((batch, R, vocab), device="cuda")
+        probs = logits if shared else torch.empty_like(logits)
+        tokens = torch.empty((batch, R), dtype=torch.int32, device="cuda"); lens = torch.empty((batch,), dtype=torch.int32, device="cuda")
+        mv.massv_accept(desc, hidden, w, drafts, q, ua, us, tokens, lens, logits, probs, ws, None)
+        res.append((tokens, lens, probs))
+    for other in res[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(res[0], other))
