@@ -790,8 +790,11 @@ template <int D, int MT, int TILE>
 cudaError_t launch_flat(const AttnParams& p, const CUtensorMap& mk, const CUtensorMap& mv, cudaStream_t stream, int* ctas) {
     using Cfg = FlatCfg<D, MT, TILE>;
     const size_t smem = (size_t)Cfg::kSmem + (size_t)(p.B + 1) * sizeof(int);
-    static_assert(Cfg::kSmem + (kFlatMaxBatchMeta + 1) * 4 <= 226 * 1024, "ring, query rows and tile counts fit shared memory");
-    cudaError_t e = cudaFuncSetAttribute(attn_flat_kernel<D, MT, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (The attribute is the process's, not the call's: every call sets the same bound, so that a small batch on one thread cannot
+    // lower it between another thread's attribute and launch.)
+    constexpr int kMaxSmem = Cfg::kSmem + (kFlatMaxBatchMeta + 1) * (int)sizeof(int);
+    static_assert(kMaxSmem <= 225 * 1024, "ring, query rows and tile counts fit shared memory");
+    cudaError_t e = cudaFuncSetAttribute(attn_flat_kernel<D, MT, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e != cudaSuccess) return e;
     *ctas = device_sm_count() * Cfg::kCtasPerSm;
     if (*ctas > kFlatMaxCtas) *ctas = kFlatMaxCtas;

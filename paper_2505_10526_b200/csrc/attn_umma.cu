@@ -875,7 +875,8 @@ cudaError_t launch_flat_combine(const AttnParams& p, int ctas, cudaStream_t stre
     while (parts < 16 && units_per_qd / (parts * 2) >= 32 && pairs * n_qd * parts < 2 * flat_sm_count()) parts *= 2;
     // (max, sum) and weight of 16 rows for at most `ctas` pieces of a pair (a pair can span every CTA)
     const size_t comb_smem = (2 * (size_t)ctas + 1) * 16 * sizeof(float) + kFlatCombineThreads * sizeof(float4);
-    const cudaError_t e = cudaFuncSetAttribute(attn_flat_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)comb_smem);
+    constexpr int kMaxSmem = (2 * kFlatMaxCtas + 1) * 16 * (int)sizeof(float) + kFlatCombineThreads * (int)sizeof(float4);      // the same bound on every call
+    const cudaError_t e = cudaFuncSetAttribute(attn_flat_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e != cudaSuccess) return e;
     return launch_pdl(attn_flat_combine_kernel, dim3(pairs, n_qd * parts), dim3(kFlatCombineThreads), comb_smem, stream, p, rows_pad, parts,
                       units_per_qd / parts);

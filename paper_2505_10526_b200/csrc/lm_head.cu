@@ -35,6 +35,7 @@ constexpr int kTileBytesW = kVocabTile * kBlockK * 2;
 constexpr int kMaxStages = 12;
 constexpr int kMaxCtas = 192;               // partial slots are sized for at most this many CTAs
 constexpr int kRingBytes = 200 * 1024;      // shared memory given to the TMA ring
+constexpr int kMaxRingSmem = kRingBytes + 1024;   // (the kernels' attribute: one bound for every call, whatever its ring takes, since it is the process's)
 constexpr int kPrefetchBlocks = 32;         // K blocks (16 KB each) of the first tile hinted into L2 before the dependency wait
 constexpr int kPairMinTile = 64;            // token rows per tile from which CTA pairs are used
 
@@ -933,7 +934,7 @@ static cudaError_t launch_lm_head_duo(const LmHeadParams& q, UmmaParams p, int c
     const size_t smem = (size_t)stages * stage_bytes + 1024;
     const TimingHooks& hooks = timing_hooks();
     if (hooks.lm_head_start && cudaEventRecord(hooks.lm_head_start, stream) != cudaSuccess) return cudaGetLastError();
-    cudaError_t e = cudaFuncSetAttribute(lm_head_duo_kernel<PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(lm_head_duo_kernel<PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRingSmem);
     if (e != cudaSuccess) return e;
     e = launch_pdl_cluster(lm_head_duo_kernel<PARTS>, dim3(groups * 2), dim3(Cfg::kThreads), smem, stream, 2, map_w, map_h, p);
     if (e != cudaSuccess) return e;
@@ -1000,12 +1001,12 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     const TimingHooks& hooks = timing_hooks();
     if (hooks.lm_head_start && cudaEventRecord(hooks.lm_head_start, stream) != cudaSuccess) return cudaGetLastError();
     if (pair) {
-        e = cudaFuncSetAttribute(lm_head_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(lm_head_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRingSmem);
         if (e != cudaSuccess) return e;
         e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * 2), dim3(lm_head_threads(true)), smem, stream, 2,
                                map_w[0], map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
     } else {
-        e = cudaFuncSetAttribute(lm_head_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(lm_head_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRingSmem);
         if (e != cudaSuccess) return e;
         e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups), dim3(lm_head_threads(false)), smem, stream, map_w[0],
                        map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
