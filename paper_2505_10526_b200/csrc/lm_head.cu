@@ -26,8 +26,8 @@ namespace massv {
 
 namespace {
 
-// Epilogue warps: two per TMEM lane quarter for single-CTA tiles (16 columns at a time), four for CTA pairs (64 columns each,
-// so that the epilogue of a 256-row tile keeps up with short K loops too).
+// Epilogue warps: two per TMEM lane quarter for single-CTA tiles (16 columns at a time), four for CTA pairs (64 columns each, 16
+// up to 64 rows, so that the epilogue keeps up with short K loops too).
 __host__ __device__ constexpr int epilogue_warps(bool pair) { return pair ? 16 : 8; }
 __host__ __device__ constexpr int lm_head_threads(bool pair) { return (2 + epilogue_warps(pair)) * 32; }
 constexpr int kBlockK = 64;                 // bf16 elements per 128-byte swizzled row
@@ -584,7 +584,9 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
         // ------------------------------------------------ epilogue
         // TMEM lanes 32*quarter .. +31 are the only ones warp (quarter = warp % 4) may read.  Pairs: the four warps of a
         // quarter take 64 columns each, copy them to registers and give the accumulator back before they compute.
-        // Single CTAs (tiles of up to 48 columns): the two warps of a quarter take alternate chunks of 16 columns.
+        // Tiles of up to 64 columns: the warps of a quarter (two in single CTAs, four in pairs) take chunks of 16 columns in turn.
+        // One job of 64 columns would leave three warps of four idle, and short K loops waited for the fourth (64 rows of
+        // hidden size 1,024, vocabulary 152,064, T = 1: 86 us with chunks of 32 by two warps, 94 with one job, 86 here; of 512: 78, 90, 71).
         const int quarter = warp & 3;
         const int part = (warp - 2) >> 2;
         // running statistics per (quarter, column); each column is touched by exactly one lane of one warp
@@ -601,7 +603,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
             tile.v0 = row_begin + t * tile_rows + (int)pair_rank * kVocabTile;     // this CTA's 128 rows
             tile.rows = max(0, min(kVocabTile, row_end - tile.v0));
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.tmem_cols / 2);
-            if constexpr (PAIR) {
+            if (PAIR && p.n_tile > 64) {
                 const int c0 = part * 64, n_cols = min(64, p.n_tile - c0);
                 uint32_t va[32], vb[32];
                 if (n_cols > 0) {                                  // the same in every lane
@@ -616,7 +618,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                 if (n_cols > 0)
                     stats_job64(p, va, vb, lane, quarter, tile, c0, n_cols, &run_m[quarter][c0], &run_s[quarter][c0], &run_i[quarter][c0]);
             } else {
-                for (int c0 = part * 16; c0 < p.n_tile; c0 += 32) {
+                for (int c0 = part * 16; c0 < p.n_tile; c0 += kEpilogueWarps * 4) {
                     // lanes 2c and 2c+1 both end up with column c of the 16; the even lane keeps it
                     const int col = c0 + (lane >> 1);
                     Stat running{run_m[quarter][col], run_s[quarter][col], run_i[quarter][col]};
@@ -627,7 +629,10 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&tmem_empty_bar[buf]);
+                if (lane == 0) {
+                    if constexpr (PAIR) mbar_arrive_at(cluster_addr(&tmem_empty_bar[buf], 0));
+                    else mbar_arrive(&tmem_empty_bar[buf]);
+                }
             }
         }
     }
