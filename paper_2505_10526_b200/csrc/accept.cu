@@ -1067,13 +1067,16 @@ __global__ void kv_commit_kernel(int B, int gamma, const int32_t* accept_len, in
 }  // namespace
 
 // CTAs per sequence of accept_row_kernel, 0 where it does not apply.  All clusters have to be resident at once: a second wave
-// would repeat the whole latency chain, where the persistent draw kernel overlaps its sequences.
+// would repeat the whole latency chain, where the persistent draw kernel overlaps its sequences.  A cluster needs its places
+// inside one group of SMs: 148 SMs hold 33 clusters of eight with two CTAs to an SM and 15 with one.  The limits stay a few
+// clusters below that, since the kernel ahead may still hold SMs, and go with the device's SMs.
 static int row_cluster(const AcceptParams& p) {
+    const long sms = device_sm_count();
     for (int c = kRowMaxCluster; c >= 1; c /= 2) {
         if (c > 1 && p.V < c * 2048) continue;
         const long bytes = ((long)(p.V + c - 1) / c + 256) * 4;
         if (bytes > kRowMaxBytes) break;
-        const long slots = bytes <= kRowPairBytes ? 224 : 96;
+        const long slots = (bytes <= kRowPairBytes ? 28 : 12) * 8 * sms / 148;
         if ((long)p.B * c <= slots) return c;
     }
     return 0;

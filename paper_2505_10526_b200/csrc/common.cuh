@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "massv.h"
 
 namespace massv {
@@ -100,11 +102,15 @@ TimingHooks& timing_hooks();
 // Host-side tally of kernel launches (see massv_launch_count).
 void count_launches(int n);
 
-// Multiprocessors of the current device (148 on B200).
+// Multiprocessors of the current device (148 on B200), asked for once per device.
 inline int device_sm_count() {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
     int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-        n = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+    if (dev < kDevices && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+    if (dev < kDevices) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
