@@ -7,10 +7,11 @@
 A step is one whole verify step (massv_verify_attn + massv_accept +
 massv_kv_commit) on one batch of a synthetic workload.  The default workload is
 the long-context Qwen2.5-VL-7B-shaped batch of 64 sequences at gamma = 5, T = 1
-(the paper's inference settings); the JSON line rank 0 prints also carries a
-`sweep` with one entry per other workload of the table (batch 1, batch 16, the
-Gemma3-12B shape, the other long-context points), each with its breakdown and a
-roofline block per dominant kernel.  With N > 1 every rank runs an independent
+(the paper's inference settings).  Rank 0 prints one JSON line with the headline
+to stdout, last, and short enough to survive in a log's tail; ahead of it, on
+stderr, one JSON line per workload with its breakdown and a roofline block per
+dominant kernel: the default workload, then a sweep over the others of the table
+(batch 1, batch 16, the Gemma3-12B shape, the other long-context points).  With N > 1 every rank runs an independent
 replica of the workload on its own GPU (the path has no cross-GPU exchange), so
 scaling is weak.
 
@@ -44,16 +45,15 @@ MIN_SPLIT_STEPS = 5
 
 # DRAM traffic of one launch of a kernel over its algorithmic bytes (dram__bytes_read.sum +
 # dram__bytes_write.sum of an ncu capture, summarised under profiles/), keyed by (kernel, shape
-# family).  Captures of the long-context attention kernel are taken at batch 16 (a few GB on the
-# device) and scaled by the K/V bytes of the launch: the kernel streams every K/V byte once, so its
-# traffic grows in proportion.  None: no capture of the kernel as it stands.
+# family).  Captures of the attention kernels are taken at smaller batches (a few GB on the
+# device) and scaled by the K/V bytes of the launch: the kernels stream every K/V byte once, so their
+# traffic grows in proportion.  A kernel without a capture of its own has no entry and reports None.
 NCU_TRAFFIC_RATIO = {
-    ("attn", "qwen"): (693.56 + 5.1) / 691.5,  # profiles/attn_umma_kernel_qwen7b_long_b16.md (batch 16, scaled by K/V bytes)
-    ("attn", "gemma"): 1.384 / 1.34,          # profiles/attn_split_kernel_gemma12b_b32_t1.md (read 1.378 GB + 6.2 MB written)
-    ("lm_head", "qwen"): 1.0934 / 1.0900,     # profiles/lm_head_umma_kernel_qwen7b_b1_t0.md (the weight-bound launches, M <= 256)
-    ("lm_head", "gemma"): (2.04619 + 0.14287) / 2.01474,   # profiles/lm_head_umma_kernel_gemma12b_b32_t1.md (weights once + the fp32 logits that left L2)
-    ("residual", "qwen"): (74.30 + 1.35) / 77.86,   # profiles/residual_sample_kernel_qwen7b_lmhead_g5_t1.md
-    ("residual", "gemma"): (62.99 + 0.08) / 67.11,    # profiles/lm_head_umma_kernel_gemma12b_b32_t1.md (second table)
+    ("attn_umma_kernel", "qwen"): (693.56 + 5.1) / 691.5,  # profiles/attn_umma_kernel_qwen7b_long_b16.md (batch 16, scaled by K/V bytes)
+    ("lm_head_umma_kernel", "qwen"): 1.0934 / 1.0900,     # profiles/lm_head_umma_kernel_qwen7b_b1_t0.md (the weight-bound launches, M <= 256)
+    ("lm_head_umma_kernel", "gemma"): (2.04619 + 0.14287) / 2.01474,   # profiles/lm_head_umma_kernel_gemma12b_b32_t1.md (weights once + the fp32 logits that left L2)
+    ("residual_sample_kernel", "qwen"): (74.30 + 1.35) / 77.86,   # profiles/residual_sample_kernel_qwen7b_lmhead_g5_t1.md
+    ("residual_sample_kernel", "gemma"): (62.99 + 0.08) / 67.11,    # profiles/lm_head_umma_kernel_gemma12b_b32_t1.md (second table)
 }
 
 
@@ -172,13 +172,22 @@ class ClockSampler:
                 "reasons": sorted(name for bit, name in self.REASONS.items() if bits & bit)}
 
 
+def short_numbers(x):
+    """Floats to seven significant digits, so that the headline stays one short line."""
+    if isinstance(x, float):
+        return float(f"{x:.7g}")
+    if isinstance(x, dict):
+        return {k: short_numbers(v) for k, v in x.items()}
+    return [short_numbers(v) for v in x] if isinstance(x, list) else x
+
+
 def config_block(cfg, mean_context, attn_kernel, world):
     """The `config` object of the JSON line; both arms print the same keys for the same workload."""
     return {"workload": cfg.name, "batch": cfg.batch, "gamma": cfg.gamma, "temperature": cfg.temperature,
             "n_q_heads": cfg.n_q_heads, "n_kv_heads": cfg.n_kv_heads, "head_dim": cfg.head_dim,
             "hidden": cfg.hidden, "vocab": cfg.vocab, "mean_context": float(mean_context),
             "attn_kernel": {0: "by shape", 1: "warp_mma", 2: "tcgen05"}[attn_kernel],
-            "l2": f"flushed between timed steps by a {L2_FLUSH_BYTES >> 20} MiB write; K/V and LM-head weights exceed L2 anyway",
+            "l2": f"flushed between timed steps ({L2_FLUSH_BYTES >> 20} MiB write)",
             "parallelism": f"replicas x{world}"}
 
 
@@ -267,9 +276,7 @@ def roofline_block(kernel, bound, algorithmic, ms, peaks, peak_src, family):
          "ms_per_launch_best": ms["best"]}
     if bound == "tensor" and peaks.get("bf16_tflops_sustained"):
         r["frac_of_sustained"] = achieved / peaks["bf16_tflops_sustained"]
-    key = {"attn_umma_kernel": "attn", "attn_split_kernel": "attn", "attn_flat_kernel": "attn", "accept_row_kernel": "residual", "lm_head_umma_kernel": "lm_head", "lm_head_duo_kernel": "lm_head",
-           "residual_sample_kernel": "residual"}[kernel]
-    ratio = NCU_TRAFFIC_RATIO.get((key, family))
+    ratio = NCU_TRAFFIC_RATIO.get((kernel, family))
     r["traffic"] = None if (ratio is None or bound == "tensor") else ratio * algorithmic
     return r
 
@@ -341,6 +348,9 @@ def measure(mv, cfg, dev, K, W, attn_kernel, peaks, peak_src, world, sampler=Non
     period = max(2, K // MIN_SPLIT_STEPS)
     is_split = [CALLS if i % period == 0 else KERNELS if i % period == 1 else PLAIN for i in range(K)]
     events = [new_events(n_ev if is_split[i] == KERNELS else 4) for i in range(K)]
+    before = mv.massv_launch_count()
+    step.accept(w)
+    accept_launches = mv.massv_launch_count() - before
     launches0 = mv.massv_launch_count()
     barrier()
     torch.cuda.synchronize()
@@ -376,7 +386,9 @@ def measure(mv, cfg, dev, K, W, attn_kernel, peaks, peak_src, world, sampler=Non
     lm_flops = 2.0 * cfg.m * cfg.vocab * cfg.hidden
     attn_bytes = kv_bytes(cfg, seq0.tolist())
     ridge = peaks["bf16_tflops"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
-    attn_name = "attn_umma_kernel" if (attn_kernel == 2 or (attn_kernel == 0 and cfg.head_dim <= 128)) else "attn_flat_kernel"
+    # (the workloads' page tables hold more than one chunk: at head_dim 256 the balanced schedule runs)
+    attn_name = ("attn_umma_kernel" if attn_kernel == 2 or (attn_kernel == 0 and cfg.head_dim <= 128)
+                 else "attn_flat_kernel" if cfg.head_dim == 256 else "attn_split_kernel")
     rl = {"attn": roofline_block(attn_name, "hbm", attn_bytes, t_attn_k, peaks, peak_src, family),
           # more than 256 token rows take the one-pass kernel (two sub-tiles of the rows in tensor memory at once)
           "lm_head": roofline_block("lm_head_duo_kernel" if cfg.m > 256 else "lm_head_umma_kernel", "tensor" if cfg.m > ridge else "hbm",
@@ -385,9 +397,9 @@ def measure(mv, cfg, dev, K, W, attn_kernel, peaks, peak_src, world, sampler=Non
     rl["lm_head"]["frac_whole_accept_call"] = rl["lm_head"]["algorithmic"] / (t_accept["mean"] * 1e-3) / \
         (1e12 if cfg.m > ridge else 1e9) / rl["lm_head"]["peak"]
     if sampling:
-        # few sequences: the accept tests and the draw are one launch (accept_row_kernel), timed as a whole
-        one_launch = cfg.batch * 8 <= (224 if cfg.vocab <= 8 * 26880 else 96)
-        rl["residual"] = roofline_block("accept_row_kernel" if one_launch else "residual_sample_kernel", "hbm", cfg.batch * cfg.vocab * 8, t_res, peaks, peak_src, family)
+        # few sequences: the accept tests and the draw are one launch (accept_row_kernel), timed as a whole; an acceptance call is then
+        # that and the LM head, otherwise the scan stands between them
+        rl["residual"] = roofline_block("accept_row_kernel" if accept_launches == 2 else "residual_sample_kernel", "hbm", cfg.batch * cfg.vocab * 8, t_res, peaks, peak_src, family)
     shares = {"attn": t_attn_k["mean"], "lm_head": t_lm["mean"]}
     if sampling:
         shares["residual"] = t_res["mean"]
@@ -599,30 +611,28 @@ def main():
             dist.destroy_process_group()
         return
 
+    for e in [main_e] + sweep:
+        print(json.dumps(e), file=sys.stderr, flush=True)
     dom = main_e["dominant"]
-    roofline = dict(main_e["rooflines"][dom])
+    roofline = {k: main_e["rooflines"][dom][k] for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source", "algorithmic",
+                                                         "ms_per_launch", "traffic")}
     roofline["share_of_step"] = main_e["share_of_step"][dom]
+    e2e = lambda e: {k: e[k] for k in ("value", "unit", "ms_per_step", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps")}
     line = {
         "metric": METRIC, "value": main_e["value"], "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
         "ms_per_step": main_e["ms_per_step"], "ms_per_step_median": main_e["ms_per_step_median"],
         "ms_per_step_best": main_e["ms_per_step_best"], "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
         "config": config_block(cfg, main_e["mean_context"], args.attn_kernel, world),
-        "breakdown_ms": main_e["breakdown_ms"], "mean_accept_len": main_e["mean_accept_len"],
-        "roofline": roofline, "rooflines": main_e["rooflines"], "clocks": clocks,
-        "e2e": main_e["e2e"], "e2e_q_resident": main_e["e2e_q_resident"],
-        "gpu_launches": main_e["gpu_launches"], "wall_s_timed_region": main_e["wall_s_timed_region"],
+        "roofline": roofline, "clocks": {k: clocks[k] for k in ("sm_mhz", "sm_max_mhz", "reasons", "samples")},
+        "e2e": e2e(main_e["e2e"]), "e2e_q_resident": e2e(main_e["e2e_q_resident"]), "gpu_launches": main_e["gpu_launches"],
     }
-    if "tvd" in main_e:
-        line["tvd"] = main_e["tvd"]
     if cpu_w is not None:
         sub_cfg, w_cpu, keep = cpu_w
         v, t, reps, cores = time_oracle(sub_cfg, w_cpu)
         line["cpu_baseline"] = {"value": v, "unit": UNIT, "cores": cores, "kind": "oracle",
-                                "sample": f"first {keep} of {cfg.batch} sequences of {cfg.name}, whole verify step, best of {reps} ({t:.2f} s)"}
-    if sweep:
-        line["sweep"] = sweep
-    print(json.dumps(line), flush=True)
+                                "sample": f"first {keep} of {cfg.batch} sequences, whole step, best of {reps} ({t:.2f} s)"}
+    print(json.dumps(short_numbers(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 

@@ -94,3 +94,29 @@ def test_rows_without_a_finite_logit():
     mv.massv_sample_top_p(z, torch.full((5,), 0.5, device="cuda"), tok, 1.0, 0.9, None, status)
     torch.cuda.synchronize()
     assert int(status.item()) == -1 and int(tok[3]) == 0 and int(tok.min()) >= 0
+
+
+@pytest.mark.parametrize("vocab", [8192, 50264, 152064])
+def test_rows_come_out_the_same_in_calls_of_any_size(vocab):
+    """The number of rows decides how many CTAs share a row, and with it the grouping of the fp64 sums: the set of tokens is exact (integer
+    masses), the normalisation may differ in its last bit, and a draw only where u falls on a step of the CDF."""
+    import paper_2505_10526_b200 as mv
+    g = torch.Generator(device="cuda").manual_seed(vocab)
+    z = 4.0 * torch.randn((150, vocab), generator=g, device="cuda")
+    u = torch.rand((150,), generator=g, device="cuda")
+
+    def run(rows, top_p):
+        tok, q = torch.empty((rows,), dtype=torch.int32, device="cuda"), torch.empty((rows, vocab), device="cuda")
+        mv.massv_sample_top_p(z[:rows], u[:rows], tok, 0.9, top_p, q, None)
+        return tok, q
+
+    for top_p in (0.8, 1.0):
+        tok, q = run(150, top_p)
+        for rows in (1, 5, 16, 40, 90):
+            t, p = run(rows, top_p)
+            assert torch.equal(p > 0, q[:rows] > 0)
+            assert float(((p - q[:rows]).abs() / q[:rows].clamp_min(1e-30)).max()) <= 2.0 ** -22
+            cdf = torch.cumsum(q[:rows].double(), -1)
+            at = t.long().clamp_min(1)
+            gap = torch.minimum((cdf.gather(-1, t.long()[:, None])[:, 0] - u[:rows]).abs(), (cdf.gather(-1, (at - 1)[:, None])[:, 0] - u[:rows]).abs())
+            assert bool(((t == tok[:rows]) | (gap < 1e-6)).all())
