@@ -351,14 +351,6 @@ __device__ __forceinline__ void walk_chunk_masses(const double* s, int n, double
     }
 }
 
-// (No eviction hint: the chunk that turns out to hold the drawn token is read a second time, and should then
-// still be in L2.)
-__device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)), "l"(src),
-                 "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
 // The sequential part of the draw for one sequence, by the 256 threads of warps 0-7: walk the chunk masses
 // (fixed summation order), then find the token inside the winning chunk.
 __device__ void draw_from_chunk_masses(const AcceptParams& p, int b, const SeqState& st, float inv_T, double* warp_sums, double* s_sums,
@@ -636,6 +628,7 @@ __global__ void __launch_bounds__(kResidualThreads, kResidualCtasPerSm) residual
                     const SeqState st = state_of(b);
                     const uint32_t bytes = (uint32_t)min(kResidualChunk, p.V - c * kResidualChunk) * 4u;
                     uint8_t* dst = res_smem + (size_t)s * kStageBytes;
+                    // (no eviction hint: the chunk that turns out to hold the drawn token is read a second time, and should then still be in L2)
                     mbar_expect_tx(&full_bar[s], st.use_q ? 2 * bytes : bytes);
                     bulk_load_1d(dst, p.logits + (size_t)(b * R + st.n) * p.V + (size_t)c * kResidualChunk, bytes, &full_bar[s]);
                     if (st.use_q)

@@ -807,7 +807,7 @@ lm_head_duo_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_co
             }
         }
     } else {
-        // ------------------------------------------------ epilogue (warps 2..13)
+        // ------------------------------------------------ epilogue (warps 2 .. 4 * PARTS + 1)
         // TMEM lanes 32*quarter .. +31 are the only ones warp (quarter = warp % 4) may read; the PARTS warps
         // of a quarter take columns 64*part .. 64*part+63 of both sub-tiles.
         const int quarter = warp & 3;

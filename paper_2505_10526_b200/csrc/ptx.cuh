@@ -64,6 +64,17 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
     asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 
+// Plain 1-D copies into shared memory, without an eviction hint: by the bulk engine (16-byte multiples, signalled on an mbarrier)
+// and by the calling thread.
+__device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
 // ---- a row held by the CTAs of one cluster (1 .. 16): barrier of all their threads, loads from a peer's shared memory
 __device__ __forceinline__ void row_barrier(int n_ctas) {        // all threads of the row's CTAs
     if (n_ctas == 1) { __syncthreads(); return; }

@@ -22,12 +22,6 @@ __device__ __forceinline__ const float* logits_row(const TvdParams& p, int row) 
     return p.logits + (size_t)(b * (p.gamma + 1) + j) * p.V;
 }
 
-// (No eviction hint.)
-__device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)), "l"(src),
-                 "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
 __device__ __forceinline__ void bulk_load_1d_hint(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t policy) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(smem_u32(dst)),
                  "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
@@ -277,10 +271,6 @@ constexpr int kRowMaxCluster = 16;
 constexpr int kRowRegGroups = 10;                    // groups of four drafter probabilities a thread holds in registers
 constexpr int kRowSlice = kRowRegGroups * 4 * kRowThreads;      // entries per CTA up to which they are all there is
 constexpr int kRowMaxSlice = 25 * 1024;              // 100 KB of logits: still two CTAs to an SM
-
-__device__ __forceinline__ void cp_async_16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
 
 struct RowPublished {
     float m;            // maximum of the slice

@@ -1,5 +1,6 @@
-"""The balanced schedule of the warp-MMA kernel at head_dim 256: pairs cut between CTAs and ranges of several pairs, every
-number of row groups, windows, lengths from zero, ragged ends, against attention in fp32 on the same bf16 values."""
+"""The warp-MMA kernel at head_dim 256, its balanced schedule (pairs cut between CTAs, ranges of several pairs, every number of row
+groups, windows) and the chunk grid where the rule keeps it; lengths from zero, ragged ends; against attention in 64 bits on the
+same bf16 values."""
 import math
 
 import pytest
@@ -66,9 +67,11 @@ def test_against_fp32(batch, gamma, q_heads, kv_heads, lo, hi, window):
     out, f32, lse = run()
     again = run()
     assert int(status.item()) == 0
-    # softmax weights carry bf16's 2^-9; values of a few units, weights that sum to one: 5e-3 of the fp32 output, bf16 on top of it
+    # softmax weights carry bf16's rounding, at most 2^-8 each: 4e-3 of a row's norm for independent values, and another 2^-8 for the
+    # bf16 output; the weights' sum is taken before the rounding.  (One position of 9,000 too many or too few is 1e-4 of the sum.)
     assert float((f32 - want).abs().max()) < 1e-2 and float((out.float() - want).abs().max()) < 3e-2
-    assert float((lse - want_lse).abs().max()) < 1e-3
+    assert float(((f32 - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 4e-3 and float(((out.float() - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 8e-3
+    assert float((lse - want_lse).abs().max()) < 2e-5
     assert all(torch.equal(a, b) for a, b in zip((out, f32, lse), again))
     for b, n in enumerate(lens):                          # the block's rows are in their slots
         for j in range(gamma + 1):
