@@ -50,6 +50,8 @@ MIN_SPLIT_STEPS = 5
 # traffic grows in proportion.  A kernel without a capture of its own has no entry and reports None.
 NCU_TRAFFIC_RATIO = {
     ("attn_umma_kernel", "qwen"): (693.56 + 5.1) / 691.5,  # profiles/attn_umma_kernel_qwen7b_long_b16.md (batch 16, scaled by K/V bytes)
+    ("attn_flat_kernel", "gemma"): (623.17 + 3.19) / 620.16,      # profiles/cluster_and_stream_kernels.md (batch 16, scaled by K/V bytes)
+    ("accept_row_kernel", "qwen"): 19.08 / 19.46,                  # profiles/cluster_and_stream_kernels.md (16 sequences, gamma 5)
     ("lm_head_umma_kernel", "qwen"): 1.0934 / 1.0900,     # profiles/lm_head_umma_kernel_qwen7b_b1_t0.md (the weight-bound launches, M <= 256)
     ("lm_head_umma_kernel", "gemma"): (2.04619 + 0.14287) / 2.01474,   # profiles/lm_head_umma_kernel_gemma12b_b32_t1.md (weights once + the fp32 logits that left L2)
     ("residual_sample_kernel", "qwen"): (74.30 + 1.35) / 77.86,   # profiles/residual_sample_kernel_qwen7b_lmhead_g5_t1.md

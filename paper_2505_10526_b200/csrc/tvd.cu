@@ -35,8 +35,8 @@ __device__ __forceinline__ void bulk_load_1d_hint(void* dst, const void* src, ui
 // warp keeps a ring of steps filled with bulk copies (two groups of four entries per consumer thread and step), so the
 // bytes in flight do not depend on what the consumers do.  The second pass walks the rows last to first: the statistics
 // pass has left the last logits in L2, and the drafter's rows pass through without displacing them.  64 x 5 rows of
-// 152,064: 130 us with a grid of (slice, row) CTAs and one 16-byte load per thread and iteration, 103 us here (44 us for
-// the first pass, 56 us for the second).
+// 152,064, calls back to back: 136 us with a grid of (slice, row) CTAs and one 16-byte load per thread and iteration, 112 us
+// here (44 - 49 us of it the first pass).
 constexpr int kStreamWarps = 24;                             // consumers
 constexpr int kStreamConsumers = kStreamWarps * 32, kStreamThreads = kStreamConsumers + 32;
 constexpr int kStepGroups = 2;
