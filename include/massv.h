@@ -239,7 +239,7 @@ size_t massv_tvd_workspace_size(const massv_accept_desc *desc);
  *   draft_probs   fp32 [B, gamma, V]
  *   tvd_out       fp32 [B, gamma];  accept_prob_out  optional fp32 [B, gamma]
  * Needs T > 0 and gamma >= 1.  Reads every drafted row once (B*gamma*V*8 bytes), the
- * logits of many rows a second time; sums run in fp64 in a fixed order.
+ * logits of many rows a second time; sums run in fp64 in an order that the descriptor fixes.
  */
 int massv_tvd(const massv_accept_desc *desc, const float *logits, const float *draft_probs,
               float *tvd_out, float *accept_prob_out,
@@ -299,7 +299,9 @@ int massv_tvd_histogram(int64_t n, const float *tvd, int32_t bins, int64_t *coun
  *   u             fp32 [rows], uniforms in [0, 1) supplied by the caller
  *   tokens        int32 [rows]
  *   probs_out     optional fp32 [rows, vocab]: q, zeros outside the nucleus
- * Math: weights exp((z - max) / T) in fp32, all sums in fp64 in a fixed order.  No workspace.  A row
+ * Math: weights exp((z - max) / T) in fp32, masses that decide the nucleus as exact integers, other sums in fp64 in an
+ * order that `rows` and `vocab` fix (calls repeat bit for bit; the same row among another number of rows may
+ * differ in the last bit of probs_out).  No workspace.  A row
  * without a finite logit stores MASSV_ERR_INVALID_ARG in dev_status and token 0.
  */
 int massv_sample_top_p(int32_t rows, int32_t vocab, float temperature, float top_p, const float *logits,
