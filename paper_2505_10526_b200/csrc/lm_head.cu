@@ -36,6 +36,13 @@ constexpr int kMaxStages = 12;
 constexpr int kMaxCtas = 192;               // partial slots are sized for at most this many CTAs
 constexpr int kRingBytes = 200 * 1024;      // shared memory given to the TMA ring
 constexpr int kMaxRingSmem = kRingBytes + 1024;   // (the kernels' attribute: one bound for every call, whatever its ring takes, since it is the process's)
+// K blocks that a ring stage of lm_head_umma_kernel holds.  With one, the two threads that copy and issue spend about 390
+// and 480 cycles a block besides their waits, more than a block takes to arrive, and every copy touches 128 bytes of a
+// weight row; two per copy halve the turns of both loops and read 256 adjacent bytes.  One -> two blocks, a call of
+// massv_accept at T = 0: vocabulary 152,064, hidden 3,584, 6 rows 173 -> 157 us (6.96 TB/s of weights), 128 rows 191 -> 171,
+// 256 rows 231 -> 221; hidden 1,024, 6 rows 72 -> 57; 262,144 x 3,840, 192 rows 412 -> 371.  Four (64 KB of weights per stage)
+// leave too few stages from 32 rows up (28 rows: 189 -> 193) and bring nothing below.
+constexpr int kStageBlocks = 2;
 constexpr int kPrefetchBlocks = 32;         // K blocks (16 KB each) of the first tile hinted into L2 before the dependency wait
 constexpr int kPairMinTile = 64;            // token rows per tile from which CTA pairs are used
 
@@ -54,7 +61,7 @@ struct UmmaParams {
     int n_part = 0;      // partial slots behind part_max / part_sum / part_idx (the debug build checks the slot index)
     int32_t* dev_status;
     int idx_offset;      // added to the argmax indices that leave the kernel
-    int test_skip_stage = 0;   // test builds only: withhold the second K block of the first tile
+    int test_skip_stage = 0;   // test builds only: withhold the last stage of the first tile
     int n_bands = 0;     // duo kernel: 256-row vocabulary bands in all
     int split_rem = 0;   // duo kernel: bands left over after tiles_per_group per pair, each cut in two half-tiles (one sub-tile each)
 };
@@ -86,6 +93,26 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
         " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
         "l"(map), "r"(x), "r"(y), "r"(bar_cluster_addr), "l"(policy)
         : "memory");
+}
+// The same for a box of several K blocks of a matrix seen as [K / 64][rows][64].
+__device__ __forceinline__ void tma_load_blocks_pair(void* dst, const CUtensorMap* map, int row, int block, uint32_t bar_cluster_addr,
+                                                     uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(0), "r"(row), "r"(block), "r"(bar_cluster_addr), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_blocks(void* dst, const CUtensorMap* map, int row, int block, uint64_t* bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(0), "r"(row), "r"(block), "r"(smem_u32(bar)), "l"(policy)
+        : "memory");
+}
+// A hint to bring such a box into L2; nothing waits on it and nothing in shared memory changes.
+__device__ __forceinline__ void tma_prefetch_blocks(const CUtensorMap* map, int row, int block) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(0), "r"(row), "r"(block) : "memory");
 }
 template <bool ACC>
 __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
@@ -402,10 +429,7 @@ __device__ __forceinline__ void stats_job64(const UmmaParams& p, uint32_t (&va)[
 // hidden-state traffic per weight byte compared with one CTA per 128 rows.
 template <bool PAIR>
 __global__ void __launch_bounds__(lm_head_threads(PAIR), 1)
-lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_constant__ CUtensorMap map_w64,
-                    const __grid_constant__ CUtensorMap map_w32, const __grid_constant__ CUtensorMap map_w16,
-                    const __grid_constant__ CUtensorMap map_w8, const __grid_constant__ CUtensorMap map_h,
-                    const UmmaParams p) {
+lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_h, const UmmaParams p) {
     constexpr int kEpilogueWarps = epilogue_warps(PAIR), kThreads = lm_head_threads(PAIR);
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages];
@@ -414,14 +438,16 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
     __shared__ __align__(8) uint64_t tmem_empty_bar[2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
-    __shared__ float run_m[4][256];
-    __shared__ float run_s[4][256];
-    __shared__ int run_i[4][256];
+    constexpr int kCols = PAIR ? 256 : kPairMinTile;           // token rows per tile at most; kept small, so that CTAs of the acceptance kernels fit beside this one
+    __shared__ float run_m[4][kCols];
+    __shared__ float run_s[4][kCols];
+    __shared__ int run_i[4][kCols];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int h_rows = PAIR ? p.n_tile / 2 : p.n_tile;       // hidden-state rows this CTA loads per K block
-    const int stage_bytes = kTileBytesW + h_rows * 128;
+    const int h_bytes = h_rows * 128;
+    const int stage_bytes = kStageBlocks * (kTileBytesW + h_bytes);      // the stage's weight blocks, then its hidden-state blocks
     const int num_kb = p.K / kBlockK;
     const uint32_t pair_rank = PAIR ? cluster_cta_rank() : 0u;
 
@@ -467,7 +493,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
     if constexpr (!PAIR) {
         if (warp == 2 && lane == 0 && n_tiles > 0) {
             const int n_pf = min(num_kb, kPrefetchBlocks);
-            for (int kb = 0; kb < n_pf; ++kb) tma_prefetch_2d(&map_w128, kb * kBlockK, row_begin);
+            for (int kb = 0; kb < n_pf; kb += kStageBlocks) tma_prefetch_blocks(&map_w, row_begin, kb);
         }
     }
     pdl_wait();          // everything above overlapped with the tail of the previous kernel
@@ -487,12 +513,11 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
             bool ok = true;
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int v0 = row_begin + t * tile_rows + (int)pair_rank * kVocabTile;
-                const int rows = PAIR ? kVocabTile : min(tile_rows, row_end - v0);
-                const uint32_t tx_bytes = (uint32_t)(rows * 128 + p.n_tile * 128);
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int kb = 0; kb < num_kb; kb += kStageBlocks) {
                     if (!mbar_wait(&empty_bar[s], ph ^ 1u, abort_ptr)) { ok = false; break; }
+                    uint8_t* h_dst = w_dst + kStageBlocks * kTileBytesW;
 #ifdef MASSV_TEST_HOOKS
-                    if (p.test_skip_stage && t == 0 && kb == 1) {
+                    if (p.test_skip_stage && t == 0 && kb + kStageBlocks >= num_kb) {
                         // nothing is announced and nothing is copied for this stage: the MMA thread's wait for it
                         // must give up by itself
                         w_dst += stage_bytes;
@@ -500,31 +525,19 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                         continue;
                     }
 #endif
-                    uint8_t* h_dst = w_dst + kTileBytesW;
+                    // rows past the end of either matrix and K blocks past its width are filled with zeros and still counted
                     if constexpr (PAIR) {
-                        // Both CTAs' copies complete on the leader's barrier; the leader announces the
-                        // bytes of the pair (two 128-row weight boxes, two halves of the hidden-state tile;
-                        // rows past the end of either matrix are filled with zeros and still counted).
+                        // Both CTAs' copies complete on the leader's barrier; the leader announces the bytes of the pair
+                        // (per K block two 128-row weight boxes, two halves of the hidden-state tile).
                         const uint32_t bar = cluster_addr(&full_bar[s], 0);
-                        if (pair_rank == 0) mbar_expect_tx_at(bar, (uint32_t)(2 * kTileBytesW + p.n_tile * 128));
-                        tma_load_2d_pair(w_dst, &map_w128, kb * kBlockK, v0, bar, pol_stream);
-                        tma_load_2d_pair(h_dst, &map_h, kb * kBlockK, (int)pair_rank * h_rows, bar, pol_keep);
-                        w_dst += stage_bytes;
-                        if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
-                        continue;
-                    }
-                    mbar_expect_tx(&full_bar[s], tx_bytes);
-                    if (rows == kVocabTile) {
-                        tma_load_2d(w_dst, &map_w128, kb * kBlockK, v0, &full_bar[s], pol_stream);
+                        if (pair_rank == 0) mbar_expect_tx_at(bar, (uint32_t)(2 * stage_bytes));
+                        tma_load_blocks_pair(w_dst, &map_w, v0, kb, bar, pol_stream);
+                        tma_load_blocks_pair(h_dst, &map_h, (int)pair_rank * h_rows, kb, bar, pol_keep);
                     } else {
-                        // rows is a multiple of 8 below 128: one box per set bit
-                        int r = 0;
-                        if (rows & 64) { tma_load_2d(w_dst + r * 128, &map_w64, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 64; }
-                        if (rows & 32) { tma_load_2d(w_dst + r * 128, &map_w32, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 32; }
-                        if (rows & 16) { tma_load_2d(w_dst + r * 128, &map_w16, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 16; }
-                        if (rows & 8) { tma_load_2d(w_dst + r * 128, &map_w8, kb * kBlockK, v0 + r, &full_bar[s], pol_stream); r += 8; }
+                        mbar_expect_tx(&full_bar[s], (uint32_t)stage_bytes);
+                        tma_load_blocks(w_dst, &map_w, v0, kb, &full_bar[s], pol_stream);
+                        tma_load_blocks(h_dst, &map_h, 0, kb, &full_bar[s], pol_keep);
                     }
-                    tma_load_2d(h_dst, &map_h, kb * kBlockK, 0, &full_bar[s], pol_keep);
                     w_dst += stage_bytes;
                     if (++s == p.stages) { s = 0; ph ^= 1u; w_dst = smem; }
                 }
@@ -541,7 +554,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                                    ((uint32_t)((PAIR ? 2 * kVocabTile : kVocabTile) >> 4) << 24);
             // The issuing thread must stay far below the 64..128 cycles one MMA takes, so the
             // loop carries only 32-bit descriptor words and a stage counter.
-            const uint32_t lo_step = (uint32_t)stage_bytes >> 4;
+            const uint32_t lo_step = (uint32_t)stage_bytes >> 4, h_step = (uint32_t)h_bytes >> 4;
             const uint32_t a_lo0 = umma_desc_lo(smem_u32(smem));
             int s = 0;
             uint32_t ph = 0, a_lo = a_lo0;
@@ -551,26 +564,25 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
                 if (!mbar_wait(&tmem_empty_bar[buf], (((uint32_t)t >> 1) & 1u) ^ 1u, abort_ptr)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * p.tmem_cols / 2);
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int kb = 0; kb < num_kb; kb += kStageBlocks) {
                     if (!mbar_wait(&full_bar[s], ph, abort_ptr)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t b_lo = a_lo + (kTileBytesW >> 4);
-                    // four K slices of 16 elements (32 bytes, i.e. 2 descriptor units) each
-                    if constexpr (PAIR) {
-                        if (kb == 0) umma_bf16_pair<false>(d_tmem, a_lo, b_lo, idesc);
-                        else umma_bf16_pair<true>(d_tmem, a_lo, b_lo, idesc);
-                        umma_bf16_pair<true>(d_tmem, a_lo + 2, b_lo + 2, idesc);
-                        umma_bf16_pair<true>(d_tmem, a_lo + 4, b_lo + 4, idesc);
-                        umma_bf16_pair<true>(d_tmem, a_lo + 6, b_lo + 6, idesc);
-                        umma_commit_pair(&empty_bar[s]);     // frees the stage in both CTAs
-                    } else {
-                        if (kb == 0) umma_bf16<false>(d_tmem, a_lo, b_lo, idesc);
-                        else umma_bf16<true>(d_tmem, a_lo, b_lo, idesc);
-                        umma_bf16<true>(d_tmem, a_lo + 2, b_lo + 2, idesc);
-                        umma_bf16<true>(d_tmem, a_lo + 4, b_lo + 4, idesc);
-                        umma_bf16<true>(d_tmem, a_lo + 6, b_lo + 6, idesc);
-                        umma_commit(&empty_bar[s]);      // frees the stage once these MMAs have read it
+                    const uint32_t b_lo = a_lo + kStageBlocks * (kTileBytesW >> 4);
+                    // four K slices of 16 elements (32 bytes, i.e. 2 descriptor units) per K block
+#pragma unroll
+                    for (int i = 0; i < 4 * kStageBlocks; ++i) {
+                        const uint32_t wd = a_lo + (uint32_t)((i >> 2) * (kTileBytesW >> 4) + (i & 3) * 2);
+                        const uint32_t hd = b_lo + (uint32_t)(i >> 2) * h_step + (uint32_t)((i & 3) * 2);
+                        if constexpr (PAIR) {
+                            if (i == 0 && kb == 0) umma_bf16_pair<false>(d_tmem, wd, hd, idesc);
+                            else umma_bf16_pair<true>(d_tmem, wd, hd, idesc);
+                        } else {
+                            if (i == 0 && kb == 0) umma_bf16<false>(d_tmem, wd, hd, idesc);
+                            else umma_bf16<true>(d_tmem, wd, hd, idesc);
+                        }
                     }
+                    if constexpr (PAIR) umma_commit_pair(&empty_bar[s]);     // frees the stage in both CTAs
+                    else umma_commit(&empty_bar[s]);                         // frees the stage once these MMAs have read it
                     a_lo += lo_step;
                     if (++s == p.stages) { s = 0; ph ^= 1u; a_lo = a_lo0; }
                 }
@@ -590,7 +602,7 @@ lm_head_umma_kernel(const __grid_constant__ CUtensorMap map_w128, const __grid_c
         const int quarter = warp & 3;
         const int part = (warp - 2) >> 2;
         // running statistics per (quarter, column); each column is touched by exactly one lane of one warp
-        for (int c = threadIdx.x - 64; c < 4 * 256; c += kEpilogueWarps * 32) {
+        for (int c = threadIdx.x - 64; c < 4 * kCols; c += kEpilogueWarps * 32) {
             (&run_m[0][0])[c] = -INFINITY; (&run_s[0][0])[c] = 0.f; (&run_i[0][0])[c] = 0x7fffffff;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(kEpilogueWarps * 32) : "memory");     // epilogue warps only
@@ -978,7 +990,7 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     groups = (bands + p.tiles_per_group - 1) / p.tiles_per_group;
     p.n_groups = groups;
     const int h_rows = pair ? p.n_tile / 2 : p.n_tile;
-    const int stage_bytes = kTileBytesW + h_rows * 128;
+    const int stage_bytes = kStageBlocks * (kTileBytesW + h_rows * 128);
     int stages = kRingBytes / stage_bytes;
     if (stages > kMaxStages) stages = kMaxStages;
     p.stages = stages;
@@ -996,10 +1008,9 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     if (slots > q.n_part) return cudaErrorInvalidValue;
     *n_part_used = slots;
 
-    CUtensorMap map_w[5], map_h;
-    for (int i = 0; i < 5; ++i)
-        if (!make_tensor_map_bf16_2d(&map_w[i], q.lm_head, q.V, q.K, kVocabTile >> i)) return cudaErrorInvalidValue;
-    if (!make_tensor_map_bf16_2d(&map_h, q.hidden, q.M, q.K, h_rows)) return cudaErrorInvalidValue;
+    CUtensorMap map_w, map_h;
+    if (!make_tensor_map_bf16_blocks(&map_w, q.lm_head, q.V, q.K, kVocabTile, kStageBlocks)) return cudaErrorInvalidValue;
+    if (!make_tensor_map_bf16_blocks(&map_h, q.hidden, q.M, q.K, h_rows, kStageBlocks)) return cudaErrorInvalidValue;
 
     const size_t smem = (size_t)stages * stage_bytes + 1024;
     cudaError_t e;
@@ -1008,13 +1019,11 @@ cudaError_t launch_lm_head(const LmHeadParams& q, cudaStream_t stream, int* n_pa
     if (pair) {
         e = cudaFuncSetAttribute(lm_head_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRingSmem);
         if (e != cudaSuccess) return e;
-        e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * 2), dim3(lm_head_threads(true)), smem, stream, 2,
-                               map_w[0], map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
+        e = launch_pdl_cluster(lm_head_umma_kernel<true>, dim3(groups * 2), dim3(lm_head_threads(true)), smem, stream, 2, map_w, map_h, p);
     } else {
         e = cudaFuncSetAttribute(lm_head_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRingSmem);
         if (e != cudaSuccess) return e;
-        e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups), dim3(lm_head_threads(false)), smem, stream, map_w[0],
-                       map_w[1], map_w[2], map_w[3], map_w[4], map_h, p);
+        e = launch_pdl(lm_head_umma_kernel<false>, dim3(groups), dim3(lm_head_threads(false)), smem, stream, map_w, map_h, p);
     }
     if (e != cudaSuccess) return e;
     if (hooks.lm_head_stop && cudaEventRecord(hooks.lm_head_stop, stream) != cudaSuccess) return cudaGetLastError();

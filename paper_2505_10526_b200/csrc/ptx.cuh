@@ -59,11 +59,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
-// A hint to bring one box of a tensor map into L2; nothing waits on it and nothing in shared memory changes.
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
-}
-
 // Plain 1-D copies into shared memory, without an eviction hint: by the bulk engine (16-byte multiples, signalled on an mbarrier)
 // and by the calling thread.
 __device__ __forceinline__ void bulk_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -100,5 +95,8 @@ __device__ __forceinline__ uint32_t peer_load_u32(const void* local, int rank) {
 // [box_rows, 64 cols] and the 128-byte swizzle.  Returns false if the driver
 // entry point is unavailable or rejects the shape.
 bool make_tensor_map_bf16_2d(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
+// The same matrix as a 3-D map [cols / 64, rows, 64], box [blocks, box_rows, 64]: one copy brings several groups of 64
+// columns (cols a multiple of 64; groups past the end are filled with zeros).
+bool make_tensor_map_bf16_blocks(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t blocks);
 
 }  // namespace massv

@@ -63,3 +63,26 @@ def test_sums_of_exponentials(batch, gamma, std, shift, T):
         worst = max(worst, float((probs[b].max(-1).values.double() / top - 1).abs().max()))
     print("worst", worst)
     assert worst < 1.5e-6
+
+
+@pytest.mark.parametrize("hidden_size", [64, 128, 320, 832, 1088])
+@pytest.mark.parametrize("batch", [1, 40, 64, 200, 256])
+def test_k_blocks(batch, hidden_size):
+    """A ring stage holds two blocks of 64 hidden elements: one block in all, full stages, a last stage with one block, rings that wrap
+    inside a tile and across tiles.  fp32 sums of K products of size 0.25 or less, in any order: below K * 2^-24 * sqrt(K) * 0.25."""
+    import paper_2505_10526_b200 as mv
+    vocab = 40008
+    g = torch.Generator(device="cuda").manual_seed(hidden_size + batch)
+    hidden = (5.0 * torch.randn((batch, 1, hidden_size), generator=g, device="cuda")).to(torch.bfloat16)
+    w = (0.05 * torch.randn((vocab, hidden_size), generator=g, device="cuda")).to(torch.bfloat16)
+    exact = torch.matmul(hidden.view(-1, hidden_size).double(), w.double().t()).view(batch, 1, vocab)
+    logits = torch.full((batch, 1, vocab), float("nan"), device="cuda")
+    tokens = torch.empty((batch, 1), dtype=torch.int32, device="cuda"); lens = torch.empty((batch,), dtype=torch.int32, device="cuda")
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    desc = mv.accept_desc(batch, 0, hidden_size, vocab, 0.0)
+    ws = mv.alloc_workspace(mv.massv_accept_workspace_size(desc), "cuda").fill_(0xff)
+    mv.massv_accept(desc, hidden, w, torch.zeros((batch, 0), dtype=torch.int32, device="cuda"), None, None, None, tokens, lens, logits, None, ws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert float((logits.double() - exact).abs().max()) < hidden_size ** 1.5 * 2 ** -24 * 0.25 + 1e-5
+    assert torch.equal(tokens[:, 0].long(), logits[:, 0].argmax(-1))
