@@ -354,15 +354,14 @@ struct RowPublished {
     unsigned long long hist[2][kTopPBins];   // two levels of the threshold search take turns
     unsigned long long max_bits;
     unsigned long long mass;                 // bits of a double: mass above the candidates (later: above tau)
-    unsigned long long n_cand;               // entries that share tau's leading 17 bits (later: equal to tau)
+    unsigned long long n_cand;               // entries that share the bits of tau found by then
     uint32_t cand[kRowCand];                 // their patterns, in no particular order
 };
 
-// What bounds it: the row crosses HBM once in and once out (8 B per entry); between the two lie four barriers of the
-// cluster (about 2 us each with the exchange behind them) and four walks over the slice in shared memory (1 - 3.5 us
-// with two CTAs on an SM), a serial chain of about 26 us per CTA.  64 rows of 152,064 with probs_out: 188 us with one CTA
-// per row re-reading it from L2 in nine passes (64 of 148 SMs busy), 60 us here (two waves of CTAs); 128 rows of 8,000:
-// 34 -> 15 us; one row of 262,144: 273 -> 23 us.
+// What bounds it: the row crosses HBM once in and once out (8 B per entry); between the two lie three barriers of the
+// cluster (about 2 us each with the exchange behind them) and three walks over the slice in shared memory (1 - 3.5 us
+// with two CTAs on an SM), a serial chain of about 22 us per CTA.  64 rows of 152,064 with probs_out: 188 us with one CTA
+// per row re-reading it from L2 in nine passes (64 of 148 SMs busy), 54 us here (two waves of CTAs).
 __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParams p, int n_ctas, int slice) {
     extern __shared__ __align__(16) float s_w[];                 // the slice: logits, then weights
     __shared__ uint32_t hist_lo[kRowCopies * kRowCopyStride], hist_hi[kRowCopies * kRowCopyStride];
@@ -375,7 +374,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
     __shared__ double s_cta_mass[kRowMaxCluster], s_cand_mass[kRowMaxCluster];
     __shared__ int s_cta_count[kRowMaxCluster], s_cand_ties[kRowMaxCluster];
     __shared__ unsigned long long s_above;
-    __shared__ int s_bin, s_n_cand, s_owner, s_owner_last;
+    __shared__ int s_bin, s_in_bin, s_n_cand, s_owner, s_owner_last;
 
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int rank = blockIdx.x % n_ctas, row = blockIdx.x / n_ctas;
@@ -441,11 +440,14 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
     }
     const RowWeight weight_of(p.inv_T, m);
 
-    // ---- threshold: largest bit pattern tau with mass{w >= tau} >= target, by radix selection (9 + 8 bits, then the few
-    // entries that share them one by one; 9 + 5 more levels where they are many).  A bin of the first level fixes the
-    // exponent, so its mass is a sum of (truncated) mantissas: a word that wraps every 256 entries at most, and a carry.
-    uint32_t prefix = 0u;                 // bits of tau found so far
-    unsigned long long mass_above = 0ull, target_fx = 0ull;
+    // ---- threshold: largest bit pattern tau with mass{w >= tau} >= target, by radix selection: a first level of 32 bins per
+    // power of two, levels of 9 bits more while more than kRowCand entries share the bits found, then those entries one by
+    // one.  A bin fixes the exponent, so its mass is a sum of (truncated) mantissas: a word that wraps every 256 entries at
+    // most, and a carry.  A language model's row needs the first level only; with two bins per power of two it took a second
+    // walk and exchange (64 rows of 152,064: 61 us, 54 here).
+    uint32_t prefix = 0u;                 // bits of tau found so far: all but the last `open` ones
+    int open = 0;
+    unsigned long long mass_above = 0ull, target_fx = 0ull, total_fx = 0ull;
     const int my_copy = (lane & (kRowCopies - 1)) * kRowCopyStride;
     auto mantissa = [&](uint32_t b) { return ((b & 0x7FFFFFu) | 0x800000u) >> min(max(106 - (int)(b >> 23), 0), 31); };      // zero below 2^-44
     // four entries at a time, so that four atomics are in flight before the first result is looked at
@@ -457,9 +459,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
         for (int j = 0; j < 4; ++j) if (old[j] > ~v[j]) atomicAdd(&hist_hi[my_copy + bin[j]], 1u);      // the word wrapped
     };
     // One level once the copies are filled: the cluster's bins, and the one in which the running mass from the top
-    // crosses the target.
+    // crosses the target.  Bin t < n_bins stands for the patterns from `low` + (t << shift) on; bin sum_bin, if the level
+    // has one, is the sum of the light entries (in units of 2^-44).
     int half = 0;                         // which of the two published histograms is next
-    auto find_bin = [&](int level, int shift, int bin_lo, int bin_hi) {          // only bins bin_lo .. bin_hi - 1 can have mass
+    auto find_bin = [&](uint32_t low, int shift, int n_bins, int sum_bin) {
         __syncthreads();
         // thread t owns bin t: its copies, cleared for the next level, then the other CTAs' share of it
         unsigned long long own = 0ull;
@@ -469,7 +472,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
             own += ((unsigned long long)hist_hi[at] << 32) + (unsigned long long)hist_lo[at];
             hist_hi[at] = 0u; hist_lo[at] = 0u;
         }
-        if (level == 0 && t == 0) {
+        if (t == sum_bin) {
             own = 0ull;
 #pragma unroll
             for (int w = 0; w < kRowWarps; ++w) own += s_warp_light[w];
@@ -480,7 +483,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
             // which it reaches after these reads)
             row_barrier(n_ctas);
             own = 0ull;
-            if ((t >= bin_lo && t < bin_hi) || (level == 0 && t == 0)) {
+            if (t < n_bins || t == sum_bin) {
                 unsigned long long part[kRowMaxCluster];
 #pragma unroll
                 for (int r = 0; r < kRowMaxCluster; ++r) part[r] = r < n_ctas ? peer_load_u64(&s_pub.hist[half][t], r) : 0ull;
@@ -488,30 +491,44 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
                 for (int r = 0; r < kRowMaxCluster; ++r) own += part[r];
             }
         }
-        // mantissas -> units of 2^-44 (bin 0 of the first level is the sum of the light entries, in these units already)
-        own <<= max((level <= 0 ? t >> 1 : (int)(prefix >> 23)) - 106, 0);
-        // suffix sums over the bins, highest first
-        unsigned long long incl = own;
+        // mantissas -> units of 2^-44
+        const uint32_t bits = low + ((uint32_t)t << shift);
+        const unsigned long long in_units = t == sum_bin ? own : own << max((int)(bits >> 23) - 106, 0);
+        // suffix sums over the bins, highest first (the light entries below all others)
+        unsigned long long incl = t == sum_bin ? 0ull : in_units;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned long long y = __shfl_down_sync(0xffffffffu, incl, o);
             if (lane + o < 32) incl += y;
         }
         if (lane == 0) s_warp[warp] = incl;
+        if (t == sum_bin) s_above = in_units;
         __syncthreads();
         unsigned long long above = 0ull, total = 0ull;
 #pragma unroll
         for (int w = 0; w < kRowWarps; ++w) { total += s_warp[w]; if (w > warp) above += s_warp[w]; }
-        if (level == 0) {
+        unsigned long long run = mass_above + above + incl - in_units;
+        if (sum_bin >= 0) {
+            if (t == sum_bin) run = total;
+            total += s_above;
+            total_fx = total;
             target_fx = (unsigned long long)ceil((double)p.top_p * (double)total);
             if (target_fx > total) target_fx = total;
             if (target_fx == 0ull) target_fx = 1ull;
+            __syncthreads();                       // s_above has been read
         }
         // the bin b with mass_above + sum(bins > b) < target <= mass_above + sum(bins >= b) exists exactly once
-        const unsigned long long run = mass_above + above + incl - own;
-        if (run < target_fx && run + own >= target_fx) { s_bin = t; s_above = run; }
+        if (run < target_fx && run + in_units >= target_fx) {
+            s_bin = t;
+            s_above = run;
+            // entries in the bin, at most: none is lighter than the bin's lower end
+            const unsigned long long most = own / max(1u, mantissa(bits));
+            s_in_bin = most < 0x7fffffffull ? (int)most : 0x7fffffff;
+        }
         __syncthreads();
-        prefix |= (uint32_t)s_bin << shift;
+        const bool among_light = s_bin == sum_bin;
+        prefix = among_light ? 0u : low + ((uint32_t)s_bin << shift);
+        open = shift;
         mass_above = s_above;
         half ^= 1;
     };
@@ -526,13 +543,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
             if (fmaxf(fmaxf(y.x, y.y), fmaxf(y.z, y.w)) >= from) f(y);          // (from > 0)
         }
     };
-    auto add_matching = [&](int done, int shift, uint32_t mask) {       // histogram of the entries that share the bits found so far
-        walk(prefix, [&](const float4& x) {
+    auto add_matching = [&](int shift) {       // histogram of the entries that share the bits found so far, by the bits from `shift` on
+        const uint32_t from = prefix;
+        const int known = open;
+        walk(from, [&](const float4& x) {
             const uint32_t b[4] = {__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z), __float_as_uint(x.w)};
             uint32_t v[4];
             int bin[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) { v[j] = (b[j] >> done) == (prefix >> done) ? mantissa(b[j]) : 0u; bin[j] = (int)((b[j] >> shift) & mask); }
+            for (int j = 0; j < 4; ++j) { v[j] = (b[j] >> known) == (from >> known) ? mantissa(b[j]) : 0u; bin[j] = (int)((b[j] - from) >> shift); }
             add4(v, bin);
         });
     };
@@ -555,7 +574,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
             const bool h = b[j] >= kLightBits;
             heavy = heavy || h;
             v[j] = h ? mantissa(b[j]) : 0u;
-            bin[j] = (int)(b[j] >> 22);
+            bin[j] = (int)((b[j] - kLightBits) >> 18);
             // floor(w * 2^44) < 2^32: the mantissa in the word's upper 24 bits, shifted down (shr gives zero from 32 on)
             uint32_t f;
             asm("shr.u32 %0, %1, %2;" : "=r"(f) : "r"(((b[j] & 0x7FFFFFu) | 0x800000u) << 8), "r"(114u - (b[j] >> 23)));
@@ -566,36 +585,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) light += __shfl_xor_sync(0xffffffffu, light, o);
     if (lane == 0) s_warp_light[warp] = light;
-    find_bin(0, 22, 2 * 115, 256);
-    if (prefix == 0u) {                           // the crossing lies in bin 0: among the light entries (same in all CTAs)
-        walk(1u, [&](const float4& x) {
-            const uint32_t b[4] = {__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z), __float_as_uint(x.w)};
-            uint32_t v[4];
-            int bin[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { v[j] = b[j] < kLightBits ? mantissa(b[j]) : 0u; bin[j] = (int)(b[j] >> 22); }
-            add4(v, bin);
-        });
-        find_bin(-1, 22, 2 * 83, 2 * 115);        // 2^-44 <= w < 2^-12
-    }
-    add_matching(22, 14, 255u);
-    find_bin(1, 14, 0, 256);
-
-    // ---- 17 bits of tau are known, and few entries share them: every CTA adds up what lies above and publishes the
-    // candidates, and the whole cluster resolves tau, the ties and the masses from one exchange.
-    double mass_gt = 0.0;
-    walk(prefix, [&](const float4& x) {
-        const float w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t b = __float_as_uint(w[j]);
-            if ((b >> 14) > (prefix >> 14)) mass_gt += (double)w[j];
-            else if ((b >> 14) == (prefix >> 14)) {
-                const int k = atomicAdd(&s_n_cand, 1);
-                if (k < kRowCand) s_pub.cand[k] = b;
-            }
-        }
-    });
+    find_bin(kLightBits, 18, 12 * 32 + 1, kRowThreads - 1);          // (2^-12 <= w <= 1; the last bin is free for the light sum)
     auto publish = [&](double mass, int count) {           // this CTA's mass and count, visible to the cluster on return
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) { mass += __shfl_xor_sync(0xffffffffu, mass, o); count += __shfl_xor_sync(0xffffffffu, count, o); }
@@ -610,15 +600,82 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
         }
         row_barrier(n_ctas);
     };
-    __syncthreads();
-    publish(mass_gt, t == 0 ? s_n_cand : 0);
+    constexpr uint32_t kLowest = 83u << 23;       // 2^-44: lighter entries have no mass
+    // What the last walk leaves: every CTA's mass above tau and the number of entries that may be tau (listed: which they are).
+    double mass_gt = 0.0;
+    int n_equal = 0;
+    const bool everything = target_fx == total_fx;        // the same in all CTAs
+    bool listed = false;
+    if (everything) {
+        // top_p takes the whole row: tau is the lightest entry that has mass
+        uint32_t least = 0xffffffffu;
+        walk(kLowest, [&](const float4& x) {
+            const float w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t b = __float_as_uint(w[j]);
+                if (b >= kLowest) {
+                    mass_gt += (double)w[j];
+                    n_equal = b < least ? 1 : n_equal + (b == least ? 1 : 0);
+                    least = min(least, b);
+                }
+            }
+        });
+        const uint32_t warp_least = __reduce_min_sync(0xffffffffu, least);
+        if (lane == 0) s_cand[warp] = warp_least;
+        __syncthreads();
+        uint32_t cta_least = s_cand[0];
+#pragma unroll
+        for (int w = 1; w < kRowWarps; ++w) cta_least = min(cta_least, s_cand[w]);
+        if (least != cta_least) n_equal = 0;
+        if (t < kRowCand) s_pub.cand[t] = cta_least;
+    } else {
+        if (prefix == 0u) {                       // the crossing lies among the light entries (same in all CTAs)
+            walk(1u, [&](const float4& x) {
+                const uint32_t b[4] = {__float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(x.z), __float_as_uint(x.w)};
+                uint32_t v[4];
+                int bin[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { v[j] = b[j] < kLightBits ? mantissa(b[j]) : 0u; bin[j] = (int)((b[j] - kLowest) >> 19); }
+                add4(v, bin);
+            });
+            find_bin(kLowest, 19, kTopPBins, -1); // 2^-44 <= w < 2^-12, 16 bins per power of two
+        }
+        while (open > 0 && s_in_bin > kRowCand) {
+            const int shift = max(open - 9, 0);
+            add_matching(shift);
+            find_bin(prefix, shift, 1 << (open - shift), -1);
+        }
+
+        // ---- Few entries share the bits of tau found so far (or all of it is known): every CTA adds up what lies above and
+        // publishes the candidates, and the whole cluster resolves tau, the ties and the masses from one exchange.
+        const uint32_t lead = prefix >> open;
+        const int known = open;
+        listed = s_in_bin <= kRowCand;            // (then the candidates of all CTAs together fit one list)
+        walk(prefix, [&](const float4& x) {
+            const float w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t b = __float_as_uint(w[j]);
+                if ((b >> known) > lead) mass_gt += (double)w[j];
+                else if ((b >> known) == lead) {
+                    ++n_equal;
+                    if (listed) {
+                        const int k = atomicAdd(&s_n_cand, 1);
+                        if (k < kRowCand) s_pub.cand[k] = b;
+                    }
+                }
+            }
+        });
+    }
+    publish(mass_gt, n_equal);
     // warp r asks CTA r: its mass, its count, and one candidate per lane
     uint32_t c = 0u;
     if (warp < kRowMaxCluster) {
         const int asked = min(warp, n_ctas - 1);
         const uint32_t theirs = peer_load_u32(&s_pub.cand[lane], asked);
         const unsigned long long mass = peer_load_u64(&s_pub.mass, asked), count = peer_load_u64(&s_pub.n_cand, asked);
-        if (warp < n_ctas && lane < (int)count) c = theirs;
+        if (everything ? warp < n_ctas : (listed && warp < n_ctas && lane < (int)count)) c = theirs;
         s_cand[t] = c;
         if (lane == 0) {
             s_cta_mass[warp] = warp < n_ctas ? __longlong_as_double((long long)mass) : 0.0;
@@ -628,11 +685,24 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
     __syncthreads();
     double mass_of[kRowMaxCluster];                        // mass above tau, later of the members, of every CTA
     int n_of[kRowMaxCluster];                              // candidates, later ties, of every CTA
-    bool fits = true;
 #pragma unroll
-    for (int r = 0; r < kRowMaxCluster; ++r) { mass_of[r] = s_cta_mass[r]; n_of[r] = s_cta_count[r]; fits = fits && n_of[r] <= kRowCand; }
-    float tau;
-    if (fits) {
+    for (int r = 0; r < kRowMaxCluster; ++r) { mass_of[r] = s_cta_mass[r]; n_of[r] = s_cta_count[r]; }
+    float tau = __uint_as_float(prefix);          // more entries than a list holds share every bit: it is tau, and they are the ties
+    if (everything) {
+        uint32_t least = 0xffffffffu;
+#pragma unroll
+        for (int r = 0; r < kRowMaxCluster; ++r) if (r < n_ctas) least = min(least, s_cand[r * kRowCand]);
+        tau = __uint_as_float(least);
+        const unsigned long long tau_fx = (unsigned long long)mantissa(least) << max((int)(least >> 23) - 106, 0);
+        unsigned long long ties_fx = 0ull;
+#pragma unroll
+        for (int r = 0; r < kRowMaxCluster; ++r) {
+            if (s_cand[r * kRowCand] != least) n_of[r] = 0;
+            mass_of[r] -= (double)n_of[r] * (double)tau;
+            ties_fx += (unsigned long long)n_of[r] * tau_fx;
+        }
+        mass_above = target_fx - ties_fx;
+    } else if (listed) {
         if (c != 0u) {
             // the candidate at which the running mass from the top crosses the target is tau (all have one exponent)
             unsigned long long gt = 0ull, eq = 0ull;
@@ -661,28 +731,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < kRowMaxCluster; ++r) { mass_of[r] += s_cand_mass[r]; n_of[r] = s_cand_ties[r]; }
-    } else {
-        // many entries share the 17 bits (equal or nearly equal logits): the last two levels, then masses and ties
-        add_matching(14, 5, 511u);
-        find_bin(2, 5, 0, 512);
-        add_matching(5, 0, 31u);
-        find_bin(3, 0, 0, 32);
-        tau = __uint_as_float(prefix);
-        int ties = 0;
-        mass_gt = 0.0;
-        walk(prefix, [&](const float4& x) {
-            const float w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { if (w[j] > tau) mass_gt += (double)w[j]; ties += w[j] == tau ? 1 : 0; }
-        });
-        publish(mass_gt, ties);
-#pragma unroll
-        for (int r = 0; r < kRowMaxCluster; ++r) {
-            if (r < n_ctas) {
-                mass_of[r] = __longlong_as_double((long long)peer_load_u64(&s_pub.mass, r));
-                n_of[r] = (int)peer_load_u64(&s_pub.n_cand, r);
-            }
-        }
     }
     if (n_ctas > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");        // done with the others' shared memory
     // how many of the tokens equal to tau the prefix takes (at least one: mass{w > tau} < target)

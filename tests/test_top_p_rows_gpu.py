@@ -120,3 +120,15 @@ def test_rows_come_out_the_same_in_calls_of_any_size(vocab):
             at = t.long().clamp_min(1)
             gap = torch.minimum((cdf.gather(-1, t.long()[:, None])[:, 0] - u[:rows]).abs(), (cdf.gather(-1, (at - 1)[:, None])[:, 0] - u[:rows]).abs())
             assert bool(((t == tok[:rows]) | (gap < 1e-6)).all())
+
+
+@pytest.mark.parametrize("std", [0.01, 0.3, 1.5, 8.0])
+@pytest.mark.parametrize("top_p", [0.05, 0.6, 0.97, 1.0])
+def test_levels(std, top_p):
+    """From rows whose first level holds thousands of entries in a bin to rows that need one level, thresholds among the heavy and
+    among the light entries, and the whole row (there entries below 2^-44 of the largest, 5e4 * 2^-44 = 3e-9 of the mass, are left out)."""
+    g = torch.Generator(device="cuda").manual_seed(int(100 * std) + int(100 * top_p))
+    z = std * torch.randn((5, 50264), generator=g, device="cuda")
+    z[1, ::3] = -float("inf")
+    z[2, 100:] = -float("inf")
+    _check(z, torch.rand((5,), generator=g, device="cuda"), 1.0, top_p, allow=5 if top_p == 1.0 else 2)
