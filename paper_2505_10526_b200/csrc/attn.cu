@@ -828,6 +828,23 @@ bool attn_use_umma(const AttnParams& p) {
     return p.d <= 128;
 }
 
+// The most positions a (sequence, KV head) pair can need.
+static long pair_tokens(const AttnParams& p) {
+    const long tokens = (long)p.max_pages * kPageSize;
+    return p.window > 0 && p.window + p.R + 64 < tokens ? p.window + p.R + 64 : tokens;
+}
+
+// tcgen05 kernel: one CTA per pair where pairs are short, instead of ranges of the line of tiles: nothing to deal out, no pieces and
+// no merge launch.  A CTA takes 6 - 7.5 us and 1.2 - 1.5 us per tile of 64 positions, the balanced line with its merge at least
+// 9 - 10 us and more the more pairs it cuts, so the line between them rises with the number of pairs.  Call times, balanced -> one
+// CTA per pair, head_dim 128, lengths from a quarter of the table to all of it: 1 x 4 pairs of up to 128 positions 10.2 -> 7.7 us,
+// 16 x 4 of 128 14.5 -> 9.1, of 256 14.6 -> 12.0, of 512 17.0 -> 17.7; 64 x 4 of 256 26.8 -> 13.7, of 512 30.5 -> 20.1, of 1,024
+// 36 -> 32; 64 x 8 of 512 50 -> 38.
+static bool one_piece_per_pair(const AttnParams& p) {
+    const long pairs = (long)p.B * p.Hkv, tiles = (pair_tokens(p) + 63) / 64;
+    return !p.chunk_forced && p.max_pages <= kMaxChunkPages && tiles <= 4 + (pairs < 96 ? pairs / 24 : 4);
+}
+
 // Balanced schedule or chunk grid for the warp-MMA kernel at head_dim 256.  The balanced one wins wherever the grid would cut
 // a pair into chunks, since that costs CTAs that retire at once and a merge as well (times of a call, page table for 8,192
 // positions: 32 x 8 pairs of 2k - 8k positions 243 -> 224 us, of 100 - 900 50 -> 38, of 1 - 100 24 -> 23; a window of 1,024 on long
@@ -840,9 +857,7 @@ bool attn_use_umma(const AttnParams& p) {
 static bool use_flat_warp_mma(const AttnParams& p, int mt) {
     if (p.d != 256 || p.chunk_forced || p.B > kFlatMaxBatchMeta) return false;
     if (mt > 1 || p.max_chunks > 1) return true;
-    long tokens = (long)p.max_pages * kPageSize;                     // the most a pair can need
-    if (p.window > 0 && p.window + p.R + 64 < tokens) tokens = p.window + p.R + 64;
-    return tokens > 544 && (long)p.B * p.Hkv > 2L * device_sm_count();
+    return pair_tokens(p) > 544 && (long)p.B * p.Hkv > 2L * device_sm_count();
 }
 
 cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream) {
@@ -858,8 +873,18 @@ cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream) {
     const TimingHooks& hooks = timing_hooks();
     if (hooks.attn_start && cudaEventRecord(hooks.attn_start, stream) != cudaSuccess) return cudaGetLastError();
     if (attn_use_umma(p)) {
-        const bool flat = !p.chunk_forced && attn_umma_flat_supported(p);
+        const bool one_piece = one_piece_per_pair(p), flat = !one_piece && !p.chunk_forced && attn_umma_flat_supported(p);
         int launched = 0;
+        if (one_piece) {
+            AttnParams q = p;
+            q.kv_chunk = (p.max_pages * kPageSize + kChunkAlign - 1) / kChunkAlign * kChunkAlign;
+            q.max_chunks = 1;
+            e = launch_attn_umma(q, mk, mv, stream, false, &launched, nullptr);
+            if (e != cudaSuccess) return e;
+            if (hooks.attn_stop && cudaEventRecord(hooks.attn_stop, stream) != cudaSuccess) return cudaGetLastError();
+            count_launches(launched);
+            return cudaGetLastError();
+        }
         e = launch_attn_umma(p, mk, mv, stream, flat, &launched, hooks.attn_stop);
         if (e != cudaSuccess) return e;
         if (flat) {

@@ -24,7 +24,7 @@
 //
 // Two schedules share the kernel.  CHUNKED: grid (chunk, KV head, sequence) as in the warp-MMA
 // kernel, one piece of work per CTA, pieces of a sequence merged by attn_combine_kernel (used
-// when the caller fixes kv_chunk).  FLAT: the tiles of all (sequence, KV head) pairs form one
+// when the caller fixes kv_chunk, and with one chunk per pair where page tables are short).  FLAT: the tiles of all (sequence, KV head) pairs form one
 // line, ordered by (sequence, head, position); a persistent grid of resident CTAs cuts the line
 // into equal ranges, so every CTA streams the same number of bytes whatever the mix of context
 // lengths, pays its set-up once, and leaves at most two partial results (a pair that began in an

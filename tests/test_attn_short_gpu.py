@@ -1,0 +1,59 @@
+"""The tcgen05 kernel with one CTA per (sequence, KV head) pair, which short page tables take: the longest table of the rule and the
+first beyond it for few and many pairs, one position, ragged ends, windows; against attention in 64 bits on the same bf16 values."""
+import math
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _reference(w, window):
+    B, R, hq, d = w["q"].shape
+    hkv = w["k_new"].shape[2]
+    G = hq // hkv
+    out = torch.empty((B, R, hq, d), dtype=torch.float64, device="cuda")
+    for b, n in enumerate(w["seq_lens"].tolist()):
+        pages = w["page_table"][b].long()
+        k, v = (torch.cat([w[p][pages].transpose(0, 1).reshape(hkv, -1, d)[:, :n], w[x][b].transpose(0, 1)], dim=1).double()
+                for p, x in (("k_pages", "k_new"), ("v_pages", "v_new")))
+        s = w["q"][b].double().view(R, hkv, G, d).permute(1, 0, 2, 3).reshape(hkv, R * G, d) @ k.transpose(1, 2) / math.sqrt(d)
+        pos, row = torch.arange(n + R, device="cuda"), n + torch.arange(R, device="cuda").repeat_interleave(G)
+        hidden = pos[None] > row[:, None]
+        if window:
+            hidden |= pos[None] <= row[:, None] - window
+        s.masked_fill_(hidden[None], -math.inf)
+        out[b] = (torch.softmax(s, -1) @ v).view(hkv, R, G, d).permute(1, 0, 2, 3).reshape(R, hq, d)
+    return out
+
+
+@pytest.mark.parametrize("batch,gamma,q_heads,kv_heads,pages,window", [
+    (1, 0, 1, 1, 1, 0), (1, 5, 4, 1, 16, 0), (1, 5, 4, 1, 17, 0), (3, 3, 16, 8, 20, 0), (3, 3, 16, 8, 21, 0), (12, 5, 28, 4, 24, 0), (24, 5, 28, 4, 32, 0),
+    (24, 5, 28, 4, 33, 0), (64, 7, 8, 8, 32, 0), (2, 1, 64, 2, 12, 0), (40, 2, 12, 4, 100, 100), (40, 2, 12, 4, 255, 300), (5, 6, 9, 1, 200, 40)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_against_64_bits(batch, gamma, q_heads, kv_heads, pages, window, d):
+    import paper_2505_10526_b200 as mv
+    R = gamma + 1
+    g = torch.Generator(device="cuda").manual_seed(batch + pages + d)
+    n_pages = batch * pages + 2
+    bf = dict(dtype=torch.bfloat16, device="cuda", generator=g)
+    lens = torch.randint(0, pages * 16 - R + 1, (batch,), generator=g, device="cuda").to(torch.int32)
+    lens[0] = pages * 16 - R                                 # a full table, and an empty context where there is another sequence
+    if batch > 1:
+        lens[1] = 0
+    w = dict(q=torch.randn((batch, R, q_heads, d), **bf), k_new=torch.randn((batch, R, kv_heads, d), **bf), v_new=torch.randn((batch, R, kv_heads, d), **bf),
+             k_pages=torch.randn((n_pages, kv_heads, 16, d), **bf), v_pages=torch.randn((n_pages, kv_heads, 16, d), **bf),
+             page_table=torch.randperm(n_pages, generator=g, device="cuda")[:batch * pages].view(batch, pages).to(torch.int32).contiguous(), seq_lens=lens)
+    want = _reference(w, window)
+    desc = mv.attn_desc(batch, gamma, q_heads, kv_heads, d, pages, n_pages, window=window)
+    ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda").fill_(0xff)
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    out = torch.full_like(w["q"], float("nan")); f32 = torch.full(out.shape, float("nan"), device="cuda")
+    mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, None, ws, status)
+    assert int(status.item()) == 0
+    # softmax weights rounded to bf16: at most 2^-8 each, 4e-3 of a row's norm for independent values; another 2^-8 for the bf16 output
+    assert float(((f32 - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 4e-3 and float(((out.double() - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 8e-3
+    for b, n in enumerate(lens.tolist()):                    # the block's rows are in their slots
+        for j in range(R):
+            page, at = int(w["page_table"][b, (n + j) // 16]), (n + j) % 16
+            assert torch.equal(w["k_pages"][page, :, at], w["k_new"][b, j]) and torch.equal(w["v_pages"][page, :, at], w["v_new"][b, j])
