@@ -250,7 +250,7 @@ __device__ __forceinline__ void drain_chunk(const UmmaParams& p, uint32_t taddr,
         const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
         const unsigned hit = __ballot_sync(0xffffffffu, key == kmax);
         const float mx = key_float(kmax);
-        sums[j] = (greedy || mx == -INFINITY) ? 0.f : exp2f((z - mx) * p.scale_log2);
+        sums[j] = (greedy || mx == -INFINITY) ? 0.f : ex2_ftz((z - mx) * p.scale_log2);
         if ((C == 32 ? lane : (lane >> 1)) == j) {
             mine.m = mx;
             mine.idx = mx == -INFINITY ? 0x7fffffff : warp_row0 + (__ffs(hit) - 1);   // lowest row attaining the max
@@ -390,12 +390,17 @@ __device__ __forceinline__ void stats_job64(const UmmaParams& p, uint32_t (&va)[
         // 4. exponentials relative to the column's maximum in this tile, summed over the thread's rows, then over the row groups
         float cs[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float bias = -mx[i] * p.scale_log2;
-            float acc = 0.f;
+        for (int i = 0; i < 16; i += 2) {                      // two columns at a time
+            const uint64_t scale = pack2(p.scale_log2, p.scale_log2), bias = pack2(-mx[i] * p.scale_log2, -mx[i + 1] * p.scale_log2);
+            uint64_t acc = 0ull;
 #pragma unroll
-            for (int h = 0; h < 4; ++h) acc += exp2f(fmaf(__uint_as_float(MASSV_VAL(i, h)), p.scale_log2, bias));
-            cs[i] = mx[i] == -INFINITY ? 0.f : acc;            // an all -inf column would give NaN
+            for (int h = 0; h < 4; ++h) {
+                const float2 e = unpack2(fma2(pack2(__uint_as_float(MASSV_VAL(i, h)), __uint_as_float(MASSV_VAL(i + 1, h))), scale, bias));
+                acc = add2(acc, pack2(ex2_ftz(e.x), ex2_ftz(e.y)));
+            }
+            const float2 sum = unpack2(acc);
+            cs[i] = mx[i] == -INFINITY ? 0.f : sum.x;          // an all -inf column would give NaN
+            cs[i + 1] = mx[i + 1] == -INFINITY ? 0.f : sum.y;
         }
         reduce_over_row_lanes(cs, lane, OpAdd());
         // The bias above is rounded at the size of max * scale, and every term of a column carries that rounding as one common
