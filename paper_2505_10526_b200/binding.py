@@ -100,6 +100,23 @@ def _load():
 _lib = _load()
 
 
+def _load_marshal():
+    """The calls a decoding loop makes every step go through a native module (csrc/marshal.cpp): the same checks as ``_ptr``'s on
+    every tensor, the same stream, the same entry points of the library loaded above."""
+    try:
+        from . import _marshal
+    except ImportError as e:
+        raise ImportError(f"{os.path.join(_PKG, '_marshal.so')} is missing or does not load ({e}): build it with "
+                          "`python -m paper_2505_10526_b200.build` (there is no fallback path)") from e
+    address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+    _marshal.bind(address(_lib.massv_verify_attn), address(_lib.massv_accept), address(_lib.massv_kv_commit),
+                  address(_lib.massv_sample_top_p), address(_lib.massv_tvd))
+    return _marshal
+
+
+_native = _load_marshal()
+
+
 def _strerror(status: int) -> str:
     return _lib.massv_strerror(int(status)).decode()
 
@@ -196,24 +213,15 @@ def alloc_workspace(nbytes: int, device) -> torch.Tensor:
 
 def massv_verify_attn(desc, q, k_new, v_new, k_pages, v_pages, page_table, seq_lens, out, out_f32=None, lse=None,
                       workspace=None, dev_status=None) -> None:
-    bf = torch.bfloat16
-    rc = _lib.massv_verify_attn(ctypes.byref(desc), _ptr(q, bf), _ptr(k_new, bf), _ptr(v_new, bf), _ptr(k_pages, bf),
-                                _ptr(v_pages, bf), _ptr(page_table, torch.int32), _ptr(seq_lens, torch.int32),
-                                _ptr(out, bf), _ptr(out_f32, torch.float32), _ptr(lse, torch.float32),
-                                _ptr(workspace), workspace.numel() if workspace is not None else 0,
-                                _ptr(dev_status, torch.int32), _stream())
+    rc = _native.verify_attn(desc, q, k_new, v_new, k_pages, v_pages, page_table, seq_lens, out, out_f32, lse, workspace, dev_status)
     if rc != 0:
         raise MassvError(rc, "massv_verify_attn")
 
 
 def massv_accept(desc, hidden, lm_head, draft_tokens, draft_probs, u_accept, u_sample, out_tokens, accept_len,
                  logits_out=None, probs_out=None, workspace=None, dev_status=None) -> None:
-    bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32
-    rc = _lib.massv_accept(ctypes.byref(desc), _ptr(hidden, bf), _ptr(lm_head, bf), _ptr(draft_tokens, i32),
-                           _ptr(draft_probs, f32), _ptr(u_accept, f32), _ptr(u_sample, f32), _ptr(out_tokens, i32),
-                           _ptr(accept_len, i32), _ptr(logits_out, f32), _ptr(probs_out, f32),
-                           _ptr(workspace), workspace.numel() if workspace is not None else 0,
-                           _ptr(dev_status, i32), _stream())
+    rc = _native.accept(desc, hidden, lm_head, draft_tokens, draft_probs, u_accept, u_sample, out_tokens, accept_len, logits_out,
+                        probs_out, workspace, dev_status)
     if rc != 0:
         raise MassvError(rc, "massv_accept")
 
@@ -237,10 +245,7 @@ def massv_tvd_workspace_size(desc: AcceptDesc) -> int:
 
 
 def massv_tvd(desc, logits, draft_probs, tvd_out, accept_prob_out=None, workspace=None, dev_status=None) -> None:
-    f32 = torch.float32
-    rc = _lib.massv_tvd(ctypes.byref(desc), _ptr(logits, f32), _ptr(draft_probs, f32), _ptr(tvd_out, f32),
-                        _ptr(accept_prob_out, f32), _ptr(workspace), workspace.numel() if workspace is not None else 0,
-                        _ptr(dev_status, torch.int32), _stream())
+    rc = _native.tvd(desc, logits, draft_probs, tvd_out, accept_prob_out, workspace, dev_status)
     if rc != 0:
         raise MassvError(rc, "massv_tvd")
 
@@ -266,10 +271,8 @@ def massv_tvd_histogram(tvd, counts) -> None:
 
 def massv_sample_top_p(logits, u, tokens, temperature, top_p, probs_out=None, dev_status=None) -> None:
     """Nucleus sampling of softmax(logits / temperature), one draw per row (logits fp32 [rows, V])."""
-    f32, i32 = torch.float32, torch.int32
     rows, vocab = logits.shape
-    rc = _lib.massv_sample_top_p(rows, vocab, float(temperature), float(top_p), _ptr(logits, f32), _ptr(u, f32),
-                                 _ptr(tokens, i32), _ptr(probs_out, f32), _ptr(dev_status, i32), _stream())
+    rc = _native.sample_top_p(rows, vocab, temperature, top_p, logits, u, tokens, probs_out, dev_status)
     if rc != 0:
         raise MassvError(rc, "massv_sample_top_p")
 
@@ -351,7 +354,6 @@ def massv_shard_set_token(desc, world, state, tokens_all, out_tokens, dev_status
 
 
 def massv_kv_commit(batch, gamma, accept_len, seq_lens, dev_status=None) -> None:
-    rc = _lib.massv_kv_commit(batch, gamma, _ptr(accept_len, torch.int32), _ptr(seq_lens, torch.int32),
-                              _ptr(dev_status, torch.int32), _stream())
+    rc = _native.kv_commit(batch, gamma, accept_len, seq_lens, dev_status)
     if rc != 0:
         raise MassvError(rc, "massv_kv_commit")

@@ -1,9 +1,10 @@
-"""Compile the CUDA sources into ``libmassv.so`` for sm_100a with nvcc."""
+"""Compile the CUDA sources into ``libmassv.so`` for sm_100a with nvcc, and the binding's argument marshalling with g++."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
@@ -14,6 +15,7 @@ SOURCES = ["api.cu", "attn.cu", "attn_umma.cu", "lm_head.cu", "accept.cu", "acce
 
 TEST_LIB = os.path.join(PKG, "libmassv_testhooks.so")
 DEBUG_LIB = os.path.join(PKG, "libmassv_debug.so")
+MARSHAL = os.path.join(PKG, "_marshal.so")
 
 
 def _stale(lib=LIB) -> bool:
@@ -42,16 +44,31 @@ def _compile(out, extra, verbose=False):
 VARIANTS = {LIB: [], TEST_LIB: ["-DMASSV_TEST_HOOKS", "-DMASSV_SPIN_LIMIT=65536u"], DEBUG_LIB: ["-DMASSV_DEBUG"]}
 
 
+def _marshal_command():
+    """The extension module against torch's own headers and libraries (found without importing torch: that takes seconds)."""
+    import importlib.util
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    include = [sysconfig.get_paths()["include"], os.path.join(torch_dir, "include"),
+               os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
+    return ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", INCLUDE] + [x for d in include for x in ("-isystem", d)] +
+            ["-o", MARSHAL, os.path.join(CSRC, "marshal.cpp"), "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+
+
 def build_all(force: bool = False):
-    """The library and its two test variants, the stale ones compiled side by side."""
-    procs = [(lib, subprocess.Popen(_command(lib, extra))) for lib, extra in VARIANTS.items() if force or _stale(lib)]
-    for lib, proc in procs:
+    """The library, its two test variants and the marshalling module, the stale ones compiled side by side."""
+    commands = {lib: _command(lib, extra) for lib, extra in VARIANTS.items()}
+    commands[MARSHAL] = _marshal_command()
+    procs = [(out, subprocess.Popen(cmd)) for out, cmd in commands.items() if force or _stale(out)]
+    for out, proc in procs:
         if proc.wait() != 0:
-            raise subprocess.CalledProcessError(proc.returncode, "nvcc -o " + lib)
-    return list(VARIANTS)
+            raise subprocess.CalledProcessError(proc.returncode, "compiler -o " + out)
+    return list(commands)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    if force or _stale(MARSHAL):
+        subprocess.run(_marshal_command(), check=True)
     if not (force or _stale()):
         return LIB
     return _compile(LIB, [], verbose)

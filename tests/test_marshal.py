@@ -1,0 +1,42 @@
+"""What the native argument marshalling refuses is what the checks in Python refused: tensors off the GPU, other types, gaps,
+things that are no tensors, the other call's descriptor."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+
+
+@pytest.fixture(scope="module")
+def mv():
+    entry.build()
+    import paper_2505_10526_b200 as pkg
+    return pkg
+
+
+def test_refused_without_a_gpu(mv):
+    a, c = mv.attn_desc(1, 1, 1, 1, 64, 1, 1), mv.accept_desc(1, 1, 64, 64, 1.0)
+    f, i, b = torch.zeros(64), torch.zeros(64, dtype=torch.int32), torch.zeros(64, dtype=torch.bfloat16)
+    with pytest.raises(ValueError, match="CUDA device"):
+        mv.massv_verify_attn(a, b, b, b, b, b, i, i, b)
+    with pytest.raises(ValueError, match="CUDA device"):
+        mv.massv_tvd(c, f, f, f)
+    with pytest.raises(ValueError, match="CUDA device"):
+        mv.massv_sample_top_p(f.view(1, 64), f, i, 1.0, 0.9)
+    with pytest.raises(ValueError, match="CUDA device"):
+        mv.massv_kv_commit(1, 1, i, i)
+    with pytest.raises(AttributeError):
+        mv.massv_kv_commit(1, 1, None, 7)
+    for wrong in (a, 3, None):
+        with pytest.raises(TypeError):
+            mv.massv_accept(wrong, b, b, i, f, f, f, i, i)
+
+
+@pytest.mark.gpu
+def test_refused_on_the_gpu(mv):
+    lens = torch.zeros((4, 2), dtype=torch.int32, device="cuda")
+    with pytest.raises(ValueError, match="contiguous"):
+        mv.massv_kv_commit(4, 1, lens[:, 0], lens[:, 1])
+    with pytest.raises(ValueError, match="expected torch.int32, got torch.float32"):
+        mv.massv_kv_commit(4, 1, lens[0].float(), lens[1])
+    with pytest.raises(mv.MassvError):
+        mv.massv_kv_commit(0, 1, lens[0].contiguous(), lens[1].contiguous())
