@@ -839,10 +839,10 @@ static long pair_tokens(const AttnParams& p) {
 // 9 - 10 us and more the more pairs it cuts, so the line between them rises with the number of pairs.  Call times, balanced -> one
 // CTA per pair, head_dim 128, lengths from a quarter of the table to all of it: 1 x 4 pairs of up to 128 positions 10.2 -> 7.7 us,
 // 16 x 4 of 128 14.5 -> 9.1, of 256 14.6 -> 12.0, of 512 17.0 -> 17.7; 64 x 4 of 256 26.8 -> 13.7, of 512 30.5 -> 20.1, of 1,024
-// 36 -> 32; 64 x 8 of 512 50 -> 38.
+// 36 -> 32; 64 x 8 of 512 50 -> 38; 1 x 4 of 250 11.2 -> 12.1, so that few pairs take three tiles at most.
 static bool one_piece_per_pair(const AttnParams& p) {
     const long pairs = (long)p.B * p.Hkv, tiles = (pair_tokens(p) + 63) / 64;
-    return !p.chunk_forced && p.max_pages <= kMaxChunkPages && tiles <= 4 + (pairs < 96 ? pairs / 24 : 4);
+    return !p.chunk_forced && p.max_pages <= kMaxChunkPages && tiles <= (pairs < 8 ? 3 : 4) + (pairs < 96 ? pairs / 24 : 4);
 }
 
 // Balanced schedule or chunk grid for the warp-MMA kernel at head_dim 256.  The balanced one wins wherever the grid would cut
