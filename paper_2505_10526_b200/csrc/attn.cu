@@ -436,6 +436,27 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 // all others up.  64 x 8 pairs of 1 - 512 positions: 81 us with 0 units, 58, 51, 50 and 50 with 2, 4, 6 and 8; 32 x 8 of
 // 2k - 8k: 225, 225, 223, 223, 231; the same with a window of 1,024: 61.3, 62.1, 62.0, 63.3, 63.7.
 constexpr int kPairUnits = 4;
+constexpr int kPairSlack = 6;              // (see flat_range)
+// By one warp: range[0], range[1] = this CTA's units of the line, range[2] = units per CTA.  Equal ranges; but a pair per CTA
+// (range[2] = 0) where the longest pair is at most kPairSlack units (fewer for short ranges) longer than a range - the window of a local
+// layer, contexts of one length - so that nothing is cut, written as pieces and merged.  Call times, equal ranges -> a pair per CTA: 256 pairs
+// of 12 rows, window 1,024 (5 units) 57 -> 53 us, window 512 38 -> 33, 1,000 positions 57 -> 46; 128 pairs of 24 rows, window 1,024 49 -> 45,
+// 4,000 positions (17 units) 127 -> 134.  (The tcgen05 kernel keeps its ranges: the longer its runs, the further its running reference leaves
+// the weights of later tiles from exact ones.)
+__device__ __forceinline__ void flat_range(const int* cum, int batch, int kv_heads, int longest, int* range) {
+    __syncwarp();
+    if ((threadIdx.x & 31) != 0) return;
+    const int total = cum[batch] * kv_heads, ctas = (int)gridDim.x, at = (int)blockIdx.x;
+    int per = max(1, (total + ctas - 1) / ctas);
+    int first = min(total, at * per), end = min(total, first + per);
+    if (batch * kv_heads <= ctas && longest <= per + min(kPairSlack, 1 + per / kPairSlack)) {
+        const int b = at / kv_heads, g = at % kv_heads, n = b < batch ? cum[b + 1] - cum[b] : 0;
+        first = b < batch ? cum[b] * kv_heads + g * n : total;
+        end = first + n;
+        per = 0;
+    }
+    range[0] = first; range[1] = end; range[2] = per;
+}
 template <int D, int MT, int TILE>
 struct FlatCfg {
     static constexpr int kTS = 2;                          // warps that share 16 query rows, each with half of a tile's tokens
@@ -462,7 +483,7 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[E], empty_bar[E];
     __shared__ float s_m[NW][16], s_l[NW][16];
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, s_range[3];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int G = p.Hq / p.Hkv, rows = G * p.R;
@@ -494,8 +515,8 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
     if (warp == 0) {
         const int per = (p.B + 31) / 32;
         const int i0 = min(p.B, lane * per), i1 = min(p.B, i0 + per);
-        int local = 0;
-        for (int i = i0; i < i1; ++i) local += s_cum[i + 1];
+        int local = 0, longest = 0;
+        for (int i = i0; i < i1; ++i) { local += s_cum[i + 1]; longest = max(longest, s_cum[i + 1]); }
         int incl = local;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -504,15 +525,14 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         }
         int run = incl - local;
         for (int i = i0; i < i1; ++i) { run += s_cum[i + 1]; s_cum[i + 1] = run; }
+        flat_range(s_cum, p.B, p.Hkv, __reduce_max_sync(0xffffffffu, longest), s_range);
     }
     __syncthreads();
-    const int total = s_cum[p.B] * p.Hkv;
-    const int per_cta = max(1, (total + (int)gridDim.x - 1) / (int)gridDim.x);
     if (blockIdx.x == 0) {          // what the merge kernel needs to find the pieces of a pair
         for (int i = threadIdx.x; i <= p.B; i += blockDim.x) p.flat_meta[2 + i] = s_cum[i];
-        if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = kPairUnits; }
+        if (threadIdx.x == 0) { p.flat_meta[0] = s_range[2]; p.flat_meta[1] = kPairUnits; }
     }
-    const int f_first = min(total, (int)blockIdx.x * per_cta), f_end = min(total, f_first + per_cta);
+    const int f_first = s_range[0], f_end = s_range[1];
     volatile int* abort_ptr = &abort_flag;
 
     // Piece of work at unit f of the line: a run of tiles of one pair, up to this CTA's end (none where that lies ahead of them).

@@ -57,3 +57,41 @@ def test_against_64_bits(batch, gamma, q_heads, kv_heads, pages, window, d):
         for j in range(R):
             page, at = int(w["page_table"][b, (n + j) // 16]), (n + j) % 16
             assert torch.equal(w["k_pages"][page, :, at], w["k_new"][b, j]) and torch.equal(w["v_pages"][page, :, at], w["v_new"][b, j])
+
+
+@pytest.mark.parametrize("batch,q_heads,kv_heads,base,longer,window", [
+    (32, 16, 8, 1500, 500, 1024), (37, 16, 8, 1000, 0, 0), (32, 16, 8, 1000, 128, 0), (32, 16, 8, 1000, 1000, 0), (18, 32, 8, 1100, 300, 512), (64, 16, 4, 700, 64, 0),
+    (1, 16, 8, 520, 0, 512)])
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_a_pair_per_cta(batch, q_heads, kv_heads, base, longer, window, d):
+    """Windows and equal lengths, where the balanced schedule of head_dim 256 gives every pair a CTA, one sequence longer by less and by
+    more than the slack, a sequence without room for its block (skipped, and reported)."""
+    import paper_2505_10526_b200 as mv
+    gamma, R = 5, 6
+    g = torch.Generator(device="cuda").manual_seed(batch + base + d)
+    pages = (base + longer + R + 15) // 16
+    n_pages = batch * pages
+    bf = dict(dtype=torch.bfloat16, device="cuda", generator=g)
+    lens = torch.full((batch,), base, dtype=torch.int32, device="cuda")
+    lens[batch // 2] += longer
+    skipped = batch > 8
+    w = dict(q=torch.randn((batch, R, q_heads, d), **bf), k_new=torch.randn((batch, R, kv_heads, d), **bf), v_new=torch.randn((batch, R, kv_heads, d), **bf),
+             k_pages=torch.randn((n_pages, kv_heads, 16, d), **bf), v_pages=torch.randn((n_pages, kv_heads, 16, d), **bf),
+             page_table=torch.randperm(n_pages, generator=g, device="cuda").view(batch, pages).to(torch.int32).contiguous(), seq_lens=lens)
+    want = _reference(w, window)
+    if skipped:
+        lens[3] = pages * 16
+    desc = mv.attn_desc(batch, gamma, q_heads, kv_heads, d, pages, n_pages, window=window)
+    ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda").fill_(0xff)
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    outs = []
+    for _ in range(2):
+        out = torch.full_like(w["q"], float("nan")); f32 = torch.full(out.shape, float("nan"), device="cuda")
+        mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, None, ws, status)
+        outs.append(f32)
+    keep = [b for b in range(batch) if not (skipped and b == 3)]
+    assert (int(status.item()) != 0) == skipped
+    # as above
+    assert float(((outs[0][keep] - want[keep]).norm(dim=-1) / want[keep].norm(dim=-1)).max()) < 4e-3
+    assert torch.equal(outs[0][keep], outs[1][keep])
+    assert not skipped or bool(outs[0][3].isnan().all())
