@@ -899,6 +899,7 @@ cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream) {
             AttnParams q = p;
             q.kv_chunk = (p.max_pages * kPageSize + kChunkAlign - 1) / kChunkAlign * kChunkAlign;
             q.max_chunks = 1;
+            q.follow_tiles = true;
             e = launch_attn_umma(q, mk, mv, stream, false, &launched, nullptr);
             if (e != cudaSuccess) return e;
             if (hooks.attn_stop && cudaEventRecord(hooks.attn_stop, stream) != cudaSuccess) return cudaGetLastError();

@@ -46,7 +46,7 @@ constexpr int kProducerWarp = 0, kMmaWarp = 1, kHelperWarp = 6;
 constexpr int kUmmaMaxChunkPages = 256;
 constexpr int kFlatMaxBatch = 1024;    // sequences the flat schedule can index in shared memory
 constexpr float kRescaleThreshold = 8.f;   // log2 units
-constexpr float kRescaleBelow = 6.f;       // how far the reference may follow a tile's maximum down
+constexpr float kRescaleBelow = 6.f;       // how far below the running maximum the reference may follow a tile's maximum (follow_tiles)
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -534,16 +534,19 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         // block row of each of this thread's two query rows (padding rows behave like the last block row)
         const int j0 = r0 < rows ? r0 / G : p.R - 1, j1 = r1 < rows ? r1 / G : p.R - 1;
         const float scale_log2 = p.scale * 1.4426950408889634f;
-        // A short pair in one piece: the reference follows every tile's maximum, so that the largest weight of each tile is exactly 1 in
-        // bf16, as it is where the balanced line cuts such a pair into pieces of a tile or two (262 positions at head_dim 64, error of
-        // the output against 64 bits: 2.1e-3 in pieces, 2.4e-3 in one run with a running reference).
-        const bool every_tile = !FLAT && p.max_chunks == 1 && !p.chunk_forced;
+        // Short pairs in one piece (follow_tiles): the reference of the weights follows every tile's maximum, so that the largest weight of a
+        // tile is exactly 1 in bf16, as it is where the balanced line cuts such a pair into pieces of a tile or two (262 positions at
+        // head_dim 64, error of the output against 64 bits: 2.1e-3 in pieces, 2.4e-3 in one run with a running reference).  It stays within
+        // kRescaleBelow of the row's running maximum, so that O and l, which are relative to it, cannot outgrow their range however
+        // far the maxima fall from tile to tile; only a tile further below has no weight of 1.
+        const bool follow = !FLAT && p.follow_tiles;
         uint8_t* p_row0 = p_smem + r0 * 128 + 4 * (lane & 3);   // this thread's 4 bytes of unit 0 of row r0 (before the swizzle)
         bool ok = true;
         int tau_base = 0;
         for (int seg = 0; ok && next_segment(sg); ++seg) {
             const int L = sg.L, b = sg.b, g = sg.g, n_tiles = sg.n_tiles, n_ctx = L + p.R;
             float m_ref[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+            float m_top[2] = {-INFINITY, -INFINITY};            // follow_tiles: running maxima
             for (int t = 0; t < n_tiles && ok; ++t) {
                 const int tau = tau_base + t, buf = tau & 1;
                 if (!mbar_wait_warp(&s_full_bar[buf], ((uint32_t)(tau >> 1)) & 1u, abort_ptr)) { ok = false; break; }
@@ -593,14 +596,28 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                 mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
                 mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
                 mx0 *= scale_log2; mx1 *= scale_log2;             // log2 domain (the scale is positive)
-                // The reference maximum of a row moves only when the row's maximum has outgrown it by the
-                // threshold (or when it is first set); O and l are then rescaled to the new reference.
+                // The reference of a row moves when the row's maximum has outgrown it by the threshold, with follow_tiles to every
+                // tile's maximum (within its bound), and when it is first set; O and l are then rescaled to the new reference.
                 float f0 = 1.f, f1 = 1.f;
-                bool grow = false;
-                if (m_ref[0] == -INFINITY) m_ref[0] = mx0;
-                else if (every_tile ? mx0 != m_ref[0] && mx0 > m_ref[0] - kRescaleBelow : mx0 > m_ref[0] + kRescaleThreshold) { f0 = exp2f(m_ref[0] - mx0); m_ref[0] = mx0; grow = true; }
-                if (m_ref[1] == -INFINITY) m_ref[1] = mx1;
-                else if (every_tile ? mx1 != m_ref[1] && mx1 > m_ref[1] - kRescaleBelow : mx1 > m_ref[1] + kRescaleThreshold) { f1 = exp2f(m_ref[1] - mx1); m_ref[1] = mx1; grow = true; }
+                bool moved = false;
+                auto move_reference = [&](float mx, float& ref, float& top, float& f) {
+                    float to = ref;
+                    if (follow) {
+                        top = fmaxf(top, mx);
+                        to = fmaxf(mx, top - kRescaleBelow);
+                    } else if (mx > ref + kRescaleThreshold) {
+                        to = mx;
+                    }
+                    if (ref == -INFINITY) {
+                        ref = mx;
+                    } else if (to != ref) {
+                        f = exp2f(ref - to);
+                        ref = to;
+                        moved = true;
+                    }
+                };
+                move_reference(mx0, m_ref[0], m_top[0], f0);
+                move_reference(mx1, m_ref[1], m_top[1], f1);
                 const float ms0 = m_ref[0] == -INFINITY ? 0.f : -m_ref[0], ms1 = m_ref[1] == -INFINITY ? 0.f : -m_ref[1];
                 float la[4] = {0.f, 0.f, 0.f, 0.f}, lb[4] = {0.f, 0.f, 0.f, 0.f};      // independent partial sums
                 uint32_t pk[TILE / 64][16];       // bf16 pairs: [2k] = row r0, [2k+1] = row r1, tokens 8k + 2*(lane%4) + {0,1}
@@ -622,7 +639,7 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                 // P and O belong to the tensor core until P V of tile t-1 is done; P V of tile t cannot
                 // start before this warp has published P below.
                 if (t >= 1 && !mbar_wait_warp(&pv_done_bar[(tau - 1) & 1], ((uint32_t)((tau - 1) >> 1)) & 1u, abort_ptr)) { ok = false; break; }
-                if (__any_sync(0xffffffffu, grow)) {
+                if (__any_sync(0xffffffffu, moved)) {
                     tc_fence_after();
 #pragma unroll 1
                     for (int c0 = 0; c0 < D; c0 += 64) {

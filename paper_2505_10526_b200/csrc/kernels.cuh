@@ -25,6 +25,7 @@ struct AttnParams {
     int32_t* dev_status;
     int path;          // 0: choose by shape, 1: warp-level MMA kernel, 2: tcgen05 kernel
     bool chunk_forced; // the caller fixed kv_chunk: keep the (chunk, KV head, sequence) grid
+    bool follow_tiles = false; // tcgen05 kernel, short pairs in one piece: the softmax reference follows every tile's maximum
     // flat schedules: two partial slots per resident CTA, and what the merge needs
     float* flat_part_o;    // [kFlatMaxCtas * 2, rows_pad, d]
     float* flat_part_ml;   // [kFlatMaxCtas * 2, rows_pad, 2]

@@ -95,3 +95,37 @@ def test_a_pair_per_cta(batch, q_heads, kv_heads, base, longer, window, d):
     assert float(((outs[0][keep] - want[keep]).norm(dim=-1) / want[keep].norm(dim=-1)).max()) < 4e-3
     assert torch.equal(outs[0][keep], outs[1][keep])
     assert not skipped or bool(outs[0][3].isnan().all())
+
+
+@pytest.mark.parametrize("step", [-9.0, -5.9, -3.0, 3.0, 5.9, 9.0])
+@pytest.mark.parametrize("batch,kv_heads,pages,window", [(1, 4, 12, 0), (24, 4, 32, 0), (24, 4, 32, 300), (1025, 2, 120, 0)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_scores_that_fall_or_rise_from_tile_to_tile(batch, kv_heads, pages, window, step, d):
+    """Tile maxima that move by `step` binary orders from one tile of 64 positions to the next, over the one-piece route (3 and 8 tiles) and,
+    with more sequences than the balanced schedule takes, over 30 tiles in one run: the weights' reference goes with them, and what it
+    has left behind must stay in range."""
+    import paper_2505_10526_b200 as mv
+    gamma, R, G = 1, 2, 2
+    g = torch.Generator(device="cuda").manual_seed(batch + pages + d)
+    n_pages = batch * pages
+    bf = dict(dtype=torch.bfloat16, device="cuda", generator=g)
+    table = torch.randperm(n_pages, generator=g, device="cuda").view(batch, pages).to(torch.int32).contiguous()
+    # q = 8 in every element, so a key of constant x scores 8 d x / sqrt(d) log2(e) binary orders; the line through zero in the middle
+    tile = torch.arange(pages, device="cuda") // 4
+    level = ((tile - tile[-1] / 2.0) * step / (8.0 * math.sqrt(d) * math.log2(math.e))).repeat(batch)
+    keys = 0.02 * torch.randn((n_pages, kv_heads, 16, d), device="cuda", generator=g)
+    keys[table.view(-1).long()] += level[:, None, None, None]
+    w = dict(q=torch.full((batch, R, kv_heads * G, d), 8.0, dtype=torch.bfloat16, device="cuda"),
+             k_new=torch.full((batch, R, kv_heads, d), float(level[-1]), dtype=torch.bfloat16, device="cuda"), v_new=torch.randn((batch, R, kv_heads, d), **bf),
+             k_pages=keys.to(torch.bfloat16), v_pages=torch.randn((n_pages, kv_heads, 16, d), **bf), page_table=table,
+             seq_lens=torch.full((batch,), pages * 16 - R, dtype=torch.int32, device="cuda"))
+    del keys
+    want = _reference(w, window)
+    desc = mv.attn_desc(batch, gamma, kv_heads * G, kv_heads, d, pages, n_pages, window=window)
+    ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda").fill_(0xff)
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    out = torch.full_like(w["q"], float("nan")); f32 = torch.full(out.shape, float("nan"), device="cuda")
+    mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, f32, None, ws, status)
+    assert int(status.item()) == 0
+    # as above: weights rounded to bf16, each by at most 2^-9
+    assert float(((f32 - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 4e-3
