@@ -850,8 +850,8 @@ bool attn_use_umma(const AttnParams& p) {
 
 // The most positions a (sequence, KV head) pair can need.
 static long pair_tokens(const AttnParams& p) {
-    const long tokens = (long)p.max_pages * kPageSize;
-    return p.window > 0 && p.window + p.R + 64 < tokens ? p.window + p.R + 64 : tokens;
+    const long tokens = (long)p.max_pages * kPageSize, seen = (long)p.window + p.R + 64;       // (a window may be any int32)
+    return p.window > 0 && seen < tokens ? seen : tokens;
 }
 
 // tcgen05 kernel: one CTA per pair where pairs are short, instead of ranges of the line of tiles: nothing to deal out, no pieces and

@@ -122,3 +122,10 @@ def test_attention_refuses_more_chunks_than_the_merge_can_index(mv):
     assert lib.massv_verify_attn(ctypes.byref(d), fake, fake, fake, fake, fake, fake, fake, fake, None, None, fake, 1 << 30, None, None) == -2
     ok = mv.attn_desc(1, 5, 4, 1, 64, 4096, 5000, kv_chunk=64)         # exactly 1024 chunks
     assert mv.massv_verify_attn_workspace_size(ok) > 0
+
+
+@pytest.mark.parametrize("pages", [1, 256, 5000])
+def test_a_window_longer_than_any_context_is_no_window(mv, pages):
+    """Windows up to 2^31 - 1 are accepted, and one that no context fills leaves the split of the scan, and so the workspace, as without."""
+    sizes = [mv.massv_verify_attn_workspace_size(mv.attn_desc(3, 3, 8, 4, 128, pages, 3 * pages, window=w)) for w in (0, 2 ** 31 - 64, 2 ** 31 - 1)]
+    assert sizes[0] > 0 and sizes[1] == sizes[2] == sizes[0]

@@ -129,3 +129,28 @@ def test_scores_that_fall_or_rise_from_tile_to_tile(batch, kv_heads, pages, wind
     assert int(status.item()) == 0
     # as above: weights rounded to bf16, each by at most 2^-9
     assert float(((f32 - want).norm(dim=-1) / want.norm(dim=-1)).max()) < 4e-3
+
+
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_a_window_longer_than_any_context(d):
+    """A window of 2^31 - 1 positions hides nothing, and takes the route of no window."""
+    import paper_2505_10526_b200 as mv
+    batch, gamma, q_heads, kv_heads, pages = 3, 3, 8, 4, 256
+    R, n_pages = gamma + 1, batch * pages
+    g = torch.Generator(device="cuda").manual_seed(d)
+    bf = dict(dtype=torch.bfloat16, device="cuda", generator=g)
+    w = dict(q=torch.randn((batch, R, q_heads, d), **bf), k_new=torch.randn((batch, R, kv_heads, d), **bf), v_new=torch.randn((batch, R, kv_heads, d), **bf),
+             k_pages=torch.randn((n_pages, kv_heads, 16, d), **bf), v_pages=torch.randn((n_pages, kv_heads, 16, d), **bf),
+             page_table=torch.randperm(n_pages, generator=g, device="cuda").view(batch, pages).to(torch.int32).contiguous(),
+             seq_lens=torch.tensor([pages * 16 - R, 2000, 77], dtype=torch.int32, device="cuda"))
+    outs, launches = [], []
+    for window in (0, 2 ** 31 - 1, pages * 16):
+        desc = mv.attn_desc(batch, gamma, q_heads, kv_heads, d, pages, n_pages, window=window)
+        ws = mv.alloc_workspace(mv.massv_verify_attn_workspace_size(desc), "cuda")
+        out = torch.empty_like(w["q"])
+        before = mv.massv_launch_count()
+        mv.massv_verify_attn(desc, w["q"], w["k_new"], w["v_new"], w["k_pages"], w["v_pages"], w["page_table"], w["seq_lens"], out, None, None, ws, None)
+        launches.append(mv.massv_launch_count() - before)
+        outs.append(out)
+    assert launches[0] == launches[1] == launches[2]
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
