@@ -438,7 +438,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 constexpr int kPairUnits = 4;
 constexpr int kPairSlack = 6;              // (see flat_range)
 // By one warp: range[0], range[1] = this CTA's units of the line, range[2] = units per CTA.  Equal ranges; but a pair per CTA
-// (range[2] = 0) where the longest pair is at most kPairSlack units (fewer for short ranges) longer than a range - the window of a local
+// (range[2] = kFlatWholePairs) where the longest pair is at most kPairSlack units (fewer for short ranges) longer than a range - the window of a local
 // layer, contexts of one length - so that nothing is cut, written as pieces and merged.  Call times, equal ranges -> a pair per CTA: 256 pairs
 // of 12 rows, window 1,024 (5 units) 57 -> 53 us, window 512 38 -> 33, 1,000 positions 57 -> 46; 128 pairs of 24 rows, window 1,024 49 -> 45,
 // 4,000 positions (17 units) 127 -> 134.  (The tcgen05 kernel keeps its ranges: the longer its runs, the further its running reference leaves
@@ -453,7 +453,7 @@ __device__ __forceinline__ void flat_range(const int* cum, int batch, int kv_hea
         const int b = at / kv_heads, g = at % kv_heads, n = b < batch ? cum[b + 1] - cum[b] : 0;
         first = b < batch ? cum[b] * kv_heads + g * n : total;
         end = first + n;
-        per = 0;
+        per = kFlatWholePairs;
     }
     range[0] = first; range[1] = end; range[2] = per;
 }
@@ -472,7 +472,9 @@ struct FlatCfg {
     static constexpr int kSmem = kStages * kStageBytes + kQBytes + 1024;      // and (B + 1) ints
 };
 
-template <int D, int MT, int TILE>
+// WHOLE: a pair per CTA is possible, and flat_range decides.  (A kernel of its own: the decision costs a short call 0.2 us, 4 x 8 pairs of
+// 41 - 65 positions 11.20 -> 11.40.)
+template <int D, int MT, int TILE, bool WHOLE>
 __global__ void __launch_bounds__((FlatCfg<D, MT, TILE>::kWarps + 1) * 32, FlatCfg<D, MT, TILE>::kCtasPerSm)
 attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_q,
                  const AttnParams p) {
@@ -525,14 +527,16 @@ attn_flat_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         }
         int run = incl - local;
         for (int i = i0; i < i1; ++i) { run += s_cum[i + 1]; s_cum[i + 1] = run; }
-        flat_range(s_cum, p.B, p.Hkv, __reduce_max_sync(0xffffffffu, longest), s_range);
+        if constexpr (WHOLE) flat_range(s_cum, p.B, p.Hkv, __reduce_max_sync(0xffffffffu, longest), s_range);
     }
     __syncthreads();
+    const int total = s_cum[p.B] * p.Hkv;
+    const int per_cta = WHOLE ? s_range[2] : max(1, (total + (int)gridDim.x - 1) / (int)gridDim.x);
     if (blockIdx.x == 0) {          // what the merge kernel needs to find the pieces of a pair
         for (int i = threadIdx.x; i <= p.B; i += blockDim.x) p.flat_meta[2 + i] = s_cum[i];
-        if (threadIdx.x == 0) { p.flat_meta[0] = s_range[2]; p.flat_meta[1] = kPairUnits; }
+        if (threadIdx.x == 0) { p.flat_meta[0] = per_cta; p.flat_meta[1] = kPairUnits; }
     }
-    const int f_first = s_range[0], f_end = s_range[1];
+    const int f_first = WHOLE ? s_range[0] : min(total, (int)blockIdx.x * per_cta), f_end = WHOLE ? s_range[1] : min(total, f_first + per_cta);
     volatile int* abort_ptr = &abort_flag;
 
     // Piece of work at unit f of the line: a run of tiles of one pair, up to this CTA's end (none where that lies ahead of them).
@@ -810,14 +814,19 @@ cudaError_t launch_flat(const AttnParams& p, const CUtensorMap& mk, const CUtens
     // lower it between another thread's attribute and launch.)
     constexpr int kMaxSmem = Cfg::kSmem + (kFlatMaxBatchMeta + 1) * (int)sizeof(int);
     static_assert(kMaxSmem <= 225 * 1024, "ring, query rows and tile counts fit shared memory");
-    cudaError_t e = cudaFuncSetAttribute(attn_flat_kernel<D, MT, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    if (e != cudaSuccess) return e;
     *ctas = device_sm_count() * Cfg::kCtasPerSm;
     if (*ctas > kFlatMaxCtas) *ctas = kFlatMaxCtas;
+    // A range is no longer than pairs / CTAs of the longest pair, which has at least kPairUnits + 1 units: with 3 pairs or fewer for 5 CTAs no
+    // lengths meet flat_range's condition for a pair per CTA, with more pairs than CTAs none can.
+    const long pairs = (long)p.B * p.Hkv;
+    const bool whole = pairs <= *ctas && 5 * pairs > 3L * *ctas;
+    const auto kernel = whole ? attn_flat_kernel<D, MT, TILE, true> : attn_flat_kernel<D, MT, TILE, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (e != cudaSuccess) return e;
     // the query rows as a [B * R * Hq, D] matrix; a box is the G adjacent heads of one block row
     CUtensorMap mq;
     if (!make_tensor_map_bf16_2d(&mq, p.q, (uint64_t)p.B * p.R * p.Hq, D, (uint32_t)(p.Hq / p.Hkv))) return cudaErrorInvalidValue;
-    return launch_pdl(attn_flat_kernel<D, MT, TILE>, dim3(*ctas), dim3((Cfg::kWarps + 1) * 32), smem, stream, mk, mv, mq, p);
+    return launch_pdl(kernel, dim3(*ctas), dim3((Cfg::kWarps + 1) * 32), smem, stream, mk, mv, mq, p);
 }
 
 template <int D>

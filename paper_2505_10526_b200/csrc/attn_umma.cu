@@ -784,7 +784,6 @@ __global__ void __launch_bounds__(kFlatCombineThreads) attn_flat_combine_kernel(
     pdl_wait();
     pdl_trigger();
     const int per_cta = p.flat_meta[0], ahead = p.flat_meta[1];     // units of a pair ahead of its first tile
-    if (per_cta == 0) return;                      // every pair had a CTA to itself
     const int cum_b = p.flat_meta[2 + b], n_b = p.flat_meta[2 + b + 1] - cum_b;
     if (n_b <= 0) return;
     const int start = cum_b * p.Hkv + g * n_b, end = start + n_b;

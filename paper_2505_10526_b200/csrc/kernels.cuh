@@ -29,10 +29,11 @@ struct AttnParams {
     // flat schedules: two partial slots per resident CTA, and what the merge needs
     float* flat_part_o;    // [kFlatMaxCtas * 2, rows_pad, d]
     float* flat_part_ml;   // [kFlatMaxCtas * 2, rows_pad, 2]
-    int32_t* flat_meta;    // [0] units per CTA (0: every pair has a CTA to itself), [1] units of a pair ahead of its tiles, [2 + b] units of sequences 0 .. b-1 (per KV head); a tile is a unit
+    int32_t* flat_meta;    // [0] units per CTA (kFlatWholePairs: every pair has a CTA to itself), [1] units of a pair ahead of its tiles, [2 + b] units of sequences 0 .. b-1 (per KV head); a tile is a unit
 };
 constexpr int kFlatMaxCtas = 320;      // resident CTAs of the flat schedule (two per SM)
 constexpr int kFlatMaxBatchMeta = 1024;
+constexpr int kFlatWholePairs = 0x7fffffff;   // more units than any line has: the merge finds every pair in one CTA's range
 int attn_rows_pad(int group_rows);                 // query rows per KV head, padded to the MMA tile
 cudaError_t launch_verify_attn(const AttnParams& p, cudaStream_t stream);
 // Merge of the pieces a flat schedule of `ctas` CTAs left (attn_umma.cu; the warp-MMA kernel's flat schedule uses it too).
