@@ -601,20 +601,13 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                 float f0 = 1.f, f1 = 1.f;
                 bool moved = false;
                 auto move_reference = [&](float mx, float& ref, float& top, float& f) {
-                    float to = ref;
+                    if (ref == -INFINITY) { ref = mx; top = mx; return; }
+                    float to = mx;
                     if (follow) {
                         top = fmaxf(top, mx);
                         to = fmaxf(mx, top - kRescaleBelow);
-                    } else if (mx > ref + kRescaleThreshold) {
-                        to = mx;
                     }
-                    if (ref == -INFINITY) {
-                        ref = mx;
-                    } else if (to != ref) {
-                        f = exp2f(ref - to);
-                        ref = to;
-                        moved = true;
-                    }
+                    if (follow ? to != ref : mx > ref + kRescaleThreshold) { f = exp2f(ref - to); ref = to; moved = true; }
                 };
                 move_reference(mx0, m_ref[0], m_top[0], f0);
                 move_reference(mx1, m_ref[1], m_top[1], f1);
