@@ -865,13 +865,25 @@ static long pair_tokens(const AttnParams& p) {
 
 // tcgen05 kernel: one CTA per pair where pairs are short, instead of ranges of the line of tiles: nothing to deal out, no pieces and
 // no merge launch.  A CTA takes 6 - 7.5 us and 1.2 - 1.5 us per tile of 64 positions, the balanced line with its merge at least
-// 9 - 10 us and more the more pairs it cuts, so the line between them rises with the number of pairs.  Call times, balanced -> one
-// CTA per pair, head_dim 128, lengths from a quarter of the table to all of it: 1 x 4 pairs of up to 128 positions 10.2 -> 7.7 us,
-// 16 x 4 of 128 14.5 -> 9.1, of 256 14.6 -> 12.0, of 512 17.0 -> 17.7; 64 x 4 of 256 26.8 -> 13.7, of 512 30.5 -> 20.1, of 1,024
-// 36 -> 32; 64 x 8 of 512 50 -> 38; 1 x 4 of 250 11.2 -> 12.1, so that few pairs take three tiles at most.
+// 9 - 10 us and more the more pairs it cuts.  The bounds are where full tables and lengths from a quarter of the table up, 1 and 42
+// rows, are all no slower this way (tables of 1 - 10 tiles, 44 batches, both head_dims).  Call times, balanced -> one CTA per pair, head_dim 128:
+//   1 x 4 pairs     2 tiles 10.4 -> 7.9 us    3 tiles 11.0 -> 9.0     4 tiles, full 11.4 -> 12.1
+//   16 x 4          2 tiles 13.8 -> 9.3       5 tiles 14.8 -> 13.9    6 tiles, full, 1 row 1.08 of the time
+//   32 x 4          7 tiles, full 23.5 -> 16.9                        8 tiles, full, 1 row 1.05
+//   32 x 8          3 tiles 15.1 -> 12.3      8 tiles 29.8 -> 20.2
+// and head_dim 64, whose CTAs are shorter: 16 x 4 of 6 tiles 13.4 -> 12.7, of 7, full, 1.06; 24 x 4 of 8 17.0 -> 15.2, of 9 14.7 -> 16.4.
+// With more pairs than places for CTAs (two on an SM) there is a second wave, and full tables of which the line takes whole pairs per
+// range cut nothing there: 64 x 8 of 4 tiles 33.7 -> 26.4, of 8 47.7 -> 40.2, but of 3 (six tiles a range) 20.9 -> 23.1; 38 x 8 of 6 tiles
+// 30.6 -> 30.4, of 7 31.5 -> 33.4; from two waves on few pairs are cut (80 x 8 of 8 full 53.0 -> 57.3), though ragged lengths still gain.
 static bool one_piece_per_pair(const AttnParams& p) {
-    const long pairs = (long)p.B * p.Hkv, tiles = (pair_tokens(p) + 63) / 64;
-    return !p.chunk_forced && p.max_pages <= kMaxChunkPages && tiles <= (pairs < 8 ? 3 : 4) + (pairs < 96 ? pairs / 24 : 4);
+    if (p.chunk_forced || p.d > 128 || p.max_pages > kMaxChunkPages) return false;
+    const long pairs = (long)p.B * p.Hkv, tiles = (pair_tokens(p) + 63) / 64, slots = 2L * device_sm_count();
+    if (pairs <= slots) {
+        if (p.d == 64) return tiles <= (pairs < 8 ? 3 : 4) + (pairs < 96 ? pairs / 24 : 4);
+        return tiles <= (pairs < 16 ? 3 : pairs < 48 ? 4 : pairs < 128 ? 5 : pairs < 192 ? 7 : 8);
+    }
+    const long range = (pairs * tiles + slots - 1) / slots;          // tiles of the line per CTA
+    return pairs <= 2 * slots && tiles >= 3 && tiles <= (2 * pairs < 3 * slots ? 6 : 8) && range % tiles != 0;
 }
 
 // Balanced schedule or chunk grid for the warp-MMA kernel at head_dim 256.  The balanced one wins wherever the grid would cut

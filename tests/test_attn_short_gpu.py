@@ -29,7 +29,9 @@ def _reference(w, window):
 
 @pytest.mark.parametrize("batch,gamma,q_heads,kv_heads,pages,window", [
     (1, 0, 1, 1, 1, 0), (1, 5, 4, 1, 16, 0), (1, 5, 4, 1, 17, 0), (3, 3, 16, 8, 20, 0), (3, 3, 16, 8, 21, 0), (12, 5, 28, 4, 24, 0), (24, 5, 28, 4, 32, 0),
-    (24, 5, 28, 4, 33, 0), (64, 7, 8, 8, 32, 0), (2, 1, 64, 2, 12, 0), (40, 2, 12, 4, 100, 100), (40, 2, 12, 4, 255, 300), (5, 6, 9, 1, 200, 40)])
+    (24, 5, 28, 4, 33, 0), (64, 7, 8, 8, 32, 0), (2, 1, 64, 2, 12, 0), (40, 2, 12, 4, 100, 100), (40, 2, 12, 4, 255, 300), (5, 6, 9, 1, 200, 40),
+    # the bounds of the rule: 16 and 48 pairs, one wave of CTAs and the first pair beyond, whole pairs per range, two waves
+    (15, 5, 7, 1, 16, 0), (16, 5, 7, 1, 16, 0), (47, 1, 3, 1, 20, 0), (48, 1, 3, 1, 20, 0), (37, 1, 8, 8, 32, 0), (99, 0, 3, 3, 24, 0), (99, 0, 3, 3, 28, 0), (64, 1, 8, 8, 12, 0), (149, 0, 4, 4, 24, 0)])
 @pytest.mark.parametrize("d", [64, 128])
 def test_against_64_bits(batch, gamma, q_heads, kv_heads, pages, window, d):
     import paper_2505_10526_b200 as mv
