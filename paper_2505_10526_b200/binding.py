@@ -110,7 +110,7 @@ def _load_marshal():
                           "`python -m paper_2505_10526_b200.build` (there is no fallback path)") from e
     address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
     _marshal.bind(address(_lib.massv_verify_attn), address(_lib.massv_accept), address(_lib.massv_kv_commit),
-                  address(_lib.massv_sample_top_p), address(_lib.massv_tvd))
+                  address(_lib.massv_sample_top_p), address(_lib.massv_tvd), AttnDesc, AcceptDesc)
     return _marshal
 
 

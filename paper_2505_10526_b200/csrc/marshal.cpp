@@ -15,6 +15,7 @@ decltype(&massv_accept) g_accept = nullptr;
 decltype(&massv_kv_commit) g_kv_commit = nullptr;
 decltype(&massv_sample_top_p) g_sample_top_p = nullptr;
 decltype(&massv_tvd) g_tvd = nullptr;
+PyObject *g_attn_desc = nullptr, *g_accept_desc = nullptr;       // the ctypes structures of the two descriptors
 
 const char* dtype_name(c10::ScalarType t) {
     switch (t) {
@@ -48,14 +49,19 @@ int32_t* i32(PyObject* o) { return static_cast<int32_t*>(pointer(o, c10::ScalarT
 void* any(PyObject* o) { return pointer(o, c10::ScalarType::Undefined); }
 size_t elements(PyObject* o) { return o == Py_None ? 0 : (size_t)THPVariable_Unpack(o).numel(); }      // (behind any(): a tensor)
 
-// A descriptor: the bytes of the ctypes structure.
+// A descriptor: the bytes of its ctypes structure (or of one derived from it, which begins with the same fields).
 template <typename Desc>
 struct DescOf {
     Py_buffer view;
-    explicit DescOf(PyObject* o) {
+    DescOf(PyObject* o, PyObject* type) {
+        const int is = PyObject_IsInstance(o, type);
+        if (is < 0) throw PythonError();
+        if (is == 0) fail(PyExc_TypeError, "massv: wrong descriptor");
         if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PythonError();
-        if (view.len != (Py_ssize_t)sizeof(Desc)) { PyBuffer_Release(&view); fail(PyExc_TypeError, "massv: wrong descriptor"); }
+        if (view.len < (Py_ssize_t)sizeof(Desc)) { PyBuffer_Release(&view); fail(PyExc_TypeError, "massv: wrong descriptor"); }
     }
+    DescOf(const DescOf&) = delete;
+    DescOf& operator=(const DescOf&) = delete;
     ~DescOf() { PyBuffer_Release(&view); }
     const Desc* get() const { return static_cast<const Desc*>(view.buf); }
 };
@@ -89,7 +95,7 @@ int unlocked(F&& f) {
 
 PyObject* py_verify_attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 13, [&] {
-        const DescOf<massv_attn_desc> d(a[0]);
+        const DescOf<massv_attn_desc> d(a[0], g_attn_desc);
         void *q = bf16(a[1]), *kn = bf16(a[2]), *vn = bf16(a[3]), *kp = bf16(a[4]), *vp = bf16(a[5]);
         int32_t *table = i32(a[6]), *lens = i32(a[7]);
         void* out = bf16(a[8]);
@@ -103,7 +109,7 @@ PyObject* py_verify_attn(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 PyObject* py_accept(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 13, [&] {
-        const DescOf<massv_accept_desc> d(a[0]);
+        const DescOf<massv_accept_desc> d(a[0], g_accept_desc);
         void *h = bf16(a[1]), *w = bf16(a[2]);
         int32_t* drafts = i32(a[3]);
         float *q = f32(a[4]), *ua = f32(a[5]), *us = f32(a[6]);
@@ -138,7 +144,7 @@ PyObject* py_sample_top_p(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 PyObject* py_tvd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 7, [&] {
-        const DescOf<massv_accept_desc> d(a[0]);
+        const DescOf<massv_accept_desc> d(a[0], g_accept_desc);
         float *z = f32(a[1]), *q = f32(a[2]), *tvd = f32(a[3]), *acc = f32(a[4]);
         void* ws = any(a[5]);
         const size_t ws_bytes = elements(a[5]);
@@ -150,7 +156,12 @@ PyObject* py_tvd(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 PyObject* py_bind(PyObject*, PyObject* args) {
     unsigned long long attn, accept, commit, top_p, tvd;
-    if (!PyArg_ParseTuple(args, "KKKKK", &attn, &accept, &commit, &top_p, &tvd)) return nullptr;
+    PyObject *attn_desc, *accept_desc;
+    if (!PyArg_ParseTuple(args, "KKKKKO!O!", &attn, &accept, &commit, &top_p, &tvd, &PyType_Type, &attn_desc, &PyType_Type, &accept_desc)) return nullptr;
+    Py_INCREF(attn_desc);
+    Py_INCREF(accept_desc);
+    Py_XSETREF(g_attn_desc, attn_desc);
+    Py_XSETREF(g_accept_desc, accept_desc);
     g_verify_attn = reinterpret_cast<decltype(g_verify_attn)>(attn);
     g_accept = reinterpret_cast<decltype(g_accept)>(accept);
     g_kv_commit = reinterpret_cast<decltype(g_kv_commit)>(commit);
@@ -161,7 +172,7 @@ PyObject* py_bind(PyObject*, PyObject* args) {
 
 #define MASSV_FAST(f) reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(f)), METH_FASTCALL
 PyMethodDef g_methods[] = {
-    {"bind", py_bind, METH_VARARGS, "addresses of the C ABI functions"},
+    {"bind", py_bind, METH_VARARGS, "addresses of the C ABI functions, types of the descriptors"},
     {"verify_attn", MASSV_FAST(py_verify_attn), nullptr},
     {"accept", MASSV_FAST(py_accept), nullptr},
     {"kv_commit", MASSV_FAST(py_kv_commit), nullptr},

@@ -1,5 +1,7 @@
 """What the native argument marshalling refuses is what the checks in Python refused: tensors off the GPU, other types, gaps,
 things that are no tensors, the other call's descriptor."""
+import ctypes
+
 import pytest
 import torch
 
@@ -26,9 +28,23 @@ def test_refused_without_a_gpu(mv):
         mv.massv_kv_commit(1, 1, i, i)
     with pytest.raises(AttributeError):
         mv.massv_kv_commit(1, 1, None, 7)
-    for wrong in (a, 3, None):
+    # another descriptor, and buffers of a descriptor's length that are none
+    for wrong in (a, 3, None, bytes(ctypes.sizeof(c)), bytearray(ctypes.sizeof(c)), (ctypes.c_char * ctypes.sizeof(c))(), type(c)):
         with pytest.raises(TypeError):
             mv.massv_accept(wrong, b, b, i, f, f, f, i, i)
+    for wrong in (c, bytes(ctypes.sizeof(a)), (ctypes.c_char * ctypes.sizeof(a))()):
+        with pytest.raises(TypeError):
+            mv.massv_verify_attn(wrong, b, b, b, b, b, i, i, b)
+
+
+def test_a_derived_descriptor_is_one(mv):
+    class Named(mv.AcceptDesc):
+        _fields_ = [("name", ctypes.c_char * 16)]
+
+    d = Named(*[getattr(mv.accept_desc(1, 1, 64, 64, 1.0), n) for n, _ in mv.AcceptDesc._fields_])
+    f = torch.zeros(64)
+    with pytest.raises(ValueError, match="CUDA device"):            # past the descriptor, at the first tensor
+        mv.massv_tvd(d, f, f, f)
 
 
 @pytest.mark.gpu
