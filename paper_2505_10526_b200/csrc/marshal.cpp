@@ -69,7 +69,13 @@ struct DescOf {
 massv_stream_t stream() { return reinterpret_cast<massv_stream_t>(c10::cuda::getCurrentCUDAStream().stream()); }
 
 long integer(PyObject* o) { const long v = PyLong_AsLong(o); if (v == -1 && PyErr_Occurred()) throw PythonError(); return v; }
-double number(PyObject* o) { const double v = PyFloat_AsDouble(o); if (v == -1.0 && PyErr_Occurred()) throw PythonError(); return v; }
+double number(PyObject* o) {                                     // whatever float() takes
+    PyObject* f = PyNumber_Float(o);
+    if (!f) throw PythonError();
+    const double v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
+    return v;
+}
 
 // Runs `call` (arguments in, status out) with the argument count checked and C++ exceptions turned into Python's; the
 // library call itself runs without the interpreter lock.

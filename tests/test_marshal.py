@@ -1,7 +1,10 @@
 """What the native argument marshalling refuses is what the checks in Python refused: tensors off the GPU, other types, gaps,
 things that are no tensors, the other call's descriptor."""
 import ctypes
+import decimal
+import fractions
 
+import numpy as np
 import pytest
 import torch
 
@@ -45,6 +48,15 @@ def test_a_derived_descriptor_is_one(mv):
     f = torch.zeros(64)
     with pytest.raises(ValueError, match="CUDA device"):            # past the descriptor, at the first tensor
         mv.massv_tvd(d, f, f, f)
+
+
+@pytest.mark.parametrize("number", ["0.75", b"0.75", fractions.Fraction(3, 4), decimal.Decimal("0.75"), np.float32(0.75), torch.tensor(0.75), 1])
+def test_numbers_are_what_float_takes(mv, number):
+    f, i = torch.zeros(64), torch.zeros(64, dtype=torch.int32)
+    with pytest.raises(ValueError, match="CUDA device"):            # past the numbers, at the first tensor
+        mv.massv_sample_top_p(f.view(1, 64), f, i, number, number)
+    with pytest.raises(TypeError):
+        mv.massv_sample_top_p(f.view(1, 64), f, i, None, number)
 
 
 @pytest.mark.gpu
