@@ -39,7 +39,7 @@ class AcceptDesc(ctypes.Structure):
 
 def _load():
     if not os.path.exists(LIB_PATH):
-        raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2505_10526_b200.build` "
+        raise ImportError(f"{LIB_PATH} is missing: build it with `python {os.path.join(_PKG, 'build.py')}` "
                           "(there is no fallback path)")
     lib = ctypes.CDLL(LIB_PATH)
     vp, i32p, f32p = ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p
@@ -107,7 +107,7 @@ def _load_marshal():
         from . import _marshal
     except ImportError as e:
         raise ImportError(f"{os.path.join(_PKG, '_marshal.so')} is missing or does not load ({e}): build it with "
-                          "`python -m paper_2505_10526_b200.build` (there is no fallback path)") from e
+                          f"`python {os.path.join(_PKG, 'build.py')}` (there is no fallback path)") from e
     address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
     _marshal.bind(address(_lib.massv_verify_attn), address(_lib.massv_accept), address(_lib.massv_kv_commit),
                   address(_lib.massv_sample_top_p), address(_lib.massv_tvd), AttnDesc, AcceptDesc)

@@ -91,4 +91,5 @@ def build_debug(force: bool = False) -> str:
 
 
 if __name__ == "__main__":
-    print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    force = "--force" in sys.argv
+    print("\n".join([build(force, verbose=True)] if "-v" in sys.argv else build_all(force)))

@@ -3,6 +3,11 @@ things that are no tensors, the other call's descriptor."""
 import ctypes
 import decimal
 import fractions
+import os
+import re
+import shutil
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -57,6 +62,20 @@ def test_numbers_are_what_float_takes(mv, number):
         mv.massv_sample_top_p(f.view(1, 64), f, i, number, number)
     with pytest.raises(TypeError):
         mv.massv_sample_top_p(f.view(1, 64), f, i, None, number)
+
+
+def test_the_command_a_missing_module_names(mv, tmp_path):
+    """A package without its native module says what builds it, and that command works although the package cannot be imported."""
+    root = os.path.dirname(os.path.dirname(mv.LIB_PATH))
+    for name in ("include", "paper_2505_10526_b200"):
+        shutil.copytree(os.path.join(root, name), tmp_path / name, ignore=shutil.ignore_patterns("_marshal*", "__pycache__"))
+    import_it = [sys.executable, "-c", "import paper_2505_10526_b200"]
+    missing = subprocess.run(import_it, cwd=tmp_path, capture_output=True, text=True)
+    assert missing.returncode != 0 and "ImportError" in missing.stderr
+    command = re.search("`(python .*)`", missing.stderr.strip().splitlines()[-1]).group(1).split()
+    assert command[0] == "python" and os.path.samefile(command[1], tmp_path / "paper_2505_10526_b200" / "build.py")
+    subprocess.run([sys.executable] + command[1:], cwd=tmp_path, check=True)
+    subprocess.run(import_it, cwd=tmp_path, check=True)
 
 
 @pytest.mark.gpu
