@@ -9,9 +9,13 @@ module without the compiled library raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
+
+from .build import marshal_path
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 # MASSV_DEBUG=1 selects the build with device-side index checks (same entry points, MASSV_ERR_BOUNDS in dev_status
@@ -103,10 +107,13 @@ _lib = _load()
 def _load_marshal():
     """The calls a decoding loop makes every step go through a native module (csrc/marshal.cpp): the same checks as ``_ptr``'s on
     every tensor, the same stream, the same entry points of the library loaded above."""
+    path, name = marshal_path(), __package__ + "._marshal"
     try:
-        from . import _marshal
+        spec = importlib.util.spec_from_file_location(name, path, loader=importlib.machinery.ExtensionFileLoader(name, path))
+        _marshal = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(_marshal)
     except ImportError as e:
-        raise ImportError(f"{os.path.join(_PKG, '_marshal.so')} is missing or does not load ({e}): build it with "
+        raise ImportError(f"{path} is missing or does not load ({e}): build it with "
                           f"`python {os.path.join(_PKG, 'build.py')}` (there is no fallback path)") from e
     address = lambda f: ctypes.cast(f, ctypes.c_void_p).value
     _marshal.bind(address(_lib.massv_verify_attn), address(_lib.massv_accept), address(_lib.massv_kv_commit),

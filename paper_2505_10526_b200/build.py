@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import runpy
 import subprocess
 import sys
 import sysconfig
@@ -15,7 +16,18 @@ SOURCES = ["api.cu", "attn.cu", "attn_umma.cu", "lm_head.cu", "accept.cu", "acce
 
 TEST_LIB = os.path.join(PKG, "libmassv_testhooks.so")
 DEBUG_LIB = os.path.join(PKG, "libmassv_debug.so")
-MARSHAL = os.path.join(PKG, "_marshal.so")
+
+
+def _torch_dir() -> str:
+    import importlib.util
+    return os.path.dirname(importlib.util.find_spec("torch").origin)          # (without importing torch: that takes seconds)
+
+
+def marshal_path() -> str:
+    """The native module's file.  It is compiled against the layout of torch's and Python's objects, so their versions are in its name:
+    after an update of either the old file is not the one that is looked for, and the build makes another."""
+    torch_version = runpy.run_path(os.path.join(_torch_dir(), "version.py"))["__version__"]
+    return os.path.join(PKG, f"_marshal.torch-{torch_version}{sysconfig.get_config_var('EXT_SUFFIX')}")
 
 
 def _stale(lib=LIB) -> bool:
@@ -45,20 +57,19 @@ VARIANTS = {LIB: [], TEST_LIB: ["-DMASSV_TEST_HOOKS", "-DMASSV_SPIN_LIMIT=65536u
 
 
 def _marshal_command():
-    """The extension module against torch's own headers and libraries (found without importing torch: that takes seconds)."""
-    import importlib.util
-    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    """The extension module against torch's own headers and libraries."""
+    torch_dir = _torch_dir()
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     include = [sysconfig.get_paths()["include"], os.path.join(torch_dir, "include"),
                os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
     return ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", INCLUDE] + [x for d in include for x in ("-isystem", d)] +
-            ["-o", MARSHAL, os.path.join(CSRC, "marshal.cpp"), "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+            ["-o", marshal_path(), os.path.join(CSRC, "marshal.cpp"), "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
 
 
 def build_all(force: bool = False):
     """The library, its two test variants and the marshalling module, the stale ones compiled side by side."""
     commands = {lib: _command(lib, extra) for lib, extra in VARIANTS.items()}
-    commands[MARSHAL] = _marshal_command()
+    commands[marshal_path()] = _marshal_command()
     procs = [(out, subprocess.Popen(cmd)) for out, cmd in commands.items() if force or _stale(out)]
     for out, proc in procs:
         if proc.wait() != 0:
@@ -67,7 +78,7 @@ def build_all(force: bool = False):
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or _stale(MARSHAL):
+    if force or _stale(marshal_path()):
         subprocess.run(_marshal_command(), check=True)
     if not (force or _stale()):
         return LIB

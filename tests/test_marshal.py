@@ -5,9 +5,11 @@ import decimal
 import fractions
 import os
 import re
+import runpy
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 import numpy as np
 import pytest
@@ -62,6 +64,21 @@ def test_numbers_are_what_float_takes(mv, number):
         mv.massv_sample_top_p(f.view(1, 64), f, i, number, number)
     with pytest.raises(TypeError):
         mv.massv_sample_top_p(f.view(1, 64), f, i, None, number)
+
+
+def test_the_module_goes_with_torch_and_python(mv, monkeypatch):
+    """Another torch or another Python: another file, which does not exist and is stale, so that it is built and never loaded in its place."""
+    from paper_2505_10526_b200 import build
+    here = build.marshal_path()
+    assert mv.binding._native.__file__ == here and not build._stale(here)
+    assert torch.__version__ in os.path.basename(here) and here.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    for target, name, value in ((runpy, "run_path", lambda path: {"__version__": "2.99.0"}), (sysconfig, "get_config_var", lambda name: ".cpython-399-x86_64-linux-gnu.so")):
+        with monkeypatch.context() as m:
+            m.setattr(target, name, value)
+            other = build.marshal_path()
+            assert other != here and build._stale(other)
+            with pytest.raises(ImportError, match="build it with"):
+                mv.binding._load_marshal()
 
 
 def test_the_command_a_missing_module_names(mv, tmp_path):
