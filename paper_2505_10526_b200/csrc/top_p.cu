@@ -69,6 +69,13 @@ struct RowWeight {
         return fminf(y, 1.0f);              // the approximation must not step past the pattern of 1.0f
     }
 };
+// The mass that the nucleus must reach, of a row of `total` units.  (top_p = 1 is the whole row as it stands: totals from 2^53 up - rows whose
+// weights add up to more than 512 - lose low bits as a double, and with them entries of the tail.)
+__device__ __forceinline__ unsigned long long target_mass(float top_p, unsigned long long total) {
+    if (top_p >= 1.f) return total;
+    const unsigned long long target = (unsigned long long)ceil((double)top_p * (double)total);
+    return min(max(target, 1ull), total);
+}
 // floor(w * 2^fx_bits) for 0 <= w <= 1 from the pattern of w: mantissa shifted by the exponent
 __device__ __forceinline__ unsigned long long fixed_point(float w, int fx_bits) {
     const uint32_t b = __float_as_uint(w);
@@ -157,9 +164,7 @@ __global__ void __launch_bounds__(kTopPThreads) top_p_kernel(TopPParams p) {
         }
     }
     const unsigned long long S_fx = (block_sum_u64(local_hi, sm_u64) << 32) + block_sum_u64(local_lo, sm_u64);
-    unsigned long long target_fx = (unsigned long long)ceil((double)p.top_p * (double)S_fx);
-    if (target_fx > S_fx) target_fx = S_fx;
-    if (target_fx == 0ull) target_fx = 1ull;
+    const unsigned long long target_fx = target_mass(p.top_p, S_fx);
 
     // ---- threshold: largest bit pattern tau with mass{w >= tau} >= target, by radix selection
     uint32_t prefix = 0u;                 // bits of tau found so far
@@ -512,9 +517,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
             if (t == sum_bin) run = total;
             total += s_above;
             total_fx = total;
-            target_fx = (unsigned long long)ceil((double)p.top_p * (double)total);
-            if (target_fx > total) target_fx = total;
-            if (target_fx == 0ull) target_fx = 1ull;
+            target_fx = target_mass(p.top_p, total);
             __syncthreads();                       // s_above has been read
         }
         // the bin b with mass_above + sum(bins > b) < target <= mass_above + sum(bins >= b) exists exactly once

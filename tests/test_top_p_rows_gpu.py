@@ -132,3 +132,21 @@ def test_levels(std, top_p):
     z[1, ::3] = -float("inf")
     z[2, 100:] = -float("inf")
     _check(z, torch.rand((5,), generator=g, device="cuda"), 1.0, top_p, allow=5 if top_p == 1.0 else 2)
+
+
+@pytest.mark.parametrize("rows,vocab", [(1, 262144), (3, 262144), (2, 393216), (2, 400000)])
+def test_the_whole_row_whatever_its_mass(rows, vocab):
+    """top_p = 1 takes every entry that has mass, also where the row's mass in units of 2^-44 has more bits than a double: flat rows with
+    five entries of 2^-40, 80 units in all, less than half a step of the double next to the row's sum of 2^62."""
+    import paper_2505_10526_b200 as mv
+    T = 1.4426950408889634                       # weights 2^(z - max)
+    z = torch.zeros((rows, vocab), device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(vocab)
+    at = torch.stack([torch.randperm(vocab, generator=g, device="cuda")[:5] for _ in range(rows)])
+    z.scatter_(1, at, -40.0)
+    tok = torch.empty((rows,), dtype=torch.int32, device="cuda")
+    q = torch.empty_like(z)
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    mv.massv_sample_top_p(z, torch.full((rows,), 0.5, device="cuda"), tok, T, 1.0, q, status)
+    assert int(status.item()) == 0
+    assert bool((q > 0).all())
