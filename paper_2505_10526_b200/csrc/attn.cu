@@ -49,12 +49,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// 2^x in one instruction (results below 2^-126 are zero): for factors between maxima.
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // Byte offset of the 16-byte unit `unit` (0..7) of row `row` inside a region of
 // 128-byte rows laid out with the 128-byte swizzle (what TMA writes).
@@ -178,7 +172,7 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
     const float mn0 = fmaxf(m_run[0], mx0), mn1 = fmaxf(m_run[1], mx1);
     const float rn0 = fmaxf(mx0, mn0 - kRefDrop), rn1 = fmaxf(mx1, mn1 - kRefDrop);
     const float ms0 = rn0 == -INFINITY ? 0.f : rn0, ms1 = rn1 == -INFINITY ? 0.f : rn1;
-    const float corr0 = ex2(r_run[0] - ms0), corr1 = ex2(r_run[1] - ms1);
+    const float corr0 = ex2_ftz(r_run[0] - ms0), corr1 = ex2_ftz(r_run[1] - ms1);
     r_run[0] = rn0; r_run[1] = rn1;
     float ls0 = 0.f, ls1 = 0.f;
     uint32_t pa[NT / 16][4];
@@ -193,11 +187,11 @@ __device__ __forceinline__ void attend_tile(const AttnParams& p, int b, int g, i
     }
     const float mt0 = mn0 == -INFINITY ? 0.f : mn0, mt1 = mn1 == -INFINITY ? 0.f : mn1;
     if (__any_sync(0xffffffffu, mn0 > m_run[0] || mn1 > m_run[1])) {
-        l_run[0] *= ex2(m_run[0] - mt0); l_run[1] *= ex2(m_run[1] - mt1);
+        l_run[0] *= ex2_ftz(m_run[0] - mt0); l_run[1] *= ex2_ftz(m_run[1] - mt1);
         m_run[0] = mn0; m_run[1] = mn1;
     }
-    l_run[0] += ls0 * ex2(rn0 - mt0);
-    l_run[1] += ls1 * ex2(rn1 - mt1);
+    l_run[0] += ls0 * ex2_ftz(rn0 - mt0);
+    l_run[1] += ls1 * ex2_ftz(rn1 - mt1);
 #pragma unroll
     for (int n = 0; n < D / 8; ++n) { o[n][0] *= corr0; o[n][1] *= corr0; o[n][2] *= corr1; o[n][3] *= corr1; }
 

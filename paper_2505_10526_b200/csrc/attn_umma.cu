@@ -110,11 +110,6 @@ __device__ __forceinline__ void ring_item_decode(int i, int n, int& t, int& is_v
     else if (i >= 2 * n - 2) { t = n - 2 + (i - (2 * n - 2)); is_v = 1; }
     else { const int j = i - 2; is_v = j & 1; t = is_v ? (j - 1) / 2 : 2 + j / 2; }
 }
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // One piece of work: a run of tiles of one (sequence, KV head) pair.
 struct Segment {
@@ -619,10 +614,10 @@ attn_umma_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         // 2^(s * scale * log2 e - reference): one multiply-add into the exponential unit
-                        const float p0 = ex2_approx(fmaf(__uint_as_float(s[h][4 * k + 0]), scale_log2, ms0));
-                        const float p1 = ex2_approx(fmaf(__uint_as_float(s[h][4 * k + 1]), scale_log2, ms0));
-                        const float p2 = ex2_approx(fmaf(__uint_as_float(s[h][4 * k + 2]), scale_log2, ms1));
-                        const float p3 = ex2_approx(fmaf(__uint_as_float(s[h][4 * k + 3]), scale_log2, ms1));
+                        const float p0 = ex2_ftz(fmaf(__uint_as_float(s[h][4 * k + 0]), scale_log2, ms0));
+                        const float p1 = ex2_ftz(fmaf(__uint_as_float(s[h][4 * k + 1]), scale_log2, ms0));
+                        const float p2 = ex2_ftz(fmaf(__uint_as_float(s[h][4 * k + 2]), scale_log2, ms1));
+                        const float p3 = ex2_ftz(fmaf(__uint_as_float(s[h][4 * k + 3]), scale_log2, ms1));
                         la[k & 3] += p0 + p1; lb[k & 3] += p2 + p3;
                         pk[h][2 * k] = pack_bf16x2(p0, p1);
                         pk[h][2 * k + 1] = pack_bf16x2(p2, p3);

@@ -40,8 +40,8 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t h) {
     return __uint_as_float(((uint32_t)h) << 16);
 }
 
-// Two fp32 operations in one instruction (sm_100), rounded as the single ones are, and 2^x by the exponential unit alone: exp2f
-// and expf wrap it in instructions for results below 2^-126, which are zero here.
+// Two fp32 operations in one instruction (sm_100), rounded as the single ones are, and 2^x as the PTX instruction gives it: a relative
+// error of 2^-22 at most, arguments and results below 2^-126 are zero.
 __device__ __forceinline__ uint64_t pack2(float a, float b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
 __device__ __forceinline__ float2 unpack2(uint64_t v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }

@@ -127,8 +127,8 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint32_t a_lo, u
 }
 // Arrive, in both CTAs of the pair, on the barrier at this shared-memory offset once the MMAs issued so far are done.
 // This barrier arrive between the two CTAs of one pair (same GPU) is the only multicast qualifier in the sources:
-// every TMA load here (tma_load_2d, tma_load_2d_pair, the 1-D bulk copies) is non-multicast and reads this GPU's
-// memory only.
+// every TMA load here (tma_load_2d, tma_load_2d_pair, tma_load_blocks, tma_load_blocks_pair, the 1-D bulk copies) is non-multicast
+// and reads this GPU's memory only.
 __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
                  "h"((uint16_t)3)

@@ -64,9 +64,7 @@ struct RowWeight {
     float k2, m2;
     __device__ RowWeight(float inv_T, float m) : k2(inv_T * 1.4426950408889634f) { m2 = -m * k2; }
     __device__ __forceinline__ float operator()(float zv) const {
-        float y;
-        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaf(zv, k2, m2)));
-        return fminf(y, 1.0f);              // the approximation must not step past the pattern of 1.0f
+        return fminf(ex2_ftz(fmaf(zv, k2, m2)), 1.0f);              // the approximation must not step past the pattern of 1.0f
     }
 };
 // The mass that the nucleus must reach, of a row of `total` units.  (top_p = 1 is the whole row as it stands: totals from 2^53 up - rows whose
@@ -449,7 +447,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) top_p_cluster_kernel(TopPParam
     // power of two, levels of 9 bits more while more than kRowCand entries share the bits found, then those entries one by
     // one.  A bin fixes the exponent, so its mass is a sum of (truncated) mantissas: a word that wraps every 256 entries at
     // most, and a carry.  A language model's row needs the first level only; with two bins per power of two it took a second
-    // walk and exchange (64 rows of 152,064: 61 us, 54 here).
+    // walk and exchange (64 rows of 152,064: 61 us, 53 here).  Rows with more entries near the threshold take the second level here too, and
+    // reading 385 bins of every peer instead of 26 shows (logits of standard deviation 2.5, one row of 152,064: 30.5 us, 32.0 here).
     uint32_t prefix = 0u;                 // bits of tau found so far: all but the last `open` ones
     int open = 0;
     unsigned long long mass_above = 0ull, target_fx = 0ull, total_fx = 0ull;
