@@ -20,7 +20,8 @@
 // accumulator), apply scale, causal / window mask and the online softmax, and write P
 // as bf16 into shared memory for the second product.  O is rescaled in tensor memory
 // only when a row's running maximum has grown by more than 2^8 since its reference
-// was set (the reference cancels in O / l, so the result is the plain softmax).
+// was set, for short pairs in one piece at every tile whose maximum is another
+// (the reference cancels in O / l, so the result is the plain softmax).
 //
 // Two schedules share the kernel.  CHUNKED: grid (chunk, KV head, sequence) as in the warp-MMA
 // kernel, one piece of work per CTA, pieces of a sequence merged by attn_combine_kernel (used
